@@ -250,6 +250,9 @@ struct Quad {                           // regular 7-point sources, owner order
     double *nx = nullptr, *ny = nullptr, *nz = nullptr, *w = nullptr;
     float *fx = nullptr, *fy = nullptr, *fz = nullptr;   // offsets from the owning leaf centre
     float *fnx = nullptr, *fny = nullptr, *fnz = nullptr, *fw = nullptr;
+    // float64 plans: offsets (x 2^-ilogb(root side)) and normals as float32
+    // pairs, high parts in fx.., fnx.., low parts here
+    float *lx = nullptr, *ly = nullptr, *lz = nullptr, *lnx = nullptr, *lny = nullptr, *lnz = nullptr;
 };
 
 struct Correction {                     // CSR by node (row), special - regular
@@ -373,8 +376,10 @@ struct bem_plan : bem::FmmState {
     bem::FmmState diag_state;           // the diagonal's order while its product runs (set-up only)
     bool diag_mode = false;             // alloc_fmm for the diagonal's order
     cudaStream_t setup_stream[3] = {nullptr, nullptr, nullptr};
-    int2 *near_items[2] = {nullptr, nullptr};   // float32 near-field work items, 64- and 32-target passes
+    int2 *near_items[2] = {nullptr, nullptr};   // near-field work items (real, complex)
     int near_nitems[2] = {0, 0};
+    int *leaf_near_ptr = nullptr, *leaf_near_idx = nullptr;   // leaf_descend = 0: near lists opened down to leaves
+    const float4 *circle = nullptr;             // unit-circle table of the float64 Helmholtz near field (the library's)
     int last_op = -1;
     // GMRES workspace
     double *V = nullptr, *H = nullptr, *gs = nullptr, *w = nullptr, *xk = nullptr, *bvec = nullptr;

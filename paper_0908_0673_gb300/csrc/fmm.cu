@@ -23,38 +23,11 @@
 #include <cmath>
 #include <mutex>
 
-#include "bem_internal.cuh"
+#include "fmm_views.cuh"
 
 namespace bem {
 
 __constant__ double c_Lq[2][NQ][6];   // shape values at the 7 rule points (tri3, tri6)
-
-struct Tabs {
-    const int *m, *n, *k, *idx3;
-    const double *fact;
-    int p, np;                          // largest order, and the coefficient count (array stride)
-    const int *lev_p;                   // order of each tree level (nullptr: p everywhere)
-};
-
-// number of multi-indices of degree <= q (the coefficients of order q)
-__host__ __device__ __forceinline__ int np_of(int q) { return (q + 1) * (q + 2) * (q + 3) / 6; }
-__device__ __forceinline__ int order_of(const Tabs &tb, int level) { return tb.lev_p ? tb.lev_p[level] : tb.p; }
-
-struct TreeView {
-    const int *level, *ix, *iy, *iz, *parent, *child0, *nchild, *nb, *ne, *eb, *ee, *leaves;
-    const int *near_ptr, *near_idx, *inter_ptr, *inter_idx, *node_perm;
-    const double *cx, *cy, *cz, *tx, *ty, *tz;
-    double side;
-};
-
-struct QuadView {
-    const double *x, *y, *z, *nx, *ny, *nz, *w;
-    const float *fx, *fy, *fz, *fnx, *fny, *fnz, *fw;
-};
-
-template <class R> struct Vec { R v[2]; };
-
-__device__ __forceinline__ int deg_of(int m, int n, int k) { return m + n + k; }
 
 // ---------------------------------------------------------------------------
 // P2Q
@@ -272,118 +245,89 @@ static void launch_p2m_stored(int nleaf, int np, const TreeView &tv, const float
 }
 
 // ---------------------------------------------------------------------------
-// near field (regular rule over the near-list boxes) fused with L2P
+// near field (regular rule over the near-list boxes) fused with L2P, float64
+// arithmetic: Helmholtz plans whose phases exceed the table of the float32-pair
+// kernel (near_f64.cu), which takes every other float64 product
 // ---------------------------------------------------------------------------
 constexpr int NF_T = 256, NF_TGT = 64, NF_SL = NF_T / NF_TGT, NF_TILE = 256;
 
-template <class R, int C, bool DL>
-__device__ __forceinline__ void pair_kernel(R rx, R ry, R rz, R nx, R ny, R nz, const R *fv, R kw, R *acc) {
-    const R r2 = rx * rx + ry * ry + rz * rz;
-    R inv;
-    if constexpr (sizeof(R) == sizeof(double)) inv = (R)rsqrt((double)r2);
-    else inv = (R)rsqrtf((float)r2);
-    if (C == 1) {
-        if (DL) acc[0] += fv[0] * (rx * nx + ry * ny + rz * nz) * inv * inv * inv;
-        else acc[0] += fv[0] * inv;
+template <bool DL>
+__device__ __forceinline__ void pair_f64(double rx, double ry, double rz, double nx, double ny, double nz,
+                                         const double *fv, double kw, double *acc) {
+    const double r2 = rx * rx + ry * ry + rz * rz, inv = rsqrt(r2), R1 = r2 * inv;
+    double sn, cs, gr, gi;
+    sincos(kw * R1, &sn, &cs);
+    if (DL) {
+        const double kr = kw * R1, rn = (rx * nx + ry * ny + rz * nz) * inv * inv * inv;
+        gr = (cs + kr * sn) * rn;
+        gi = (sn - kr * cs) * rn;
     } else {
-        const R R1 = r2 * inv;
-        R sn, cs;
-        if constexpr (sizeof(R) == sizeof(double)) sincos((double)(kw * R1), (double *)&sn, (double *)&cs);
-        else sincosf((float)(kw * R1), (float *)&sn, (float *)&cs);
-        R gr, gi;
-        if (DL) {
-            const R kr = kw * R1, rn = (rx * nx + ry * ny + rz * nz) * inv * inv * inv;
-            gr = (cs + kr * sn) * rn;
-            gi = (sn - kr * cs) * rn;
-        } else {
-            gr = cs * inv;
-            gi = sn * inv;
-        }
-        acc[0] += gr * fv[0] - gi * fv[1];
-        acc[1] += gr * fv[1] + gi * fv[0];
+        gr = cs * inv;
+        gi = sn * inv;
     }
+    acc[0] += gr * fv[0] - gi * fv[1];
+    acc[1] += gr * fv[1] + gi * fv[0];
 }
 
-template <class R, int C, bool DL>
-__global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, QuadView qv, double kwave,
-                                               const R *__restrict__ f, const R *__restrict__ L,
+template <bool DL>
+__global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, QuadView qv, double kw,
+                                               const double *__restrict__ f, const double *__restrict__ L,
                                                double *__restrict__ ytmp, const int *__restrict__ skip) {
     if (skip && *skip) return;
+    constexpr int C = 2;
     const int li = blockIdx.x;
     if (li >= nleaf) return;
     const int b = tv.leaves[li];
     const int tid = threadIdx.x, tt = tid % NF_TGT, sl = tid / NF_TGT;
     const int np = tb.np, p = order_of(tb, tv.level[b]), npl = np_of(p);   // the leaf's order; np the stride
-    __shared__ R sx[NF_TILE], sy[NF_TILE], sz[NF_TILE], snx[NF_TILE], sny[NF_TILE], snz[NF_TILE];
-    __shared__ R sf[NF_TILE][C];
+    __shared__ double sx[NF_TILE], sy[NF_TILE], sz[NF_TILE], snx[NF_TILE], sny[NF_TILE], snz[NF_TILE];
+    __shared__ double sf[NF_TILE][C];
     __shared__ double red[NF_T][C];
     const double cbx = tv.cx[b], cby = tv.cy[b], cbz = tv.cz[b];
     const double h = scalbn(tv.side, -tv.level[b]);
-    const R kw = (R)kwave;
     for (int t0 = tv.nb[b]; t0 < tv.ne[b]; t0 += NF_TGT) {
         const int tk = t0 + tt;
         const bool active = tk < tv.ne[b];
-        // target position: absolute (F64) or offset from this leaf's centre (F32)
-        double txd = active ? tv.tx[tk] : cbx, tyd = active ? tv.ty[tk] : cby, tzd = active ? tv.tz[tk] : cbz;
-        double acc[C];
-#pragma unroll
-        for (int c = 0; c < C; c++) acc[c] = 0.0;
+        const double tx = active ? tv.tx[tk] : cbx, ty = active ? tv.ty[tk] : cby, tz = active ? tv.tz[tk] : cbz;
+        double acc[C] = {0.0, 0.0};
         for (int u = tv.near_ptr[b]; u < tv.near_ptr[b + 1]; u++) {
             const int s = tv.near_idx[u];
             const int q0 = tv.eb[s] * NQ, q1 = tv.ee[s] * NQ;
-            R tx, ty, tz;
-            if constexpr (sizeof(R) == sizeof(double)) {
-                tx = (R)txd; ty = (R)tyd; tz = (R)tzd;
-            } else {
-                // r = (c_b - c_s) + (t - c_b) - (q - c_s), each part small
-                tx = (R)(cbx - tv.cx[s]) + (R)(txd - cbx);
-                ty = (R)(cby - tv.cy[s]) + (R)(tyd - cby);
-                tz = (R)(cbz - tv.cz[s]) + (R)(tzd - cbz);
-            }
-            R part[C];
-#pragma unroll
-            for (int c = 0; c < C; c++) part[c] = (R)0;
+            double part[C] = {0.0, 0.0};
             for (int base = q0; base < q1; base += NF_TILE) {
                 const int nt = min(NF_TILE, q1 - base);
                 __syncthreads();
                 if (tid < nt) {
                     const int o = base + tid;
-                    if constexpr (sizeof(R) == sizeof(double)) {
-                        sx[tid] = (R)qv.x[o]; sy[tid] = (R)qv.y[o]; sz[tid] = (R)qv.z[o];
-                        if (DL) { snx[tid] = (R)qv.nx[o]; sny[tid] = (R)qv.ny[o]; snz[tid] = (R)qv.nz[o]; }
-                    } else {
-                        sx[tid] = (R)qv.fx[o]; sy[tid] = (R)qv.fy[o]; sz[tid] = (R)qv.fz[o];
-                        if (DL) { snx[tid] = (R)qv.fnx[o]; sny[tid] = (R)qv.fny[o]; snz[tid] = (R)qv.fnz[o]; }
-                    }
-#pragma unroll
-                    for (int c = 0; c < C; c++) sf[tid][c] = f[(size_t)o * C + c];
+                    sx[tid] = qv.x[o]; sy[tid] = qv.y[o]; sz[tid] = qv.z[o];
+                    if (DL) { snx[tid] = qv.nx[o]; sny[tid] = qv.ny[o]; snz[tid] = qv.nz[o]; }
+                    sf[tid][0] = f[(size_t)o * C];
+                    sf[tid][1] = f[(size_t)o * C + 1];
                 }
                 __syncthreads();
                 if (active)
                     for (int j = sl; j < nt; j += NF_SL)
-                        pair_kernel<R, C, DL>(tx - sx[j], ty - sy[j], tz - sz[j], DL ? snx[j] : (R)0,
-                                              DL ? sny[j] : (R)0, DL ? snz[j] : (R)0, sf[j], kw, part);
+                        pair_f64<DL>(tx - sx[j], ty - sy[j], tz - sz[j], DL ? snx[j] : 0.0, DL ? sny[j] : 0.0,
+                                     DL ? snz[j] : 0.0, sf[j], kw, part);
             }
-#pragma unroll
-            for (int c = 0; c < C; c++) acc[c] += (double)part[c];
+            acc[0] += part[0];
+            acc[1] += part[1];
         }
         // local expansion at the target: sum_b Ls_b ((x - c)/h)^b, slices split b
-        double loc[C];
-#pragma unroll
-        for (int c = 0; c < C; c++) loc[c] = 0.0;
+        double loc[C] = {0.0, 0.0};
         if (active) {
-            const R dx = (R)((txd - cbx) / h), dy = (R)((tyd - cby) / h), dz = (R)((tzd - cbz) / h);
-            R px[PMAX + 1], py[PMAX + 1], pz[PMAX + 1];
-            px[0] = py[0] = pz[0] = (R)1;
+            const double dx = (tx - cbx) / h, dy = (ty - cby) / h, dz = (tz - cbz) / h;
+            double px[PMAX + 1], py[PMAX + 1], pz[PMAX + 1];
+            px[0] = py[0] = pz[0] = 1.0;
             for (int e = 1; e <= p; e++) {
                 px[e] = px[e - 1] * dx;
                 py[e] = py[e - 1] * dy;
                 pz[e] = pz[e - 1] * dz;
             }
             for (int a = sl; a < npl; a += NF_SL) {
-                const R mono = px[tb.m[a]] * py[tb.n[a]] * pz[tb.k[a]];
+                const double mono = px[tb.m[a]] * py[tb.n[a]] * pz[tb.k[a]];
 #pragma unroll
-                for (int c = 0; c < C; c++) loc[c] += (double)(mono * L[((size_t)b * np + a) * C + c]);
+                for (int c = 0; c < C; c++) loc[c] += mono * L[((size_t)b * np + a) * C + c];
             }
         }
         __syncthreads();
@@ -391,9 +335,7 @@ __global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, 
         for (int c = 0; c < C; c++) red[tid][c] = acc[c] * (0.25 / M_PI) + loc[c];
         __syncthreads();
         if (sl == 0 && active) {
-            double s[C];
-#pragma unroll
-            for (int c = 0; c < C; c++) s[c] = red[tid][c];
+            double s[C] = {red[tid][0], red[tid][1]};
             for (int u = 1; u < NF_SL; u++)
 #pragma unroll
                 for (int c = 0; c < C; c++) s[c] += red[tid + u * NF_TGT][c];
@@ -427,8 +369,8 @@ __host__ __device__ constexpr int nf2_tile(int C) { return C == 1 ? 1024 : NF2_T
 // float4 slots of the staged-source region
 __host__ __device__ constexpr int nf2_stage(int C) { return C == 1 ? 3 * nf2_tile(1) : 2 * NF2_TILE; }
 
-// Work items of the float32 near field: one per (leaf, pass of up to 8 U
-// targets), ordered by decreasing pair count (targets x near sources, ties in
+// Work items of the near field: one per (leaf, pass of up to 8 U targets, or
+// ND_SLOTS in float64 plans), ordered by decreasing pair count (targets x near sources, ties in
 // leaf order), so the largest blocks start first and the last wave is made of
 // the smallest.  Each target is summed by one block whatever the order.
 int build_near_items(bem_plan *P) {
@@ -442,6 +384,32 @@ int build_near_items(bem_plan *P) {
     BEM_CUDA(cudaMemcpy(eb.data(), t.eb, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
     BEM_CUDA(cudaMemcpy(ee.data(), t.ee, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
     BEM_CUDA(cudaMemcpy(lv.data(), t.leaves, sizeof(int) * t.nleaf, cudaMemcpyDeviceToHost));
+    // A literal list (leaf_descend = 0) may hold non-leaf boxes.  The float64
+    // near field takes a source's position from its own leaf's centre, so such
+    // an entry becomes its subtree's leaves, in element order.
+    if (!P->prm.leaf_descend) {
+        std::vector<int> child0(t.nbox), nchild(t.nbox), ptr(t.nbox + 1, 0), idx, stack;
+        BEM_CUDA(cudaMemcpy(child0.data(), t.child0, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
+        BEM_CUDA(cudaMemcpy(nchild.data(), t.nchild, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
+        for (int b = 0; b < t.nbox; b++) {
+            if (nchild[b] == 0)                       // only leaves are targets
+                for (int u = nptr[b]; u < nptr[b + 1]; u++) {
+                    stack.push_back(nidx[u]);
+                    while (!stack.empty()) {
+                        const int s = stack.back();
+                        stack.pop_back();
+                        if (nchild[s] == 0) idx.push_back(s);
+                        for (int q = nchild[s] - 1; q >= 0; q--) stack.push_back(child0[s] + q);
+                    }
+                }
+            ptr[b + 1] = (int)idx.size();
+        }
+        BEM_TRY(P->arena.alloc(&P->leaf_near_ptr, ptr.size()));
+        BEM_TRY(P->arena.alloc(&P->leaf_near_idx, idx.size()));
+        BEM_CUDA(cudaMemcpy(P->leaf_near_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice));
+        if (!idx.empty())
+            BEM_CUDA(cudaMemcpy(P->leaf_near_idx, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice));
+    }
     int64_t pairs = 0;
     std::vector<int64_t> src(t.nleaf);
     for (int li = 0; li < t.nleaf; li++) {
@@ -455,7 +423,7 @@ int build_near_items(bem_plan *P) {
     // real items for every plan (the diagonal's product is Laplace), complex
     // ones for Helmholtz plans only
     for (int v = 0; v < (P->green == BEM_HELMHOLTZ ? 2 : 1); v++) {
-        const int slots = 8 * nf2_u(v + 1);
+        const int slots = P->prm.precision == BEM_MIXED ? 8 * nf2_u(v + 1) : ND_SLOTS;
         std::vector<int2> items;
         std::vector<int64_t> cost;
         for (int li = 0; li < t.nleaf; li++) {
@@ -952,21 +920,22 @@ void MIndex::init(int p_) {
     deg_off[p + 1] = c;
 }
 
-static Tabs tabs_of(const bem_plan *P) {
+Tabs tabs_of(const bem_plan *P) {
     return Tabs{P->d_m, P->d_n, P->d_k, P->d_idx3, P->d_fact, P->mi.p, P->mi.np,
                 P->lev_var ? P->d_lev_p : nullptr};
 }
 
-static TreeView view_of(const bem_plan *P) {
+TreeView view_of(const bem_plan *P) {
     const Tree &t = P->t;
     return TreeView{t.level, t.ix, t.iy, t.iz, t.parent, t.child0, t.nchild, t.nb, t.ne, t.eb, t.ee, t.leaves,
-                    t.near_ptr, t.near_idx, t.inter_ptr, t.inter_idx, t.node_perm, t.cx, t.cy, t.cz,
+                    t.near_ptr, t.near_idx, t.inter_ptr, t.inter_idx, t.node_perm, t.cx, t.cy, t.cz, t.r,
                     t.tx, t.ty, t.tz, t.side};
 }
 
-static QuadView quad_of(const bem_plan *P) {
+QuadView quad_of(const bem_plan *P) {
     const Quad &q = P->q;
-    return QuadView{q.x, q.y, q.z, q.nx, q.ny, q.nz, q.w, q.fx, q.fy, q.fz, q.fnx, q.fny, q.fnz, q.fw};
+    return QuadView{q.x, q.y, q.z, q.nx, q.ny, q.nz, q.w, q.fx, q.fy, q.fz, q.fnx, q.fny, q.fnz, q.fw,
+                    q.lx, q.ly, q.lz, q.lnx, q.lny, q.lnz};
 }
 
 // Shape-function values at the 7 rule points, in constant memory.  Written
@@ -1062,6 +1031,7 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
     }
     set_translation_attributes();
     set_near_attributes();
+    if (!mx) BEM_TRY(near_pairs_prepare(P));
     BEM_TRY(build_translation_tables(P, s));
     BEM_LAUNCH_CHECK();
     return BEM_OK;
@@ -1104,8 +1074,12 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
             else (k_near_f32<C, false><<<ni, NF2_T, tile_sm, s>>>(ni, it, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
         }
     } else {
-        if (op == BEM_OP_A) (k_near<R, C, true><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
-        else (k_near<R, C, false><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
+        if (near_pairs_apply(P, C, kwave)) {
+            BEM_TRY(launch_near_pairs<C>(P, op, kwave, f, L, ytmp, s));
+        } else if constexpr (C == 2) {
+            if (op == BEM_OP_A) (k_near<true><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
+            else (k_near<false><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
+        }
     }
     BEM_LAUNCH_CHECK();
     if (ev) BEM_CUDA(cudaEventRecord(ev[6], s));

@@ -136,8 +136,7 @@ __device__ __forceinline__ void normal_jac(int npe, double s, double t, const do
 __global__ void k_geometry(int E, int npe, const int *__restrict__ el_phi, const double *__restrict__ nodes,
                            const int *__restrict__ leaf_of_node, const double *__restrict__ cx,
                            const double *__restrict__ cy, const double *__restrict__ cz, double *qx, double *qy,
-                           double *qz, double *qnx, double *qny, double *qnz, double *qw, float *fx, float *fy,
-                           float *fz, float *fnx, float *fny, float *fnz, float *fw) {
+                           double *qz, double *qnx, double *qny, double *qnz, double *qw, Quad out, double scale) {
     int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= E * NQ) return;
     int i = o / NQ, q = o % NQ;
@@ -151,11 +150,15 @@ __global__ void k_geometry(int E, int npe, const int *__restrict__ el_phi, const
     qnx[o] = n[0]; qny[o] = n[1]; qnz[o] = n[2];
     qw[o] = w;
     int leaf = leaf_of_node[el_phi[(size_t)i * npe]];
-    fx[o] = (float)(x[0] - cx[leaf]);
-    fy[o] = (float)(x[1] - cy[leaf]);
-    fz[o] = (float)(x[2] - cz[leaf]);
-    fnx[o] = (float)n[0]; fny[o] = (float)n[1]; fnz[o] = (float)n[2];
-    fw[o] = (float)w;
+    const double d[3] = {(x[0] - cx[leaf]) * scale, (x[1] - cy[leaf]) * scale, (x[2] - cz[leaf]) * scale};
+    const float dh[3] = {(float)d[0], (float)d[1], (float)d[2]}, nh[3] = {(float)n[0], (float)n[1], (float)n[2]};
+    out.fx[o] = dh[0]; out.fy[o] = dh[1]; out.fz[o] = dh[2];
+    out.fnx[o] = nh[0]; out.fny[o] = nh[1]; out.fnz[o] = nh[2];
+    out.fw[o] = (float)w;
+    if (out.lx) {                                   // float64 plans: the low parts of the pairs
+        out.lx[o] = (float)(d[0] - dh[0]); out.ly[o] = (float)(d[1] - dh[1]); out.lz[o] = (float)(d[2] - dh[2]);
+        out.lnx[o] = (float)(n[0] - nh[0]); out.lny[o] = (float)(n[1] - nh[1]); out.lnz[o] = (float)(n[2] - nh[2]);
+    }
 }
 
 // Also writes a float32 bound per element for the pair search: the centroid
@@ -220,9 +223,17 @@ int build_geometry(bem_plan *P, cudaStream_t s) {
     BEM_TRY(A.alloc(&q.fx, Q)); BEM_TRY(A.alloc(&q.fy, Q)); BEM_TRY(A.alloc(&q.fz, Q));
     BEM_TRY(A.alloc(&q.fnx, Q)); BEM_TRY(A.alloc(&q.fny, Q)); BEM_TRY(A.alloc(&q.fnz, Q));
     BEM_TRY(A.alloc(&q.fw, Q));
+    // float64 plans keep float32 pairs, scaled by a power of two so that any
+    // body's coordinates fit float32's range
+    double scale = 1.0;
+    if (P->prm.precision == BEM_F64) {
+        BEM_TRY(A.alloc(&q.lx, Q)); BEM_TRY(A.alloc(&q.ly, Q)); BEM_TRY(A.alloc(&q.lz, Q));
+        BEM_TRY(A.alloc(&q.lnx, Q)); BEM_TRY(A.alloc(&q.lny, Q)); BEM_TRY(A.alloc(&q.lnz, Q));
+        scale = std::ldexp(1.0, -std::ilogb(t.side));
+    }
     (k_geometry<<<(int)((Q + 255) / 256), 256, 0, s>>>((int)P->E, P->npe, t.el_phi, P->nodes, t.leaf_of_node, t.cx,
-                                                       t.cy, t.cz, q.x, q.y, q.z, q.nx, q.ny, q.nz, q.w, q.fx, q.fy,
-                                                       q.fz, q.fnx, q.fny, q.fnz, q.fw), ::bem::count_launch());
+                                                       t.cy, t.cz, q.x, q.y, q.z, q.nx, q.ny, q.nz, q.w, q, scale),
+     ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     return BEM_OK;
 }
