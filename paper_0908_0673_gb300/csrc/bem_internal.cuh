@@ -43,6 +43,9 @@ extern thread_local long long *tl_capture_count;
 constexpr int QBITS = 21;   // Morton bits per axis
 constexpr int PMAX = 20;    // largest supported expansion order
 constexpr int NQ = 7;       // regular quadrature points per element
+// the six axis permutations of the M2L's canonical offset classes:
+// SY_PERMS[q][i] = canonical position of axis i
+constexpr int SY_PERMS[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
 
 // Radon's 7-point degree-5 rule on the reference triangle (Stroud T2:5-1),
 // point q in owner order: the centroid with weight 9/80, then two orbits,
@@ -326,6 +329,14 @@ struct FmmState {
     float *sy_img = nullptr;            // [class][hi, lo][image floats] class-matrix images (tensor-core form)
     void *sy_Lp = nullptr;              // [pair][sy_ldp][C] canonical-frame local contributions
     bem::TcPlan sy_g;
+    // SIMT form (m2l_simt.cu)
+    int sg_kt = 0, sg_ldq = 0;          // first column of the tail; row stride of the permuted moments
+    int sg_batch = 0;                   // classes whose images are held at a time
+    std::vector<int> sy_htile;          // host: class of every tile
+    size_t sg_vec = 0;                  // float4 of a class's image
+    int *sg_colx = nullptr, *sg_E = nullptr;   // column extents and offsets; float64 plans: exponent of each box's moments
+    void *sg_img = nullptr;             // [class][sg_vec] float4: T in the order it is consumed
+    float *sg_Mq = nullptr;             // [box][6][sg_ldq][words] moments under each axis permutation, per product
     float *p2m_W = nullptr;             // [Q][np] stored double-layer P2M weights (float32 plans)
     float *xf = nullptr;                // float32 copy of a product's input (correction product)
     std::vector<int> lev_p;             // expansion order of each tree level
@@ -419,7 +430,7 @@ int launch_m2l_tc(bem_plan *P, const float *M, float *L, cudaStream_t s);
 void set_tc_attributes();
 template <class R, int C>
 int launch_m2l_sy(bem_plan *P, const R *M, R *L, cudaStream_t s);
-size_t sy_simt_smem_bytes(int prec_float, int C, int np, int p);
+int build_simt_tables(bem_plan *P, cudaStream_t s);
 void set_sy_attributes();
 int launch_m2l_derivs(bem_plan *P, int ncls, const double *rho, const double *kh, double *D, float *fD,
                       cudaStream_t s);

@@ -51,9 +51,6 @@ constexpr int TC_NPROD = TC_T / 32 - TC_PROD0;
 constexpr long long TC_WAIT = 4000000000ll;      // clock cycles before a wait gives up
 constexpr int TC_SMEM_MAX = 227 * 1024;
 
-// the six axis permutations; PERMS[q][i] = canonical position of axis i
-constexpr int PERMS[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-
 struct TcArgs {
     TcPlan g;
     int np, ldp, ntile, nkc;
@@ -525,7 +522,7 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
         int pi[3];
         for (int j = 0; j < 3; j++) pi[order[j]] = j;
         int q = 0;
-        while (!(PERMS[q][0] == pi[0] && PERMS[q][1] == pi[1] && PERMS[q][2] == pi[2])) q++;
+        while (!(SY_PERMS[q][0] == pi[0] && SY_PERMS[q][1] == pi[1] && SY_PERMS[q][2] == pi[2])) q++;
         fsig[c] = q * 8 + ((K[0] < 0 ? 1 : 0) | (K[1] < 0 ? 2 : 0) | (K[2] < 0 ? 4 : 0));
         fkey[c] = Key{{(long long)dls[c], (long long)levs[c], std::llabs(K[order[0]]), std::llabs(K[order[1]]),
                        std::llabs(K[order[2]])}};
@@ -600,13 +597,17 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
 }
 
 // Batches and tiles for rows of row_bytes: the targets are cut into runs whose
-// interaction lists hold at most SY_LP_BYTES of rows together (a run holds at
-// least one whole list), and within a run the pairs are sorted by canonical
-// class (counting sort, stable in list order) and cut into tiles of up to
-// 128 pairs of one class.  Each run's rows are computed into the same buffer
-// and gathered before the next run starts, so the buffer is bounded however
-// large the mesh, and every target's sum keeps its list order.
-constexpr size_t SY_LP_BYTES = (size_t)128 << 20;
+// interaction lists hold at most SY_LP_BYTES of rows together, or SY_LP_NODE a
+// node if that is more (a run holds at least one whole list), and within a run
+// the pairs are sorted by canonical class (counting sort, stable in list order)
+// and cut into tiles of up to 128 pairs of one class.  Each run's rows are
+// computed into the same buffer and gathered before the next run starts, so the
+// buffer is bounded by the mesh, and every target's sum keeps its list order.
+// Fewer runs fill the tiles and the last waves better (the complex M2L of a
+// sphere of 20,480 tri6: 1182, 1024, 916, 789 us with 64, 128, 256 MB and one
+// run); a node's rows are about 13 KB at p = 10 there.  The diagonal's
+// temporary state, held beside the plan's own, stays at SY_LP_BYTES.
+constexpr size_t SY_LP_BYTES = (size_t)128 << 20, SY_LP_NODE = 14 << 10;
 
 static int build_sym_tiles(bem_plan *P, size_t row_bytes, int64_t &max_rows, cudaStream_t s) {
     const int nbox = P->t.nbox, nc = P->sy_ncls;
@@ -614,7 +615,8 @@ static int build_sym_tiles(bem_plan *P, size_t row_bytes, int64_t &max_rows, cud
     const int64_t npair = P->t.n_inter;
     int64_t longest = 0;
     for (int b = 0; b < nbox; b++) longest = std::max<int64_t>(longest, ip[b + 1] - ip[b]);
-    const int64_t cap = std::max<int64_t>(std::max<int64_t>(1, longest), (int64_t)(SY_LP_BYTES / row_bytes));
+    const size_t bytes = P->diag_mode ? SY_LP_BYTES : std::max(SY_LP_BYTES, SY_LP_NODE * (size_t)P->N);
+    const int64_t cap = std::max<int64_t>(std::max<int64_t>(1, longest), (int64_t)(bytes / row_bytes));
     std::vector<int> psrc(std::max<int64_t>(1, npair)), psig(std::max<int64_t>(1, npair)),
         pu(std::max<int64_t>(1, npair)), tcls, tst, tcnt, cnt(nc + 1);
     P->sy_bt.assign(1, 0);
@@ -647,6 +649,7 @@ static int build_sym_tiles(bem_plan *P, size_t row_bytes, int64_t &max_rows, cud
         t0 = t1;
     }
     P->sy_ntile = (int)tcls.size();
+    P->sy_htile = tcls;
     Arena &A = P->arena;
     auto up = [&](auto **d, const auto &h) -> int {
         using T = std::decay_t<decltype(h[0])>;
@@ -735,7 +738,7 @@ int build_sym_tables(bem_plan *P, cudaStream_t s) {
     for (int q = 0; q < 6; q++)
         for (int sb = 0; sb < 8; sb++) {
             const int sig = q * 8 + sb;
-            const int *pi = PERMS[q];
+            const int *pi = SY_PERMS[q];
             int pinv[3];
             for (int i = 0; i < 3; i++) pinv[pi[i]] = i;
             for (int h = 0; h < np; h++) {
@@ -763,8 +766,8 @@ int build_sym_tables(bem_plan *P, cudaStream_t s) {
     BEM_TRY(up(&P->sy_invf, invf));
     const int ncls = P->sy_ncls;
     BEM_TRY(A.alloc(&P->sy_D, std::max<size_t>(1, (size_t)ncls * np * C)));
-    if (mx) BEM_TRY(A.alloc(&P->sy_fD, std::max<size_t>(1, (size_t)ncls * np * C)));
-    BEM_TRY(launch_m2l_derivs(P, ncls, P->sy_rho, C == 2 ? P->sy_kh : nullptr, P->sy_D, mx ? P->sy_fD : nullptr, s));
+    if (mx && C == 1) BEM_TRY(A.alloc(&P->sy_fD, std::max<size_t>(1, (size_t)ncls * np)));
+    BEM_TRY(launch_m2l_derivs(P, ncls, P->sy_rho, C == 2 ? P->sy_kh : nullptr, P->sy_D, P->sy_fD, s));
     TcPlan g{};
     int ldp = 0, nkc = 0;
     const bool tc = C == 1 && mx && ncls > 0 && !P->lev_var && tc_plan(mi, deg, g, ldp, nkc);
@@ -826,10 +829,7 @@ int build_sym_tables(bem_plan *P, cudaStream_t s) {
         P->sy_nkc = nkc;
     } else {
         ldp = (np + 3) / 4 * 4;
-        if (sy_simt_smem_bytes(mx, C, np, p) > (size_t)200 * 1024) {
-            set_error("M2L: order %d needs more shared memory than a block has", p);
-            return BEM_EINVAL;
-        }
+        BEM_TRY(build_simt_tables(P, s));
     }
     int64_t max_rows = 0;
     BEM_TRY(build_sym_tiles(P, (size_t)ldp * C * (mx ? sizeof(float) : sizeof(double)), max_rows, s));
@@ -847,8 +847,11 @@ void free_sym_tables(bem_plan *P) {
     for (void *q : {(void *)P->sy_img, (void *)P->sy_fwdq, (void *)P->sy_sgn, (void *)P->sy_Mq, (void *)P->sy_fwd, (void *)P->sy_inv, (void *)P->sy_D,
                     (void *)P->sy_fD, (void *)P->sy_Lp, (void *)P->sy_mexp, (void *)P->sy_invf, (void *)P->sy_ord,
                     (void *)P->sy_tile_cls, (void *)P->sy_tile_start, (void *)P->sy_tile_cnt, (void *)P->sy_src,
-                    (void *)P->sy_sig, (void *)P->sy_pair})
+                    (void *)P->sy_sig, (void *)P->sy_pair, (void *)P->sg_colx, (void *)P->sg_img, (void *)P->sg_Mq, (void *)P->sg_E})
         A.release(q);
+    P->sg_colx = P->sg_E = nullptr;
+    P->sg_img = nullptr;
+    P->sg_Mq = nullptr;
     P->sy_tile_cls = P->sy_tile_start = P->sy_tile_cnt = P->sy_src = P->sy_sig = P->sy_pair = nullptr;
     P->sy_ord = nullptr;
     P->sy_ntile = 0;

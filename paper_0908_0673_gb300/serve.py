@@ -96,9 +96,11 @@ class EngineError(RuntimeError):
 # exist at the set-up peak) and the Krylov basis.  The values bound the
 # measured peaks (9-28 kB per node on spheres, ellipsoids and graded cubes of
 # 1k-18k quadratic elements, before the two orders overlapped) with a margin;
-# the GPU tests check the bound.  The fixed part holds the M2L row buffers of
-# the two orders, each capped at 128 MiB whatever the mesh (rows are computed
-# and gathered in runs of targets), and 64 MiB of small tables.
+# the GPU tests check the bound.  The M2L row buffers (rows are computed and
+# gathered in runs of targets) are capped: the diagonal's order at 128 MiB and
+# the plan's own at the larger of 128 MiB and 14 KiB per node, the class images
+# of the SIMT form at 48 MiB and 4 KiB per node.  The fixed part holds the two
+# 128 MiB and 64 MiB of small tables.
 _BYTES_PER_NODE = {
     (bem.BEM_LAPLACE, bem.BEM_F64): 36_000,
     (bem.BEM_LAPLACE, bem.BEM_MIXED): 36_000,
