@@ -192,6 +192,7 @@ static int plan_setup(bem_plan *P, cudaStream_t s) {
     if (rc == BEM_OK) rc = diagonal_product(P, s2);
     if (rc == BEM_OK) BEM_CUDA(cudaEventRecord(ev[3], s2));
     if (rc == BEM_OK) rc = alloc_fmm(P, s3);
+    if (rc == BEM_OK) rc = field_prepare(P);
     if (rc == BEM_OK) BEM_CUDA(cudaEventRecord(ev[5], s3));
     if (rc == BEM_OK) BEM_CUDA(cudaStreamWaitEvent(s, ev[5], 0));
     if (rc == BEM_OK) BEM_CUDA(cudaStreamWaitEvent(s, ev[3], 0));

@@ -392,6 +392,10 @@ struct bem_plan : bem::FmmState {
     int *leaf_near_ptr = nullptr, *leaf_near_idx = nullptr;   // leaf_descend = 0: near lists opened down to leaves
     const float4 *circle = nullptr;             // unit-circle table of the float64 Helmholtz near field (the library's)
     int last_op = -1;
+    // field evaluation workspaces (field.cu): strengths of phi and chi, monomial
+    // element data, centroids, harmonic coefficients of the boxes
+    double *fd_str = nullptr, *fd_elem = nullptr, *fd_cen = nullptr, *fd_harm = nullptr;
+    void *fd_fcen = nullptr;
     // GMRES workspace
     double *V = nullptr, *H = nullptr, *gs = nullptr, *w = nullptr, *xk = nullptr, *bvec = nullptr;
     double *zbuf = nullptr;             // the preconditioned Arnoldi vector M^-1 V_j (the product's input)
@@ -438,6 +442,7 @@ template <class R, int C>
 int launch_translations(bem_plan *P, R *M, R *L, cudaStream_t s, cudaEvent_t *ev);
 template <class R, int C>
 int launch_m2m(bem_plan *P, R *M, cudaStream_t s, int lmin = 0);
+int field_prepare(bem_plan *P);
 int field_moments(bem_plan *P, const void *phi, const void *chi, cudaStream_t s);
 int build_near_items(bem_plan *P);
 int diagonal_prepare(bem_plan *P, cudaStream_t s);

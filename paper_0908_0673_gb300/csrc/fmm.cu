@@ -1103,12 +1103,19 @@ static int field_moments_t(bem_plan *P, const void *phi, const void *chi, R *f, 
     const Tree &t = P->t;
     const int Q = (int)P->Q;
     const int *sk = P->skip;
-    BEM_TRY(set_slots(P, phi, nullptr, s));
-    (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, t.el_phi, P->q.w, P->xptr, f, sk), ::bem::count_launch());
-    launch_p2m<R, C, true>(t.nleaf, tb, tv, qv, f, M, sk, s);
-    BEM_TRY(set_slots(P, chi, nullptr, s));
-    (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, t.el_chi, P->q.w, P->xptr, f, sk), ::bem::count_launch());
-    launch_p2m<R, C, false>(t.nleaf, tb, tv, qv, f, Bm, sk, s);
+    // strengths in float64 for the direct part, and in the plan's precision for
+    // the moments (float64 plans: the same array)
+    for (int part = 0; part < 2; part++) {
+        double *str = P->fd_str + (size_t)part * Q * C;
+        const int *el = part ? t.el_chi : t.el_phi;
+        BEM_TRY(set_slots(P, part ? chi : phi, nullptr, s));
+        (k_p2q<double, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, str, sk), ::bem::count_launch());
+        const R *src = f;
+        if constexpr (sizeof(R) == sizeof(double)) src = str;
+        else (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, f, sk), ::bem::count_launch());
+        if (part) launch_p2m<R, C, false>(t.nleaf, tb, tv, qv, src, Bm, sk, s);
+        else launch_p2m<R, C, true>(t.nleaf, tb, tv, qv, src, M, sk, s);
+    }
     const size_t n = (size_t)t.nbox * P->mi.np * C;
     (k_sub_moments<R><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, M, Bm), ::bem::count_launch());
     BEM_LAUNCH_CHECK();
