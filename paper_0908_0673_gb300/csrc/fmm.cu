@@ -55,7 +55,8 @@ __global__ void k_p2q(int Q, int npe, const int *__restrict__ el_idx, const doub
 }
 
 // ---------------------------------------------------------------------------
-// P2M: one block per leaf, threads over multi-indices, sources in batches of 32
+// P2M of float32 plans: one block per leaf, threads over multi-indices, sources
+// in batches of 32 (float64 plans: p2m_f64.cu)
 // ---------------------------------------------------------------------------
 constexpr int P2M_T = 128, P2M_B = 32;
 // index slots per thread (NS >= ceil(n_p / P2M_T)): instantiated for orders
@@ -70,10 +71,11 @@ constexpr int p2m_slots(int np) { return np <= 3 * P2M_T ? 3 : np <= 8 * P2M_T ?
 // monopole coefficient is Px Py Pz and a double-layer one, the normal
 // derivative of the monomial, (Qx Py + Px Qy) Pz + Px Py Qz: three paired
 // loads and no branches per (point, coefficient).
-template <class R, int C, bool DL, bool WEIGHTS, int NS>
-__global__ void __launch_bounds__(P2M_T) k_p2m(int nleaf, Tabs tb, TreeView tv, QuadView qv, const R *__restrict__ f,
-                                               R *__restrict__ M, const int *__restrict__ skip, R *__restrict__ W = nullptr) {
-    using R2 = typename std::conditional<sizeof(R) == sizeof(float), float2, double2>::type;
+template <int C, bool DL, bool WEIGHTS, int NS>
+__global__ void __launch_bounds__(P2M_T) k_p2m(int nleaf, Tabs tb, TreeView tv, QuadView qv, const float *__restrict__ f,
+                                               float *__restrict__ M, const int *__restrict__ skip, float *__restrict__ W = nullptr) {
+    using R = float;
+    using R2 = float2;
     if (skip && *skip) return;
     const int li = blockIdx.x;
     if (li >= nleaf) return;
@@ -84,7 +86,6 @@ __global__ void __launch_bounds__(P2M_T) k_p2m(int nleaf, Tabs tb, TreeView tv, 
     __shared__ R sf[P2M_B][C];
     const double h = scalbn(tv.side, -tv.level[b]);
     const R hinv = (R)(1.0 / h);
-    const double c0 = tv.cx[b], c1 = tv.cy[b], c2 = tv.cz[b];
     int am[NS], an[NS], ak[NS];
     R acc[NS][C];
 #pragma unroll
@@ -105,16 +106,9 @@ __global__ void __launch_bounds__(P2M_T) k_p2m(int nleaf, Tabs tb, TreeView tv, 
             R d = (R)0, nd = (R)0;
             if (pt < nb) {
                 int o = base + pt;
-                if constexpr (sizeof(R) == sizeof(double)) {
-                    double xx = ax == 0 ? qv.x[o] - c0 : (ax == 1 ? qv.y[o] - c1 : qv.z[o] - c2);
-                    d = (R)(xx / h);
-                    if (DL) nd = (R)(ax == 0 ? qv.nx[o] : (ax == 1 ? qv.ny[o] : qv.nz[o]));
-                } else {
-                    // float path: offsets from the owning leaf (this box) centre
-                    R xx = ax == 0 ? (R)qv.fx[o] : (ax == 1 ? (R)qv.fy[o] : (R)qv.fz[o]);
-                    d = xx * hinv;
-                    if (DL) nd = (R)(ax == 0 ? qv.fnx[o] : (ax == 1 ? qv.fny[o] : qv.fnz[o]));
-                }
+                // offsets from the owning leaf (this box) centre
+                d = (ax == 0 ? qv.fx[o] : (ax == 1 ? qv.fy[o] : qv.fz[o])) * hinv;
+                if (DL) nd = ax == 0 ? qv.fnx[o] : (ax == 1 ? qv.fny[o] : qv.fnz[o]);
             }
             nd *= hinv;
             R v = (R)1, vm = (R)0;                    // d^e, d^(e-1)
@@ -226,13 +220,13 @@ __global__ void __launch_bounds__(P2S_T) k_p2m_stored(int nleaf, int np, TreeVie
 
 
 // P2M launches with the slot count of the plan's largest order
-template <class R, int C, bool DL, bool WEIGHTS = false>
-static void launch_p2m(int nleaf, const Tabs &tb, const TreeView &tv, const QuadView &qv, const R *f, R *M,
-                       const int *skip, cudaStream_t s, R *W = nullptr) {
+template <int C, bool DL, bool WEIGHTS = false>
+static void launch_p2m(int nleaf, const Tabs &tb, const TreeView &tv, const QuadView &qv, const float *f, float *M,
+                       const int *skip, cudaStream_t s, float *W = nullptr) {
     const int ns = p2m_slots(tb.np);
-    if (ns == 3) (k_p2m<R, C, DL, WEIGHTS, 3><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
-    else if (ns == 8) (k_p2m<R, C, DL, WEIGHTS, 8><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
-    else (k_p2m<R, C, DL, WEIGHTS, 14><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
+    if (ns == 3) (k_p2m<C, DL, WEIGHTS, 3><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
+    else if (ns == 8) (k_p2m<C, DL, WEIGHTS, 8><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
+    else (k_p2m<C, DL, WEIGHTS, 14><<<nleaf, P2M_T, 0, s>>>(nleaf, tb, tv, qv, f, M, skip, W), ::bem::count_launch());
 }
 
 template <int C>
@@ -1025,13 +1019,16 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
         // stored P2M weights of the double layer (op A, every product of a solve)
         BEM_TRY(A.alloc(&P->p2m_W, (size_t)P->Q * np));
         const Tree &t = P->t;
-        launch_p2m<float, 1, true, true>(t.nleaf, tabs_of(P), view_of(P), quad_of(P), nullptr, nullptr, nullptr, s,
+        launch_p2m<1, true, true>(t.nleaf, tabs_of(P), view_of(P), quad_of(P), nullptr, nullptr, nullptr, s,
                                          P->p2m_W);
         BEM_LAUNCH_CHECK();
     }
     set_translation_attributes();
     set_near_attributes();
-    if (!mx) BEM_TRY(near_pairs_prepare(P));
+    if (!mx) {
+        BEM_TRY(near_pairs_prepare(P));
+        BEM_TRY(p2m_pairs_prepare());
+    }
     BEM_TRY(build_translation_tables(P, s));
     BEM_LAUNCH_CHECK();
     return BEM_OK;
@@ -1056,11 +1053,10 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     if constexpr (sizeof(R) == sizeof(float)) {
         if (op == BEM_OP_A && P->p2m_W)
             launch_p2m_stored<C>(t.nleaf, np, tv, P->p2m_W, f, M, sk, s);
-        else if (op == BEM_OP_A) launch_p2m<R, C, true>(t.nleaf, tb, tv, qv, f, M, sk, s);
-        else launch_p2m<R, C, false>(t.nleaf, tb, tv, qv, f, M, sk, s);
+        else if (op == BEM_OP_A) launch_p2m<C, true>(t.nleaf, tb, tv, qv, f, M, sk, s);
+        else launch_p2m<C, false>(t.nleaf, tb, tv, qv, f, M, sk, s);
     } else {
-        if (op == BEM_OP_A) launch_p2m<R, C, true>(t.nleaf, tb, tv, qv, f, M, sk, s);
-        else launch_p2m<R, C, false>(t.nleaf, tb, tv, qv, f, M, sk, s);
+        BEM_TRY(launch_p2m_pairs<C>(P, op == BEM_OP_A, f, M, s));
     }
     BEM_LAUNCH_CHECK();
     if (ev) BEM_CUDA(cudaEventRecord(ev[2], s));
@@ -1110,11 +1106,14 @@ static int field_moments_t(bem_plan *P, const void *phi, const void *chi, R *f, 
         const int *el = part ? t.el_chi : t.el_phi;
         BEM_TRY(set_slots(P, part ? chi : phi, nullptr, s));
         (k_p2q<double, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, str, sk), ::bem::count_launch());
-        const R *src = f;
-        if constexpr (sizeof(R) == sizeof(double)) src = str;
-        else (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, f, sk), ::bem::count_launch());
-        if (part) launch_p2m<R, C, false>(t.nleaf, tb, tv, qv, src, Bm, sk, s);
-        else launch_p2m<R, C, true>(t.nleaf, tb, tv, qv, src, M, sk, s);
+        if constexpr (sizeof(R) == sizeof(double)) {
+            BEM_TRY(launch_p2m_pairs<C>(P, !part, str, part ? Bm : M, s));
+        } else {
+            (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, f, sk), ::bem::count_launch());
+            if (part) launch_p2m<C, false>(t.nleaf, tb, tv, qv, f, Bm, sk, s);
+            else if (P->p2m_W) launch_p2m_stored<C>(t.nleaf, P->mi.np, tv, P->p2m_W, f, M, sk, s);
+            else launch_p2m<C, true>(t.nleaf, tb, tv, qv, f, M, sk, s);
+        }
     }
     const size_t n = (size_t)t.nbox * P->mi.np * C;
     (k_sub_moments<R><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, M, Bm), ::bem::count_launch());

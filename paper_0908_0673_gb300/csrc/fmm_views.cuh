@@ -40,4 +40,9 @@ bool near_pairs_apply(const bem_plan *P, int C, double kwave);
 template <int C>
 int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, const double *L, double *ytmp, cudaStream_t s);
 
+// P2M of float64 plans in float32 pairs (p2m_f64.cu)
+int p2m_pairs_prepare();
+template <int C>
+int launch_p2m_pairs(bem_plan *P, bool dl, const double *f, double *M, cudaStream_t s);
+
 }  // namespace bem

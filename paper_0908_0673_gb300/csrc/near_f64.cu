@@ -38,6 +38,7 @@
 #include <mutex>
 #include <vector>
 
+#include "cluster.cuh"
 #include "dfloat.cuh"
 #include "fmm_views.cuh"
 
@@ -247,24 +248,6 @@ __device__ __forceinline__ void pair_step(const P2 (&tH)[3], const P2 (&t1)[3], 
     pmacc(B, nB, Bl, -s.fh[C - 1], -s.fl[C - 1], ah[0], al[0]);
     pmacc(A, nA, Al, s.fh[C - 1], s.fl[C - 1], ah[C - 1], al[C - 1]);
     pmacc(B, nB, Bl, s.fh[0], s.fl[0], ah[C - 1], al[C - 1]);
-}
-
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
-}
-// a double of another block's shared memory, at the address p has here
-__device__ __forceinline__ double peer_double(const double *p, unsigned rank) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-    unsigned r;
-    double v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r));
-    return v;
 }
 
 template <int C, bool DL>
@@ -607,24 +590,14 @@ int launch(bem_plan *P, double kwave, const double *f, const double *L, double *
     // four times over (a last wave of small shares), at most a portable cluster
     int ns = 1;
     while (ns < ND_MAXC && ni * ns < 8 * P->sm_count) ns *= 2;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ns;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(ni * ns));
-    cfg.blockDim = dim3(ND_T);
-    cfg.dynamicSmemBytes = nd_dyn_bytes(C, DL);
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = ns > 1 ? 1 : 0;
     TreeView tv = view_of(P);
     if (P->leaf_near_ptr) {                          // every entry a leaf, the sources' own box
         tv.near_ptr = P->leaf_near_ptr;
         tv.near_idx = P->leaf_near_idx;
     }
-    BEM_CUDA(cudaLaunchKernelEx(&cfg, k_near_pairs<C, DL>, ns, (const int2 *)P->near_items[C - 1], tabs_of(P), tv, quad_of(P), kwave, f, L, ytmp, P->circle, (const int *)P->skip));
-    count_launch();
+    BEM_TRY(launch_cluster(k_near_pairs<C, DL>, (unsigned)(ni * ns), ND_T, nd_dyn_bytes(C, DL), ns, s, ns,
+                           (const int2 *)P->near_items[C - 1], tabs_of(P), tv, quad_of(P), kwave, f, L, ytmp, P->circle,
+                           (const int *)P->skip));
     return BEM_OK;
 }
 
