@@ -329,6 +329,7 @@ struct FmmState {
     float *sy_img = nullptr;            // [class][hi, lo][image floats] class-matrix images (tensor-core form)
     void *sy_Lp = nullptr;              // [pair][sy_ldp][C] canonical-frame local contributions
     bem::TcPlan sy_g;
+    void *shift_G = nullptr;            // per-axis shift factors [M2M, L2L][p + 1][p + 1] in the plan's precision
     // SIMT form (m2l_simt.cu)
     int sg_kt = 0, sg_ldq = 0;          // first column of the tail; row stride of the permuted moments
     int sg_batch = 0;                   // classes whose images are held at a time

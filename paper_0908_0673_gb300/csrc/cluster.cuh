@@ -24,6 +24,16 @@ __device__ __forceinline__ double peer_double(const double *p, unsigned rank) {
     return v;
 }
 
+__device__ __forceinline__ double peer_load(const double *p, unsigned rank) { return peer_double(p, rank); }
+__device__ __forceinline__ float peer_load(const float *p, unsigned rank) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    unsigned r;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r));
+    return v;
+}
+
 template <class... P, class... A>
 int launch_cluster(void (*kernel)(P...), unsigned blocks, int threads, size_t smem, int cluster, cudaStream_t s, A... args) {
     cudaLaunchAttribute at[1];

@@ -26,7 +26,7 @@
 #include <unordered_map>
 #include <vector>
 
-#include "bem_internal.cuh"
+#include "cluster.cuh"
 
 namespace bem {
 
@@ -46,204 +46,165 @@ __device__ __forceinline__ void cmac(R *acc, R cf, const R *v) {
 // (s_i = -1 where the child lies on the low side of axis i), so each shift is
 // done axis by axis: an output of one pass sums at most p + 1 terms, and the
 // degree bound |.| <= p carries through the passes unchanged.  Multi-index
-// table and per-axis factors sit in shared memory.  M2M: every child of the
-// parent at once, children then added in a fixed order; L2L: one child per
-// block.  Deterministic.
+// table and per-axis factors sit in shared memory.  One child per block either
+// way.  Deterministic.
+//
+// A level is bound by its blocks' latency (it takes as long for one parent as
+// for hundreds), so a block does little one after the other: its coefficients,
+// the packed multi-indices and the factors come in one round of loads, and the
+// eight children of a parent go to the eight blocks of a cluster, whose sums
+// are added in child order through distributed shared memory.  With the
+// children in one block and the factors computed there, M2M of the cube of 24,300
+// tri6 (float32, four levels) took 57 us, now 36, of 8,748 (float64) 137, now
+// 40; L2L 31 -> 21 and 33 -> 20.
 // ---------------------------------------------------------------------------
-constexpr int MM_T = 512;
+constexpr int MM_T = 320, MM_CL = 8;      // threads; blocks per parent (M2M)
 
-// Shift tables in shared memory, built from the multi-indices alone: the np
-// coefficients' (m, n, k) packed as m | n << 8 | k << 16, the index of every
-// multi-index of degree <= p (the only ones a pass looks up) at
-// (m (p + 1) + n) (p + 1) + k, and the per-axis factors from exact integer
-// binomials.  One round of global loads (tm, tn, tk) per block.
-__device__ __forceinline__ int binom_int(int n, int k) {
-    int b = 1;                                  // C(n - k + i, i) after step i: exact
-    for (int i = 1; i <= k; i++) b = b * (n - k + i) / i;
-    return b;
-}
-template <class R>
-__device__ __forceinline__ void shift_tables(int p, int np, const int *__restrict__ tm, const int *__restrict__ tn,
-                                             const int *__restrict__ tk, bool m2m, short *sIdx, R *sG, int *sMNK) {
-    const int P1 = p + 1;
-    for (int a = threadIdx.x; a < np; a += blockDim.x) {
-        const int m = tm[a], n = tn[a], k = tk[a];
-        sMNK[a] = m | n << 8 | k << 16;
-        sIdx[(m * P1 + n) * P1 + k] = (short)a;
-    }
-    for (int i = threadIdx.x; i < P1 * P1; i += blockDim.x) {
-        const int a = i / P1, g = i - a * P1;
-        // M2M: binom(a, g) 2^-g (g <= a);  L2L: binom(a + g, a) 4^-g (a + g <= p)
-        R v = (R)0, sc = (R)1;
-        for (int j = 0; j < g; j++) sc *= m2m ? (R)0.5 : (R)0.25;
-        if (m2m && g <= a) v = (R)binom_int(a, g) * sc;
-        if (!m2m && a + g <= p) v = (R)binom_int(a + g, a) * sc;
-        sG[i] = v;
-    }
-}
-
-// shared-memory bytes of the shift tables at order p (sG, sIdx, sMNK)
+// shared-memory bytes of the shift tables at order p: factors [P1][P1], index
+// of every multi-index of degree <= p (the only ones a pass looks up) at
+// (m (p + 1) + n) (p + 1) + k, packed multi-indices [np]
 template <class R>
 __host__ __device__ inline size_t shift_tab_bytes(int p, int np) {
     const int P1 = p + 1;
     return (((size_t)sizeof(R) * P1 * P1 + sizeof(short) * P1 * P1 * P1 + 15) / 16) * 16 + 4 * (size_t)np + 16;
 }
 
-// one axis pass over nv vectors: out[v][a] = sum_g G[a_ax][g] s_v^g in[v][a -/+ g e_ax]
+// The tables and the block's nt source values, all loads of a thread in flight
+// before the first is stored.  G: factors [a][g] of stride Pm1 for the pass
+// direction; mexp: packed multi-indices.
+template <class R, int U>
+__device__ __forceinline__ void shift_load(int p, int np, int Pm1, const R *__restrict__ G, const int *__restrict__ mexp,
+                                           const R *src, int nt, short *sIdx, R *sG, int *sMNK, R *sA) {
+    const int P1 = p + 1, tid = threadIdx.x;
+    R v[U];
+    int e[2];
+#pragma unroll
+    for (int u = 0; u < U; u++) v[u] = tid + u * MM_T < nt ? src[tid + u * MM_T] : (R)0;
+#pragma unroll
+    for (int u = 0; u < 2; u++) e[u] = tid + u * MM_T < np ? __ldg(mexp + tid + u * MM_T) : 0;
+    const R g0 = tid < P1 * P1 ? G[tid / P1 * Pm1 + tid % P1] : (R)0;
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int a = tid + u * MM_T;
+        if (a < np) {
+            sMNK[a] = e[u];
+            sIdx[((e[u] & 255) * P1 + (e[u] >> 8 & 255)) * P1 + (e[u] >> 16 & 255)] = (short)a;
+        }
+    }
+    for (int a = tid + 2 * MM_T; a < np; a += MM_T) {
+        const int x = __ldg(mexp + a);
+        sMNK[a] = x;
+        sIdx[((x & 255) * P1 + (x >> 8 & 255)) * P1 + (x >> 16 & 255)] = (short)a;
+    }
+    if (tid < P1 * P1) sG[tid] = g0;
+    for (int i = tid + MM_T; i < P1 * P1; i += MM_T) sG[i] = G[i / P1 * Pm1 + i % P1];
+#pragma unroll
+    for (int u = 0; u < U; u++)
+        if (tid + u * MM_T < nt) sA[tid + u * MM_T] = v[u];
+    for (int t = tid + U * MM_T; t < nt; t += MM_T) sA[t] = src[t];
+}
+
+// one axis pass: out[a] = sum_g G[a_ax][g] s^g in[a -/+ g e_ax]
 template <class R, int C, bool DOWN>
-__device__ __forceinline__ void shift_pass(int ax, int nv, int p, int np, const int *sMNK, const short *sIdx,
-                                           const R *sG, const int *smask, const R *in, R *out) {
-    const int P1 = p + 1;
-    for (int t = threadIdx.x; t < nv * np; t += blockDim.x) {
-        const int v = t / np, a = t - v * np;
-        const int mnk = sMNK[a];
-        int c3[3] = {mnk & 255, (mnk >> 8) & 255, mnk >> 16};
-        const int e = c3[ax], rest = p - (c3[0] + c3[1] + c3[2]);
-        const R sg = (smask[v] >> ax) & 1 ? (R)-1 : (R)1;
-        const R *iv = in + (size_t)v * np * C;
+__device__ __forceinline__ void shift_pass(int ax, int p, int np, const int *sMNK, const short *sIdx, const R *sG,
+                                           int mask, const R *in, R *out) {
+    const int P1 = p + 1, st = ax == 0 ? P1 * P1 : ax == 1 ? P1 : 1;
+    const R sg = (mask >> ax) & 1 ? (R)-1 : (R)1;
+    for (int a = threadIdx.x; a < np; a += MM_T) {
+        const int mnk = sMNK[a], e = mnk >> (8 * ax) & 255, rest = p - (mnk >> 24);
+        const short *id = sIdx + ((mnk & 255) * P1 + (mnk >> 8 & 255)) * P1 + (mnk >> 16 & 255);
+        const R *Ge = sG + e * P1;
         R acc[C];
 #pragma unroll
         for (int c = 0; c < C; c++) acc[c] = (R)0;
         R gs = (R)1;
         const int ng = DOWN ? e : rest;          // M2M: g <= a_ax;  L2L: |a| + g <= p
-        for (int g = 0; g <= ng; g++, gs *= sg) {
-            c3[ax] = DOWN ? e - g : e + g;
-            const int src = sIdx[(c3[0] * P1 + c3[1]) * P1 + c3[2]];
-            cmac<R, C>(acc, gs * sG[e * P1 + g], iv + src * C);
-        }
+#pragma unroll 4
+        for (int g = 0; g <= ng; g++, gs *= sg) cmac<R, C>(acc, gs * Ge[g], in + id[DOWN ? -g * st : g * st] * C);
 #pragma unroll
-        for (int c = 0; c < C; c++) out[((size_t)v * np + a) * C + c] = acc[c];
+        for (int c = 0; c < C; c++) out[(size_t)a * C + c] = acc[c];
     }
 }
 
 // 2^-|a| of the coefficient with packed multi-index mnk
 template <class R>
 __device__ __forceinline__ R deg_scale(int mnk) {
-    const int d = (mnk & 255) + ((mnk >> 8) & 255) + (mnk >> 16);
+    const int d = mnk >> 24;
     if constexpr (sizeof(R) == sizeof(float)) return ldexpf(1.f, -d);
     else return ldexp(1.0, -d);
 }
 
+// block 8 i + j of the grid: child j of the level's i-th box
 template <class R, int C>
-__global__ void __launch_bounds__(MM_T) k_m2m_sep(int off, int cnt, const int *__restrict__ child0,
-                                                  const int *__restrict__ nchild, const int *__restrict__ ix,
-                                                  const int *__restrict__ iy, const int *__restrict__ iz, int p, int np,
-                                                  int nps, int npc, int grp, const int *__restrict__ tm,
-                                                  const int *__restrict__ tn, const int *__restrict__ tk,
-                                                  R *__restrict__ M, const int *__restrict__ skip) {
+__global__ void __launch_bounds__(MM_T) __cluster_dims__(MM_CL, 1, 1)
+    k_m2m_sep(int off, const int *__restrict__ child0, const int *__restrict__ nchild, const int *__restrict__ ix,
+              const int *__restrict__ iy, const int *__restrict__ iz, int p, int np, int nps, int npc, int Pm1,
+              const R *__restrict__ G, const int *__restrict__ mexp, R *__restrict__ M, const int *__restrict__ skip) {
     if (skip && *skip) return;
-    extern __shared__ unsigned char smem_raw[];
-    const int P1 = p + 1;
-    R *sA = (R *)smem_raw;                                  // [grp][np][C]
-    R *sB = sA + (size_t)grp * np * C;                       // [grp][np][C]
-    R *sS = sB + (size_t)grp * np * C;                       // [np][C] sum over children
-    R *sG = sS + (size_t)np * C;                             // [P1][P1]
-    short *sIdx = (short *)(sG + P1 * P1);                   // [P1^3]
-    int *sMNK = (int *)((unsigned char *)sG + (shift_tab_bytes<R>(p, np) - 4 * (size_t)np - 16));   // [np]
-    __shared__ int smask[8];
-    if (blockIdx.x >= cnt) return;
-    const int b = off + blockIdx.x, nch = nchild[b], c0 = child0[b], tid = threadIdx.x;
-    if (nch == 0) return;
-    // children (consecutive boxes, row stride nps) hold npc coefficients; the
-    // rest enter as zero.  U values per thread are loaded before any is
-    // stored, so their latencies overlap (and the first ones the tables')
-    constexpr int U = 6 * C;
-    R v[U];
-    auto load = [&](int g0, int nt, int t0) {
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int t = t0 + u * MM_T;
-            const int j = t / (np * C), r = t - j * np * C, a = r / C;
-            v[u] = t < nt && a < npc ? M[((size_t)(c0 + g0 + j) * nps) * C + r] : (R)0;
-        }
-    };
-    auto store = [&](int nt, int t0) {
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (t0 + u * MM_T < nt) sA[t0 + u * MM_T] = v[u];
-    };
-    load(0, min(grp, nch) * np * C, tid);
-    shift_tables<R>(p, np, tm, tn, tk, true, sIdx, sG, sMNK);
-    for (int g0 = 0; g0 < nch; g0 += grp) {
-        const int ng = min(grp, nch - g0), nt = ng * np * C;
-        __syncthreads();
-        if (g0 > 0) load(g0, nt, tid);
-        store(nt, tid);
-        for (int t0 = tid + U * MM_T; t0 < nt; t0 += U * MM_T) {
-            load(g0, nt, t0);
-            store(nt, t0);
-        }
-        // a child on the low side of an axis has offset -1/4 of the parent edge
-        if (tid < ng) {
-            const int c = c0 + g0 + tid;
-            smask[tid] = ((ix[c] & 1) ? 0 : 1) | ((iy[c] & 1) ? 0 : 2) | ((iz[c] & 1) ? 0 : 4);
-        }
-        __syncthreads();
-        shift_pass<R, C, true>(0, ng, p, np, sMNK, sIdx, sG, smask, sA, sB);
-        __syncthreads();
-        shift_pass<R, C, true>(1, ng, p, np, sMNK, sIdx, sG, smask, sB, sA);
-        __syncthreads();
-        shift_pass<R, C, true>(2, ng, p, np, sMNK, sIdx, sG, smask, sA, sB);
-        __syncthreads();
-        for (int t = tid; t < np * C; t += MM_T) {
-            R sum = g0 == 0 ? (R)0 : sS[t];
-            for (int j = 0; j < ng; j++) sum += sB[(size_t)j * np * C + t];
-            sS[t] = sum;
-        }
-    }
-    __syncthreads();
-    for (int a = tid; a < np; a += MM_T) {
-        const R sc = deg_scale<R>(sMNK[a]);
-#pragma unroll
-        for (int c = 0; c < C; c++) M[((size_t)b * nps + a) * C + c] = sS[(size_t)a * C + c] * sc;
-    }
-}
-
-template <class R, int C>
-__global__ void __launch_bounds__(MM_T) k_l2l_sep(int off, int cnt, const int *__restrict__ parent,
-                                                  const int *__restrict__ ix, const int *__restrict__ iy,
-                                                  const int *__restrict__ iz, int p, int np, int nps, int npo,
-                                                  const int *__restrict__ tm, const int *__restrict__ tn,
-                                                  const int *__restrict__ tk, R *__restrict__ L,
-                                                  const int *__restrict__ skip) {
-    if (skip && *skip) return;
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P1 = p + 1;
     R *sA = (R *)smem_raw;                                  // [np][C]
     R *sB = sA + (size_t)np * C;                             // [np][C]
     R *sG = sB + (size_t)np * C;                             // [P1][P1]
     short *sIdx = (short *)(sG + P1 * P1);                   // [P1^3]
     int *sMNK = (int *)((unsigned char *)sG + (shift_tab_bytes<R>(p, np) - 4 * (size_t)np - 16));   // [np]
-    __shared__ int smask[1];
-    if (blockIdx.x >= cnt) return;
-    const int b = off + blockIdx.x, pa = parent[b], tid = threadIdx.x;
-    // the parent's np coefficients, all of a thread's in flight before the tables
-    constexpr int U = 2 * C;
-    const int nt = np * C;
-    R v[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int t = tid + u * MM_T;
-        v[u] = t < nt ? L[(size_t)pa * nps * C + t] : (R)0;
+    const int b = off + blockIdx.x / MM_CL, j = blockIdx.x % MM_CL, nch = nchild[b], tid = threadIdx.x;
+    if (nch == 0) return;                                    // all blocks of the cluster
+    if (j < nch) {
+        // the child (consecutive boxes, row stride nps) holds npc coefficients; the rest enter as zero
+        const int c = child0[b] + j, nt = npc * C;
+        for (int t = nt + tid; t < np * C; t += MM_T) sA[t] = (R)0;
+        // a child on the low side of an axis has offset -1/4 of the parent edge
+        const int mask = ((ix[c] & 1) ? 0 : 1) | ((iy[c] & 1) ? 0 : 2) | ((iz[c] & 1) ? 0 : 4);
+        shift_load<R, 2 * C>(p, np, Pm1, G, mexp, M + (size_t)c * nps * C, min(nt, np * C), sIdx, sG, sMNK, sA);
+        __syncthreads();
+        shift_pass<R, C, true>(0, p, np, sMNK, sIdx, sG, mask, sA, sB);
+        __syncthreads();
+        shift_pass<R, C, true>(1, p, np, sMNK, sIdx, sG, mask, sB, sA);
+        __syncthreads();
+        shift_pass<R, C, true>(2, p, np, sMNK, sIdx, sG, mask, sA, sB);
     }
-    if (tid == 0) smask[0] = ((ix[b] & 1) ? 0 : 1) | ((iy[b] & 1) ? 0 : 2) | ((iz[b] & 1) ? 0 : 4);
-    shift_tables<R>(p, np, tm, tn, tk, false, sIdx, sG, sMNK);
+    cluster_sync();
+    if (j < nch)                                             // these hold the multi-indices
+        for (int t = j * MM_T + tid; t < np * C; t += nch * MM_T) {
+            R v[MM_CL];
 #pragma unroll
-    for (int u = 0; u < U; u++)
-        if (tid + u * MM_T < nt) sA[tid + u * MM_T] = v[u];
-    for (int t = tid + U * MM_T; t < nt; t += MM_T) sA[t] = L[(size_t)pa * nps * C + t];
-    __syncthreads();
-    shift_pass<R, C, false>(2, 1, p, np, sMNK, sIdx, sG, smask, sA, sB);
-    __syncthreads();
-    shift_pass<R, C, false>(1, 1, p, np, sMNK, sIdx, sG, smask, sB, sA);
-    __syncthreads();
-    shift_pass<R, C, false>(0, 1, p, np, sMNK, sIdx, sG, smask, sA, sB);
-    __syncthreads();
-    for (int a = tid; a < npo; a += MM_T) {         // the child keeps its own order's npo coefficients (npo <= np)
-        const R sc = deg_scale<R>(sMNK[a]);
+            for (int q = 0; q < MM_CL; q++) v[q] = q < nch ? peer_load(sB + t, q) : (R)0;
+            R sum = (R)0;
 #pragma unroll
-        for (int c = 0; c < C; c++) L[((size_t)b * nps + a) * C + c] += sB[(size_t)a * C + c] * sc;
-    }
+            for (int q = 0; q < MM_CL; q++)
+                if (q < nch) sum += v[q];
+            M[(size_t)b * nps * C + t] = sum * deg_scale<R>(sMNK[t / C]);
+        }
+    cluster_sync();                                          // no block leaves while others read its sums
+}
+
+template <class R, int C>
+__global__ void __launch_bounds__(MM_T) k_l2l_sep(int off, const int *__restrict__ parent, const int *__restrict__ ix,
+                                                  const int *__restrict__ iy, const int *__restrict__ iz, int p, int np,
+                                                  int nps, int npo, int Pm1, const R *__restrict__ G,
+                                                  const int *__restrict__ mexp, R *__restrict__ L,
+                                                  const int *__restrict__ skip) {
+    if (skip && *skip) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int P1 = p + 1;
+    R *sA = (R *)smem_raw;                                  // [np][C]
+    R *sB = sA + (size_t)np * C;                             // [np][C]
+    R *sG = sB + (size_t)np * C;                             // [P1][P1]
+    short *sIdx = (short *)(sG + P1 * P1);                   // [P1^3]
+    int *sMNK = (int *)((unsigned char *)sG + (shift_tab_bytes<R>(p, np) - 4 * (size_t)np - 16));   // [np]
+    const int b = off + blockIdx.x, tid = threadIdx.x;
+    const int mask = ((ix[b] & 1) ? 0 : 1) | ((iy[b] & 1) ? 0 : 2) | ((iz[b] & 1) ? 0 : 4);
+    shift_load<R, 2 * C>(p, np, Pm1, G, mexp, L + (size_t)parent[b] * nps * C, np * C, sIdx, sG, sMNK, sA);
+    __syncthreads();
+    shift_pass<R, C, false>(2, p, np, sMNK, sIdx, sG, mask, sA, sB);
+    __syncthreads();
+    shift_pass<R, C, false>(1, p, np, sMNK, sIdx, sG, mask, sB, sA);
+    __syncthreads();
+    shift_pass<R, C, false>(0, p, np, sMNK, sIdx, sG, mask, sA, sB);
+    __syncthreads();
+    for (int t = tid; t < npo * C; t += MM_T)        // the child keeps its own order's npo coefficients (npo <= np)
+        L[(size_t)b * nps * C + t] += sB[t] * deg_scale<R>(sMNK[t / C]);
 }
 
 // ---------------------------------------------------------------------------
@@ -480,9 +441,31 @@ int launch_m2l_derivs(bem_plan *P, int ncls, const double *rho, const double *kh
 }
 
 // M2L tables for the current order (called by alloc_fmm).
-int build_translation_tables(bem_plan *P, cudaStream_t s) { return build_sym_tables(P, s); }
+int build_translation_tables(bem_plan *P, cudaStream_t s) {
+    // per-axis shift factors [M2M, L2L][a][g], in the plan's precision
+    const int n = P->mi.p + 1;
+    std::vector<double> b((size_t)(2 * n) * (2 * n), 0.0), G(2 * (size_t)n * n, 0.0);   // binomials, exact
+    for (int i = 0; i < 2 * n; i++)
+        for (int j = 0; j <= i; j++) b[i * 2 * n + j] = j == 0 || j == i ? 1.0 : b[(i - 1) * 2 * n + j - 1] + b[(i - 1) * 2 * n + j];
+    for (int a = 0; a < n; a++)
+        for (int g = 0; g < n; g++) {
+            if (g <= a) G[a * n + g] = std::ldexp(b[a * 2 * n + g], -g);
+            G[n * n + a * n + g] = std::ldexp(b[(a + g) * 2 * n + a], -2 * g);
+        }
+    const bool mx = P->prm.precision == BEM_MIXED;
+    const std::vector<float> Gf(G.begin(), G.end());
+    const size_t bytes = (mx ? sizeof(float) : sizeof(double)) * G.size();
+    BEM_TRY(P->arena.alloc((char **)&P->shift_G, bytes));
+    // (pageable source: staged before the call returns)
+    BEM_CUDA(cudaMemcpyAsync(P->shift_G, mx ? (const void *)Gf.data() : (const void *)G.data(), bytes, cudaMemcpyHostToDevice, s));
+    return build_sym_tables(P, s);
+}
 
-void free_translation_tables(bem_plan *P) { free_sym_tables(P); }
+void free_translation_tables(bem_plan *P) {
+    P->arena.release(P->shift_G);
+    P->shift_G = nullptr;
+    free_sym_tables(P);
+}
 
 // ---------------------------------------------------------------------------
 // host: launchers
@@ -502,12 +485,9 @@ int launch_m2m(bem_plan *P, R *M, cudaStream_t s, int lmin) {
     for (int l = t.nlev - 2; l >= std::max(0, lmin); l--) {
         const int off = t.lev_off[l], cnt = t.lev_off[l + 1] - off;
         const int p = level_order(P, l), np = np_host(p), npc = np_host(level_order(P, l + 1));
-        const size_t tab_sm = shift_tab_bytes<R>(p, np);
-        int grp = 8;                             // children shifted together (shared memory permitting)
-        while (grp > 1 && sizeof(R) * (2 * grp + 1) * np * C + tab_sm > 220 * 1024) grp /= 2;
-        const size_t m2m_sm = sizeof(R) * (2 * grp + 1) * np * C + tab_sm;
-        (k_m2m_sep<R, C><<<cnt, MM_T, m2m_sm, s>>>(off, cnt, t.child0, t.nchild, t.ix, t.iy, t.iz, p, np, nps, npc, grp,
-                                                   P->d_m, P->d_n, P->d_k, M, sk),
+        const size_t sm = sizeof(R) * 2 * np * C + shift_tab_bytes<R>(p, np);
+        (k_m2m_sep<R, C><<<cnt * MM_CL, MM_T, sm, s>>>(off, t.child0, t.nchild, t.ix, t.iy, t.iz, p, np, nps, npc,
+                                                       P->mi.p + 1, (const R *)P->shift_G, P->sy_mexp, M, sk),
          ::bem::count_launch());
     }
     BEM_LAUNCH_CHECK();
@@ -538,9 +518,10 @@ int launch_translations(bem_plan *P, R *M, R *L, cudaStream_t s, cudaEvent_t *ev
         const int off = t.lev_off[l], cnt = t.lev_off[l + 1] - off;
         const int p = level_order(P, l - 1), pnp = np_host(p), npo = np_host(level_order(P, l));
         const size_t tab_sm = shift_tab_bytes<R>(p, pnp);
-        (k_l2l_sep<R, C><<<cnt, MM_T, sizeof(R) * 2 * pnp * C + tab_sm, s>>>(off, cnt, t.parent, t.ix, t.iy, t.iz, p,
-                                                                           pnp, np, npo, P->d_m, P->d_n, P->d_k, L,
-                                                                           sk),
+        const int n = P->mi.p + 1;
+        (k_l2l_sep<R, C><<<cnt, MM_T, sizeof(R) * 2 * pnp * C + tab_sm, s>>>(off, t.parent, t.ix, t.iy, t.iz, p, pnp, np, npo,
+                                                                           n, (const R *)P->shift_G + n * n, P->sy_mexp,
+                                                                           L, sk),
          ::bem::count_launch());
     }
     BEM_LAUNCH_CHECK();
