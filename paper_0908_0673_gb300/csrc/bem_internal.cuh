@@ -391,6 +391,7 @@ struct bem_plan : bem::FmmState {
     int2 *near_items[2] = {nullptr, nullptr};   // near-field work items (real, complex)
     int near_nitems[2] = {0, 0};
     int *leaf_near_ptr = nullptr, *leaf_near_idx = nullptr;   // leaf_descend = 0: near lists opened down to leaves
+    const float *wave = nullptr;                // unit-circle table of the float32 Helmholtz near field (the library's)
     const float4 *circle = nullptr;             // unit-circle table of the float64 Helmholtz near field (the library's)
     int last_op = -1;
     // field evaluation workspaces (field.cu): strengths of phi and chi, monomial

@@ -19,6 +19,10 @@ __device__ __forceinline__ P2 padd(P2 a, P2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ P2 pmul(P2 a, P2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ P2 pfma(P2 a, P2 b, P2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ P2 psub(P2 a, P2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// the sign flipped by integer operations, off the float32 pipe
+__device__ __forceinline__ P2 pxneg(P2 a) {
+    return make_float2(__int_as_float(__float_as_int(a.x) ^ 0x80000000), __int_as_float(__float_as_int(a.y) ^ 0x80000000));
+}
 __device__ __forceinline__ P2 pneg(P2 a) { return make_float2(-a.x, -a.y); }
 
 // s + e = a + b exactly

@@ -23,6 +23,8 @@
 #include <cmath>
 #include <mutex>
 
+#include "cluster.cuh"
+#include "dfloat.cuh"
 #include "fmm_views.cuh"
 
 namespace bem {
@@ -342,28 +344,42 @@ __global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, 
 
 
 // ---------------------------------------------------------------------------
-// near field + L2P, float32 form.  A block takes one leaf and up to SLOTS of
+// near field + L2P, float32 form.  A block takes one leaf and up to 64 of
 // its targets per pass: G = ceil(targets / U) target groups x (256 / G)
 // source slices, each thread holding U targets (8 real, 4 complex) so that
 // every source read from shared memory serves U pairs.  The near-list
 // sources are packed into full tiles across box boundaries; each staged
 // source is rebased to the target leaf's centre (box offset in float64,
-// rounded once).  For the real double layer the strength is folded into the
-// staged normal, so a pair costs 3 subtractions, two 3-term dot products, one
-// reciprocal square root and three multiplies.  Tile partial sums are added
-// with compensation, slices and the local expansion combine in float64.
+// rounded once).  Pairs run two targets to a packed instruction.  For the real
+// double layer the strength is folded into the staged normal, so a pair costs 3
+// subtractions, two 3-term dot products, one reciprocal square root and three
+// multiplies.  Complex pairs (33 packed operations) take e^{jkr} from a table of
+// the unit circle and the first two terms of the rest (sincosf cost more than
+// the rest of the pair: sphere of 20,480 tri6 738 -> 573 us, of 81,920 3142 ->
+// 2290, FMA pipe 65 % busy).  Tile partial sums are added with compensation,
+// slices as float32 pairs, the local expansion in float64.
 // ---------------------------------------------------------------------------
-constexpr int NF2_T = 256, NF2_TILE = 1024, NF2_ENT = 256;
+constexpr int NF2_T = 256, NF2_ENT = 256, NF2_SLOTS = 64, NF2_MAXC = 8;
 __host__ __device__ constexpr int nf2_u(int C) { return C == 1 ? 8 : 4; }
-// sources per staged round: 3 float4 each in the packed real form, 2 complex
-// (1024 real sources per round, three blocks per SM: 0.437 ms against 0.456 for
-// 640 at four blocks on the cube workload, the rounds' barriers and staging
-// halved)
-__host__ __device__ constexpr int nf2_tile(int C) { return C == 1 ? 1024 : NF2_TILE; }
-// float4 slots of the staged-source region
-__host__ __device__ constexpr int nf2_stage(int C) { return C == 1 ? 3 * nf2_tile(1) : 2 * NF2_TILE; }
+// Complex pairs take e^{jkr} from a table of the unit circle (TAB): 1,024 steps
+// leave an angle below 3.1e-3, whose sine is itself to 2^-27.  k r in table steps
+// must stay below 2^22, where adding 1.5 2^23 still rounds to the index; plans
+// beyond it (k x side above 1,600) take sincosf.
+constexpr int NF2_TAB = 1024;
+constexpr double NF2_MAXPHASE = 4194304.0;
+// A cluster of up to NF2_MAXC blocks shares an item's sources and expansion terms
+// where items would not fill two waves of three blocks per SM (59 -> 34 us for 72
+// leaves, 121 -> 76 for 56 complex ones); the kernel without the cluster's code
+// is the faster one where they do (429 against 444 us for 1,180 items).
+constexpr int NF2_WAVES = 2;
+// sources staged per round, and float4 of each: packed forms hold every value
+// twice, for the two targets of a float2 operation.  Real: 1024 per round, three
+// blocks per SM (0.437 ms against 0.456 for 640 at four blocks on the cube
+// workload, the rounds' barriers and staging halved).
+__host__ __device__ constexpr int nf2_tile(int C, bool TAB) { return C == 2 && TAB ? 640 : 1024; }
+__host__ __device__ constexpr int nf2_stage(int C, bool TAB) { return nf2_tile(C, TAB) * (C == 1 ? 3 : TAB ? 4 : 2); }
 
-// Work items of the near field: one per (leaf, pass of up to 8 U targets, or
+// Work items of the near field: one per (leaf, pass of up to NF2_SLOTS targets,
 // ND_SLOTS in float64 plans), ordered by decreasing pair count (targets x near sources, ties in
 // leaf order), so the largest blocks start first and the last wave is made of
 // the smallest.  Each target is summed by one block whatever the order.
@@ -417,7 +433,7 @@ int build_near_items(bem_plan *P) {
     // real items for every plan (the diagonal's product is Laplace), complex
     // ones for Helmholtz plans only
     for (int v = 0; v < (P->green == BEM_HELMHOLTZ ? 2 : 1); v++) {
-        const int slots = P->prm.precision == BEM_MIXED ? 8 * nf2_u(v + 1) : ND_SLOTS;
+        const int slots = P->prm.precision == BEM_MIXED ? NF2_SLOTS : ND_SLOTS;
         std::vector<int2> items;
         std::vector<int64_t> cost;
         for (int li = 0; li < t.nleaf; li++) {
@@ -491,31 +507,32 @@ struct KahanF {
 
 // shared memory of the float32 near field beyond its static part: the staged
 // sources (sa, sb) and the per-thread compensated sums
-__host__ __device__ constexpr size_t nf2_dyn_bytes(int C) {
-    return (size_t)nf2_stage(C) * sizeof(float4) + 2 * (size_t)nf2_u(C) * C * NF2_T * sizeof(float);
+__host__ __device__ constexpr size_t nf2_dyn_bytes(int C, bool TAB) {
+    return (size_t)nf2_stage(C, TAB) * sizeof(float4) + 2 * (size_t)nf2_u(C) * C * NF2_T * sizeof(float) +
+           (C == 2 && TAB ? NF2_TAB * sizeof(float2) : 0);
 }
 
-template <int C, bool DL>
-__global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__restrict__ items, Tabs tb, TreeView tv,
-                                                       QuadView qv, double kwave, const float *__restrict__ f,
-                                                       const float *__restrict__ L, double *__restrict__ ytmp,
-                                                       const int *__restrict__ skip) {
+template <int C, bool DL, bool TAB, bool CL>
+__global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
+    k_near_f32(int ns_, const int2 *__restrict__ items, Tabs tb, TreeView tv, QuadView qv, double kwave,
+               const float *__restrict__ f, const float *__restrict__ L, double *__restrict__ ytmp,
+               const float *__restrict__ wave, const int *__restrict__ skip) {
     constexpr int U = nf2_u(C);                       // targets per thread
-    constexpr int SLOTS = 8 * U;                      // targets per pass (at most 8 groups)
+    constexpr int SLOTS = NF2_SLOTS;                  // targets per pass (at most SLOTS / U groups)
     constexpr int LP = NF2_T / SLOTS;                 // threads per target in the local expansion
     constexpr int UC = U * C;
-    constexpr int TILE = nf2_tile(C);                 // sources staged per round
-    if (skip && *skip) return;
-    if ((int)blockIdx.x >= nitem) return;
-    const int2 item = items[blockIdx.x];              // (leaf, first target of the pass)
+    constexpr int TILE = nf2_tile(C, TAB);            // sources staged per round
+    if (skip && *skip) return;                        // every block of the cluster reads the same word
+    const int ns = CL ? ns_ : 1, rank = CL ? (int)cluster_rank() : 0;
+    const int2 item = items[blockIdx.x / ns];         // (leaf, first target of the pass)
     const int b = tv.leaves[item.x];
     const int tid = threadIdx.x, lane = tid & 31;
     // The staged-source region is reused once the sources are done: slice
     // sums, local-expansion partials and the targets' powers (23 KB at most).
     extern __shared__ float4 near_tile[];
-    float4 *sa = near_tile, *sb = near_tile + NF2_TILE;                 // C = 2: position | Re f, normal | Im f
-    float4 *s0 = near_tile, *s1 = s0 + TILE, *s2 = s1 + TILE;           // C = 1: packed (see the staging)
-    float *ks = (float *)(near_tile + nf2_stage(C));  // [UC][NF2_T] compensated sums
+    float4 *sa = near_tile, *sb = near_tile + TILE;                     // sincosf form: position | Re f, normal | Im f
+    float4 *s0 = near_tile, *s1 = s0 + TILE, *s2 = s1 + TILE, *s3 = s2 + TILE;   // packed forms (see the staging)
+    float *ks = (float *)(near_tile + nf2_stage(C, TAB));   // [UC][NF2_T] compensated sums
     float *kc = ks + UC * NF2_T;                      // [UC][NF2_T] their carries
     float *red = (float *)near_tile;                  // [slice][slot][C]
     float *lred = red + NF2_T * UC;                   // [part][slot][C]
@@ -524,8 +541,14 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
     __shared__ int ebase[NF2_ENT];                    // first quadrature point of each entry's box
     __shared__ float eoff[NF2_ENT][3];                // entry box centre - target leaf centre
     __shared__ float toff[SLOTS][3];                  // target - target leaf centre
+    __shared__ double share[SLOTS][C];                // this block's sums, for the cluster's first
     const double cbx = tv.cx[b], cby = tv.cy[b], cbz = tv.cz[b];
     const float kw = (float)kwave;
+    float *sw = kc + UC * NF2_T;                      // the unit circle: cosines, then sines
+    const double ktd = kwave * (NF2_TAB / (2.0 * M_PI));
+    const float kt = (float)ktd, ktl = (float)(ktd - (double)kt);   // k in table steps per length
+    if (C == 2 && TAB)
+        for (int i = tid; i < 2 * NF2_TAB; i += NF2_T) sw[i] = wave[i];
     const int np = tb.np, p = order_of(tb, tv.level[b]), npl = np_of(p);   // the leaf's order; np the stride
     const int t0 = item.y, nt = min(SLOTS, tv.ne[b] - t0);
     const int G = (nt + U - 1) / U, S = NF2_T / G, tg = tid % G, sl = tid / G;
@@ -574,11 +597,12 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
             if (lane == 0) pref[0] = 0;
         }
         __syncthreads();
-        const int total = pref[ne_];
-        for (int base = 0; base < total; base += TILE) {
+        // this block's share of the chunk's sources
+        const int j0 = (int)((long long)pref[ne_] * rank / ns), j1 = (int)((long long)pref[ne_] * (rank + 1) / ns);
+        for (int base = j0; base < j1; base += TILE) {
             __syncthreads();
             int lo = 0;                               // entry holding j: pref[lo] <= j < pref[lo + 1]
-            if (base + tid < total) {
+            if (base + tid < j1) {
                 int hi = ne_ - 1;
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
@@ -587,7 +611,7 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
             }
             for (int jj = tid; jj < TILE; jj += NF2_T) {
                 const int j = base + jj;
-                if (j >= total) break;
+                if (j >= j1) break;
                 while (pref[lo + 1] <= j) lo++;       // j grows with jj: the entry only moves forward
                 const int o = ebase[lo] + (j - pref[lo]);
                 const float4 xa = make_float4(eoff[lo][0] + qv.fx[o], eoff[lo][1] + qv.fy[o], eoff[lo][2] + qv.fz[o], 0.f);
@@ -603,6 +627,17 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
                     } else {
                         s1[jj] = make_float4(-xa.z, -xa.z, fo, fo);
                     }
+                } else if constexpr (TAB) {
+                    const float fr = f[(size_t)o * C], fi = f[(size_t)o * C + 1];
+                    s0[jj] = make_float4(-xa.x, -xa.x, -xa.y, -xa.y);
+                    s1[jj] = make_float4(-xa.z, -xa.z, fr, fr);
+                    if (DL) {
+                        const float nx = qv.fnx[o], ny = qv.fny[o], nz = qv.fnz[o];
+                        s2[jj] = make_float4(fi, fi, nx, nx);
+                        s3[jj] = make_float4(ny, ny, nz, nz);
+                    } else {
+                        s2[jj] = make_float4(fi, fi, 0.f, 0.f);
+                    }
                 } else {
                     sa[jj] = make_float4(xa.x, xa.y, xa.z, f[(size_t)o * C]);
                     sb[jj] = make_float4(DL ? qv.fnx[o] : 0.f, DL ? qv.fny[o] : 0.f, DL ? qv.fnz[o] : 0.f,
@@ -610,7 +645,7 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
                 }
             }
             __syncthreads();
-            const int nq = min(TILE, total - base);
+            const int nq = min(TILE, j1 - base);
             float part[U][C];
 #pragma unroll
             for (int u = 0; u < U; u++)
@@ -666,6 +701,67 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
                 for (int v = 0; v < U / 2; v++) {
                     part[2 * v][0] = p2[v].x;
                     part[2 * v + 1][0] = p2[v].y;
+                }
+            } else if constexpr (TAB) {
+                // packed as the real form; e^{jkr} = table entry times the small rest
+                float2 t2x[U / 2], t2y[U / 2], t2z[U / 2], pr[U / 2], pi[U / 2];
+#pragma unroll
+                for (int v = 0; v < U / 2; v++) {
+                    t2x[v] = make_float2(tx[2 * v], tx[2 * v + 1]);
+                    t2y[v] = make_float2(ty[2 * v], ty[2 * v + 1]);
+                    t2z[v] = make_float2(tz[2 * v], tz[2 * v + 1]);
+                    pr[v] = pi[v] = make_float2(0.f, 0.f);
+                }
+                if (worker)
+                    for (int q = sl; q < nq; q += S) {
+                        const float4 a0 = s0[q], a1 = s1[q], a2 = s2[q];
+                        const float2 mx = make_float2(a0.x, a0.y), my = make_float2(a0.z, a0.w), mz = make_float2(a1.x, a1.y),
+                                     fr = make_float2(a1.z, a1.w), fi = make_float2(a2.x, a2.y);
+                        float2 nx, ny, nz;
+                        if (DL) {
+                            const float4 a3 = s3[q];
+                            nx = make_float2(a2.z, a2.w);
+                            ny = make_float2(a3.x, a3.y);
+                            nz = make_float2(a3.z, a3.w);
+                        }
+#pragma unroll
+                        for (int v = 0; v < U / 2; v++) {
+                            const float2 rx = padd(t2x[v], mx), ry = padd(t2y[v], my), rz = padd(t2z[v], mz);
+                            const float2 r2 = pfma(rx, rx, pfma(ry, ry, pmul(rz, rz)));
+                            const float2 inv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)), R1 = pmul(r2, inv);
+                            // k r = j + d table steps, both exact products: adding 1.5 2^23 rounds to j
+                            const float2 jf = pfma(p2(kt), R1, p2(12582912.f)), nj = psub(p2(12582912.f), jf);
+                            const float2 d = pfma(p2(ktl), R1, pfma(p2(kt), R1, nj));
+                            const int i0 = __float_as_int(jf.x) & (NF2_TAB - 1), i1 = __float_as_int(jf.y) & (NF2_TAB - 1);
+                            const float2 Cs = make_float2(sw[i0], sw[i1]), Sn = make_float2(sw[NF2_TAB + i0], sw[NF2_TAB + i1]);
+                            // e^{jg} = (1 - g^2 / 2) + j g to 2^-27, g = d 2 pi / 1024
+                            constexpr float st = (float)(2.0 * M_PI / NF2_TAB);
+                            const float2 g = pmul(d, p2(st)), q1 = pfma(pmul(d, d), p2(-0.5f * st * st), p2(1.f));
+                            const float2 cs = pfma(Cs, q1, pmul(Sn, pxneg(g))), sn = pfma(Sn, q1, pmul(Cs, g));
+                            // H = (1 - j k r) (r . n) / r^3 f, or f / r; then times cs + j sn
+                            float2 hr, hi;
+                            if (DL) {
+                                const float2 dot = pfma(rx, nx, pfma(ry, ny, pmul(rz, nz)));
+                                const float2 w = pmul(pmul(dot, inv), pmul(inv, inv));
+                                const float2 gr = pmul(fr, w), gi = pmul(fi, w), kr = pmul(p2(kw), R1);
+                                hr = pfma(kr, gi, gr);
+                                hi = pfma(kr, pxneg(gr), gi);
+                            } else {
+                                hr = pmul(fr, inv);
+                                hi = pmul(fi, inv);
+                            }
+                            pr[v] = pfma(cs, hr, pr[v]);
+                            pi[v] = pfma(cs, hi, pi[v]);
+                            pr[v] = pfma(pxneg(sn), hi, pr[v]);
+                            pi[v] = pfma(sn, hr, pi[v]);
+                        }
+                    }
+#pragma unroll
+                for (int v = 0; v < U / 2; v++) {
+                    part[2 * v][0] = pr[v].x;
+                    part[2 * v + 1][0] = pr[v].y;
+                    part[2 * v][C - 1] = pi[v].x;
+                    part[2 * v + 1][C - 1] = pi[v].y;
                 }
             } else if (worker) {
                 // two sources per iteration (fewer loop instructions, more independent work)
@@ -728,7 +824,7 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
         KahanF loc[C];
         if (slot < nt) {
             const float *sp = spow + (size_t)slot * 3 * (PMAX + 1);
-            for (int a = part_id; a < npl; a += LP) {
+            for (int a = rank * LP + part_id; a < npl; a += ns * LP) {
                 const float mono = sp[tb.m[a]] * sp[PMAX + 1 + tb.n[a]] * sp[2 * (PMAX + 1) + tb.k[a]];
 #pragma unroll
                 for (int c = 0; c < C; c++) loc[c].add(mono * L[((size_t)b * np + a) * C + c]);
@@ -738,19 +834,37 @@ __global__ void __launch_bounds__(NF2_T, 4) k_near_f32(int nitem, const int2 *__
         for (int c = 0; c < C; c++) lred[(part_id * SLOTS + slot) * C + c] = loc[c].s;
     }
     __syncthreads();
-    if (tid < nt) {
-        // target t0 + tid sits in slot tid = tg + G u of every slice
-        KahanF sum[C], loc[C];
-        for (int q = 0; q < S; q++)
+    {
+        // four threads per target add every fourth slice (target t0 + slot sits in
+        // place slot = tg + G u of each), then each other's sums
+        static_assert(NF2_T == 4 * SLOTS && LP == 4, "four threads per target");
+        const int slot = tid >> 2, q0 = tid & 3;
 #pragma unroll
-            for (int c = 0; c < C; c++) sum[c].add(red[((size_t)q * G * U + tid) * C + c]);
-        for (int q = 0; q < LP; q++)
+        for (int c = 0; c < C; c++) {
+            KahanF k;
+            if (slot < nt)
+                for (int q = q0; q < S; q += 4) k.add(red[((size_t)q * G * U + slot) * C + c]);
+            // float32 pairs (few float64 operations: 1 / 64 of the rate)
+            float h = k.s, l = -k.c, lh = lred[(q0 * SLOTS + slot) * C + c], ll = 0.f;
 #pragma unroll
-            for (int c = 0; c < C; c++) loc[c].add(lred[(q * SLOTS + tid) * C + c]);
+            for (int o = 1; o < 4; o <<= 1) {
+                df_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+                df_add(lh, ll, __shfl_xor_sync(0xffffffffu, lh, o), __shfl_xor_sync(0xffffffffu, ll, o));
+            }
+            if (q0 == 0) share[slot][c] = ((double)h + (double)l) * (0.25 / M_PI) + ((double)lh + (double)ll);
+        }
+    }
+    if (CL) cluster_sync(); else __syncthreads();
+    if (rank == 0 && tid < nt) {
         const int node = tv.node_perm[t0 + tid];
 #pragma unroll
-        for (int c = 0; c < C; c++) ytmp[(size_t)node * C + c] = (double)sum[c].s * (0.25 / M_PI) + (double)loc[c].s;
+        for (int c = 0; c < C; c++) {
+            double y = share[tid][c];
+            for (int q = 1; q < ns; q++) y += peer_double(&share[tid][c], q);
+            ytmp[(size_t)node * C + c] = y;
+        }
     }
+    if (CL) cluster_sync();                           // no block leaves while block 0 reads its share
 }
 
 // ---------------------------------------------------------------------------
@@ -959,14 +1073,45 @@ static int init_shape_table(int device) {
     return BEM_OK;
 }
 
+// The unit circle at 2 pi j / 1024 for the float32 Helmholtz near field, filled
+// once per device (under a lock, as the shape table).
+__device__ float g_wave[2 * NF2_TAB];
+static int wave_table(int device, const float **out) {
+    static std::mutex mu;
+    static const float *addr[64] = {};
+    std::lock_guard<std::mutex> lock(mu);
+    if (device < 0 || device >= 64) { set_error("device %d out of range", device); return BEM_EINVAL; }
+    if (!addr[device]) {
+        std::vector<float> t(2 * NF2_TAB);
+        for (int j = 0; j < NF2_TAB; j++) {
+            t[j] = (float)std::cos(2.0 * M_PI * j / NF2_TAB);
+            t[NF2_TAB + j] = (float)std::sin(2.0 * M_PI * j / NF2_TAB);
+        }
+        void *p = nullptr;
+        BEM_CUDA(cudaGetSymbolAddress(&p, g_wave));
+        BEM_CUDA(cudaMemcpy(p, t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice));
+        addr[device] = (const float *)p;
+    }
+    *out = addr[device];
+    return BEM_OK;
+}
+
 // the float32 near-field kernels stage their source tile in dynamic shared
 // memory above the 48 KB default (set outside any graph capture)
 static void set_near_attributes() {
     const int big = 100 * 1024;
-    cudaFuncSetAttribute(k_near_f32<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_near_f32<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_near_f32<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_near_f32<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<1, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<1, true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<1, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<1, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_near_f32<2, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 int alloc_fmm(bem_plan *P, cudaStream_t s) {
@@ -1025,6 +1170,7 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
     }
     set_translation_attributes();
     set_near_attributes();
+    if (mx && P->green == BEM_HELMHOLTZ) BEM_TRY(wave_table(P->device, &P->wave));
     if (!mx) {
         BEM_TRY(near_pairs_prepare(P));
         BEM_TRY(p2m_pairs_prepare());
@@ -1062,12 +1208,27 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     if (ev) BEM_CUDA(cudaEventRecord(ev[2], s));
     BEM_TRY((launch_translations<R, C>(P, M, L, s, ev)));
     if constexpr (sizeof(R) == sizeof(float)) {
-        constexpr size_t tile_sm = nf2_dyn_bytes(C);
         const int ni = P->near_nitems[C - 1];
         const int2 *it = P->near_items[C - 1];
+        // blocks per item
+        int ns = 1;
+        while (ns < NF2_MAXC && ni * ns < NF2_WAVES * 3 * P->sm_count) ns *= 2;
+        auto near = [&](auto shared, auto alone, size_t sm) {
+            return launch_cluster(ns > 1 ? shared : alone, (unsigned)(ni * ns), NF2_T, sm, ns, s, ns, it, tb, tv, qv, kwave,
+                                  (const float *)f, (const float *)L, ytmp, P->wave, sk);
+        };
+#define BEM_NEAR(C_, DL_, TAB_) \
+    BEM_TRY(near(k_near_f32<C_, DL_, TAB_, true>, k_near_f32<C_, DL_, TAB_, false>, nf2_dyn_bytes(C_, TAB_)))
         if (ni > 0) {
-            if (op == BEM_OP_A) (k_near_f32<C, true><<<ni, NF2_T, tile_sm, s>>>(ni, it, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
-            else (k_near_f32<C, false><<<ni, NF2_T, tile_sm, s>>>(ni, it, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
+            // (two points of one near field are at most some 4 sides apart; see near_pairs_apply)
+            if (C == 2 && kwave * t.side * 8.0 * (NF2_TAB / (2.0 * M_PI)) >= NF2_MAXPHASE) {
+                if (op == BEM_OP_A) BEM_NEAR(2, true, false);
+                else BEM_NEAR(2, false, false);
+            } else {
+                if (op == BEM_OP_A) BEM_NEAR(C, true, true);
+                else BEM_NEAR(C, false, true);
+            }
+#undef BEM_NEAR
         }
     } else {
         if (near_pairs_apply(P, C, kwave)) {
