@@ -59,12 +59,20 @@ int set_slots(bem_plan *P, const void *x, void *y, cudaStream_t s) {
 int enqueue_matvec(bem_plan *P, int op, int green, double k, cudaStream_t s) {
     cudaGraphExec_t &ge = P->graph[op];
     if (!ge) {
-        if (!P->capture_stream) BEM_CUDA(cudaStreamCreateWithFlags(&P->capture_stream, cudaStreamNonBlocking));
+        if (!P->fork_ev[1]) {
+            // the expansions' chain of short kernels before the near field's long one
+            int least = 0, greatest = 0;
+            BEM_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+            if (!P->capture_stream) BEM_CUDA(cudaStreamCreateWithPriority(&P->capture_stream, cudaStreamNonBlocking, greatest));
+            if (!P->fork_stream) BEM_CUDA(cudaStreamCreateWithPriority(&P->fork_stream, cudaStreamNonBlocking, least));
+            for (auto &e : P->fork_ev)
+                if (!e) BEM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        }
         cudaGraph_t g = nullptr;
         BEM_CUDA(cudaStreamBeginCapture(P->capture_stream, cudaStreamCaptureModeThreadLocal));
         P->graph_kernels[op] = 0;
         tl_capture_count = &P->graph_kernels[op];
-        int rc = enqueue_matvec_raw(P, op, green, k, 1, P->capture_stream);
+        int rc = enqueue_matvec_raw(P, op, green, k, 1, P->capture_stream, nullptr, nullptr, P->fork_stream);
         tl_capture_count = nullptr;
         cudaError_t e = cudaStreamEndCapture(P->capture_stream, &g);
         const bool invalidated = e == cudaErrorStreamCaptureInvalidated ||
@@ -233,6 +241,9 @@ bem_plan::~bem_plan() {
     if (cycle_graph) cudaGraphExecDestroy(cycle_graph);
     if (hostbuf) cudaFreeHost(hostbuf);
     if (capture_stream) cudaStreamDestroy(capture_stream);
+    if (fork_stream) cudaStreamDestroy(fork_stream);
+    for (auto e : fork_ev)
+        if (e) cudaEventDestroy(e);
     for (auto st : setup_stream)
         if (st) cudaStreamDestroy(st);
 }

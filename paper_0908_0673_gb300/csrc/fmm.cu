@@ -241,8 +241,7 @@ static void launch_p2m_stored(int nleaf, int np, const TreeView &tv, const float
 }
 
 // ---------------------------------------------------------------------------
-// near field (regular rule over the near-list boxes) fused with L2P, float64
-// arithmetic: Helmholtz plans whose phases exceed the table of the float32-pair
+// near field (regular rule over the near-list boxes), float64 arithmetic: Helmholtz plans whose phases exceed the table of the float32-pair
 // kernel (near_f64.cu), which takes every other float64 product
 // ---------------------------------------------------------------------------
 constexpr int NF_T = 256, NF_TGT = 64, NF_SL = NF_T / NF_TGT, NF_TILE = 256;
@@ -266,21 +265,19 @@ __device__ __forceinline__ void pair_f64(double rx, double ry, double rz, double
 }
 
 template <bool DL>
-__global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, QuadView qv, double kw,
-                                               const double *__restrict__ f, const double *__restrict__ L,
-                                               double *__restrict__ ytmp, const int *__restrict__ skip) {
+__global__ void __launch_bounds__(NF_T) k_near(int nleaf, TreeView tv, QuadView qv, double kw,
+                                               const double *__restrict__ f, double *__restrict__ ytmp,
+                                               const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int C = 2;
     const int li = blockIdx.x;
     if (li >= nleaf) return;
     const int b = tv.leaves[li];
     const int tid = threadIdx.x, tt = tid % NF_TGT, sl = tid / NF_TGT;
-    const int np = tb.np, p = order_of(tb, tv.level[b]), npl = np_of(p);   // the leaf's order; np the stride
     __shared__ double sx[NF_TILE], sy[NF_TILE], sz[NF_TILE], snx[NF_TILE], sny[NF_TILE], snz[NF_TILE];
     __shared__ double sf[NF_TILE][C];
     __shared__ double red[NF_T][C];
     const double cbx = tv.cx[b], cby = tv.cy[b], cbz = tv.cz[b];
-    const double h = scalbn(tv.side, -tv.level[b]);
     for (int t0 = tv.nb[b]; t0 < tv.ne[b]; t0 += NF_TGT) {
         const int tk = t0 + tt;
         const bool active = tk < tv.ne[b];
@@ -309,26 +306,9 @@ __global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, 
             acc[0] += part[0];
             acc[1] += part[1];
         }
-        // local expansion at the target: sum_b Ls_b ((x - c)/h)^b, slices split b
-        double loc[C] = {0.0, 0.0};
-        if (active) {
-            const double dx = (tx - cbx) / h, dy = (ty - cby) / h, dz = (tz - cbz) / h;
-            double px[PMAX + 1], py[PMAX + 1], pz[PMAX + 1];
-            px[0] = py[0] = pz[0] = 1.0;
-            for (int e = 1; e <= p; e++) {
-                px[e] = px[e - 1] * dx;
-                py[e] = py[e - 1] * dy;
-                pz[e] = pz[e - 1] * dz;
-            }
-            for (int a = sl; a < npl; a += NF_SL) {
-                const double mono = px[tb.m[a]] * py[tb.n[a]] * pz[tb.k[a]];
-#pragma unroll
-                for (int c = 0; c < C; c++) loc[c] += mono * L[((size_t)b * np + a) * C + c];
-            }
-        }
         __syncthreads();
 #pragma unroll
-        for (int c = 0; c < C; c++) red[tid][c] = acc[c] * (0.25 / M_PI) + loc[c];
+        for (int c = 0; c < C; c++) red[tid][c] = acc[c] * (0.25 / M_PI);
         __syncthreads();
         if (sl == 0 && active) {
             double s[C] = {red[tid][0], red[tid][1]};
@@ -344,7 +324,7 @@ __global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, 
 
 
 // ---------------------------------------------------------------------------
-// near field + L2P, float32 form.  A block takes one leaf and up to 64 of
+// near field, float32 form.  A block takes one leaf and up to 64 of
 // its targets per pass: G = ceil(targets / U) target groups x (256 / G)
 // source slices, each thread holding U targets (8 real, 4 complex) so that
 // every source read from shared memory serves U pairs.  The near-list
@@ -357,7 +337,7 @@ __global__ void __launch_bounds__(NF_T) k_near(int nleaf, Tabs tb, TreeView tv, 
 // the unit circle and the first two terms of the rest (sincosf cost more than
 // the rest of the pair: sphere of 20,480 tri6 738 -> 573 us, of 81,920 3142 ->
 // 2290, FMA pipe 65 % busy).  Tile partial sums are added with compensation,
-// slices as float32 pairs, the local expansion in float64.
+// slices as float32 pairs.
 // ---------------------------------------------------------------------------
 constexpr int NF2_T = 256, NF2_ENT = 256, NF2_SLOTS = 64, NF2_MAXC = 8;
 __host__ __device__ constexpr int nf2_u(int C) { return C == 1 ? 8 : 4; }
@@ -514,12 +494,11 @@ __host__ __device__ constexpr size_t nf2_dyn_bytes(int C, bool TAB) {
 
 template <int C, bool DL, bool TAB, bool CL>
 __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
-    k_near_f32(int ns_, const int2 *__restrict__ items, Tabs tb, TreeView tv, QuadView qv, double kwave,
-               const float *__restrict__ f, const float *__restrict__ L, double *__restrict__ ytmp,
+    k_near_f32(int ns_, const int2 *__restrict__ items, TreeView tv, QuadView qv, double kwave,
+               const float *__restrict__ f, double *__restrict__ ytmp,
                const float *__restrict__ wave, const int *__restrict__ skip) {
     constexpr int U = nf2_u(C);                       // targets per thread
     constexpr int SLOTS = NF2_SLOTS;                  // targets per pass (at most SLOTS / U groups)
-    constexpr int LP = NF2_T / SLOTS;                 // threads per target in the local expansion
     constexpr int UC = U * C;
     constexpr int TILE = nf2_tile(C, TAB);            // sources staged per round
     if (skip && *skip) return;                        // every block of the cluster reads the same word
@@ -527,16 +506,13 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
     const int2 item = items[blockIdx.x / ns];         // (leaf, first target of the pass)
     const int b = tv.leaves[item.x];
     const int tid = threadIdx.x, lane = tid & 31;
-    // The staged-source region is reused once the sources are done: slice
-    // sums, local-expansion partials and the targets' powers (23 KB at most).
+    // The staged-source region is reused for the slices' sums once the sources are done.
     extern __shared__ float4 near_tile[];
     float4 *sa = near_tile, *sb = near_tile + TILE;                     // sincosf form: position | Re f, normal | Im f
     float4 *s0 = near_tile, *s1 = s0 + TILE, *s2 = s1 + TILE, *s3 = s2 + TILE;   // packed forms (see the staging)
     float *ks = (float *)(near_tile + nf2_stage(C, TAB));   // [UC][NF2_T] compensated sums
     float *kc = ks + UC * NF2_T;                      // [UC][NF2_T] their carries
     float *red = (float *)near_tile;                  // [slice][slot][C]
-    float *lred = red + NF2_T * UC;                   // [part][slot][C]
-    float *spow = lred + NF2_T * C;                   // [slot][3][PMAX + 1]
     __shared__ int pref[NF2_ENT + 1];
     __shared__ int ebase[NF2_ENT];                    // first quadrature point of each entry's box
     __shared__ float eoff[NF2_ENT][3];                // entry box centre - target leaf centre
@@ -549,7 +525,6 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
     const float kt = (float)ktd, ktl = (float)(ktd - (double)kt);   // k in table steps per length
     if (C == 2 && TAB)
         for (int i = tid; i < 2 * NF2_TAB; i += NF2_T) sw[i] = wave[i];
-    const int np = tb.np, p = order_of(tb, tv.level[b]), npl = np_of(p);   // the leaf's order; np the stride
     const int t0 = item.y, nt = min(SLOTS, tv.ne[b] - t0);
     const int G = (nt + U - 1) / U, S = NF2_T / G, tg = tid % G, sl = tid / G;
     const bool worker = sl < S;
@@ -800,44 +775,11 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
         for (int u = 0; u < U; u++)
 #pragma unroll
             for (int c = 0; c < C; c++) red[((size_t)sl * G * U + tg + G * u) * C + c] = ks[(u * C + c) * NF2_T + tid];
-    // local expansion at the targets: powers of the scaled offsets, then
-    // LP threads per target each take every LP-th term
-    if (tid < nt) {
-        const int k = t0 + tid;
-        const double ih = scalbn(1.0 / tv.side, tv.level[b]);   // 1 / h of the leaf
-        const float dx = (float)((tv.tx[k] - cbx) * ih), dy = (float)((tv.ty[k] - cby) * ih),
-                    dz = (float)((tv.tz[k] - cbz) * ih);
-        float qx = 1.f, qy = 1.f, qz = 1.f;
-        float *sp = spow + (size_t)tid * 3 * (PMAX + 1);
-        for (int e = 0; e <= p; e++) {
-            sp[e] = qx;
-            sp[PMAX + 1 + e] = qy;
-            sp[2 * (PMAX + 1) + e] = qz;
-            qx *= dx;
-            qy *= dy;
-            qz *= dz;
-        }
-    }
-    __syncthreads();
-    {
-        const int slot = tid % SLOTS, part_id = tid / SLOTS;
-        KahanF loc[C];
-        if (slot < nt) {
-            const float *sp = spow + (size_t)slot * 3 * (PMAX + 1);
-            for (int a = rank * LP + part_id; a < npl; a += ns * LP) {
-                const float mono = sp[tb.m[a]] * sp[PMAX + 1 + tb.n[a]] * sp[2 * (PMAX + 1) + tb.k[a]];
-#pragma unroll
-                for (int c = 0; c < C; c++) loc[c].add(mono * L[((size_t)b * np + a) * C + c]);
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < C; c++) lred[(part_id * SLOTS + slot) * C + c] = loc[c].s;
-    }
     __syncthreads();
     {
         // four threads per target add every fourth slice (target t0 + slot sits in
         // place slot = tg + G u of each), then each other's sums
-        static_assert(NF2_T == 4 * SLOTS && LP == 4, "four threads per target");
+        static_assert(NF2_T == 4 * SLOTS, "four threads per target");
         const int slot = tid >> 2, q0 = tid & 3;
 #pragma unroll
         for (int c = 0; c < C; c++) {
@@ -845,13 +787,11 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
             if (slot < nt)
                 for (int q = q0; q < S; q += 4) k.add(red[((size_t)q * G * U + slot) * C + c]);
             // float32 pairs (few float64 operations: 1 / 64 of the rate)
-            float h = k.s, l = -k.c, lh = lred[(q0 * SLOTS + slot) * C + c], ll = 0.f;
+            float h = k.s, l = -k.c;
 #pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
+            for (int o = 1; o < 4; o <<= 1)
                 df_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
-                df_add(lh, ll, __shfl_xor_sync(0xffffffffu, lh, o), __shfl_xor_sync(0xffffffffu, ll, o));
-            }
-            if (q0 == 0) share[slot][c] = ((double)h + (double)l) * (0.25 / M_PI) + ((double)lh + (double)ll);
+            if (q0 == 0) share[slot][c] = ((double)h + (double)l) * (0.25 / M_PI);
         }
     }
     if (CL) cluster_sync(); else __syncthreads();
@@ -868,12 +808,91 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
 }
 
 // ---------------------------------------------------------------------------
+// L2P: the local expansion at the targets of a leaf (the near field's work
+// items).  256 / SLOTS threads per target share its rows (m, n) of polynomials
+// in z (Horner), float32 rows added with compensation.  The result goes to y, or
+// is added to it (ADD, where the near field wrote the same array before).
+// ---------------------------------------------------------------------------
+constexpr int L2P_T = 256;
+template <class R, int C, int SLOTS>
+__global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, Tabs tb, TreeView tv, const R *__restrict__ L,
+                                               double *__restrict__ y, int add, const int *__restrict__ skip) {
+    if (skip && *skip) return;
+    constexpr int PARTS = L2P_T / SLOTS;
+    extern __shared__ __align__(16) unsigned char l2p_sm[];
+    __shared__ R px[PMAX + 1][SLOTS], py[PMAX + 1][SLOTS];
+    __shared__ double red[PARTS][SLOTS][C];
+    R *sL = (R *)l2p_sm;                              // [np of the leaf's order][C]
+    const int2 item = items[blockIdx.x];
+    const int b = tv.leaves[item.x], tid = threadIdx.x, slot = tid % SLOTS, part = tid / SLOTS;
+    const int t0 = item.y, nt = min(SLOTS, tv.ne[b] - t0), k = t0 + (slot < nt ? slot : 0);
+    const int p = order_of(tb, tv.level[b]), npl = np_of(p);
+    for (int i = tid; i < npl * C; i += L2P_T) sL[i] = L[(size_t)b * tb.np * C + i];
+    const double ih = scalbn(1.0 / tv.side, tv.level[b]);     // 1 / edge of the leaf
+    const R z = (R)((tv.tz[k] - tv.cz[b]) * ih);
+    if (part < 2) {
+        const R d = (R)((part ? tv.ty[k] - tv.cy[b] : tv.tx[k] - tv.cx[b]) * ih);
+        R (*pw)[SLOTS] = part ? py : px, v = (R)1;
+        for (int e = 0; e <= p; e++) {
+            pw[e][slot] = v;
+            v *= d;
+        }
+    }
+    __syncthreads();
+    const int nrow = (p + 1) * (p + 2) / 2;
+    R sum[C], car[C];
+#pragma unroll
+    for (int c = 0; c < C; c++) sum[c] = car[c] = (R)0;
+    int m = 0, first = 0;                             // rows of m start at first
+    for (int r = part; r < nrow; r += PARTS) {
+        while (r - first >= p + 1 - m) first += p + 1 - m++;
+        const int n = r - first;
+        // coefficients (m, n, e) from the highest degree down: index differences d (d + 1) / 2 + d - m + 1
+        int i = npl - np_of(p) + (p > 0 ? np_of(p - 1) : 0) + (p - m) * (p - m + 1) / 2 + (p - m - n);
+        R v[C];
+#pragma unroll
+        for (int c = 0; c < C; c++) v[c] = (R)0;
+        for (int d = p; d >= m + n; d--) {
+#pragma unroll
+            for (int c = 0; c < C; c++) v[c] = fma(v[c], z, sL[i * C + c]);
+            i -= d * (d + 1) / 2 + d - m + 1;
+        }
+        const R xy = px[m][slot] * py[n][slot];
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            if constexpr (sizeof(R) == sizeof(float)) {
+                const R a = __fmaf_rn(v[c], xy, -car[c]), t = __fadd_rn(sum[c], a);
+                car[c] = __fsub_rn(__fsub_rn(t, sum[c]), a);
+                sum[c] = t;
+            } else {
+                sum[c] = fma(v[c], xy, sum[c]);
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < C; c++) red[part][slot][c] = (double)sum[c] - (double)car[c];
+    __syncthreads();
+    if (tid < nt) {
+        const int node = tv.node_perm[t0 + tid];
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            double v = 0.0;
+#pragma unroll
+            for (int q = 0; q < PARTS; q++) v += red[q][tid][c];
+            double *o = y + (size_t)node * C + c;
+            *o = add ? *o + v : v;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // correction SpMV + diagonal: one warp per node row
-//   op A: y = C x - (ytmp + K_D x);  op B: y = -(ytmp + K_S x)
+//   op A: y = C x - (near + far + K_D x);  op B: y = -(near + far + K_S x)
+// (yfar null: ytmp holds near + far)
 // ---------------------------------------------------------------------------
 template <class RV, int C, bool OPA>
 __global__ void k_combine(int N, const int *__restrict__ ptr, const int *__restrict__ col, const RV *__restrict__ val,
-                          const double *__restrict__ Cdiag, const double *__restrict__ ytmp,
+                          const double *__restrict__ Cdiag, const double *__restrict__ ytmp, const double *__restrict__ yfar,
                           const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
                           const int *__restrict__ skip) {
     if (skip && *skip) return;
@@ -912,7 +931,7 @@ __global__ void k_combine(int N, const int *__restrict__ ptr, const int *__restr
     if (lane == 0) {
 #pragma unroll
         for (int c = 0; c < C; c++) {
-            const double tot = ytmp[(size_t)w * C + c] + s[c];
+            const double reg = ytmp[(size_t)w * C + c], tot = (yfar ? reg + yfar[(size_t)w * C + c] : reg) + s[c];
             y[(size_t)w * C + c] = OPA ? Cdiag[w] * x[(size_t)w * C + c] - tot : -tot;
         }
     }
@@ -934,7 +953,7 @@ template <int C, bool OPA>
 __global__ void k_combine_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
                             const float *__restrict__ val, const float *__restrict__ xf,
                             const double *__restrict__ Cdiag, const double *__restrict__ ytmp,
-                            const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
+                            const double *__restrict__ yfar, const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
                             const int *__restrict__ skip) {
     if (skip && *skip) return;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -984,7 +1003,7 @@ __global__ void k_combine_f(int N, const int *__restrict__ ptr, const int *__res
         double *y = (double *)*yslot;
 #pragma unroll
         for (int c = 0; c < C; c++) {
-            const double tot = ytmp[(size_t)w * C + c] + s[c];
+            const double reg = ytmp[(size_t)w * C + c], tot = (yfar ? reg + yfar[(size_t)w * C + c] : reg) + s[c];
             y[(size_t)w * C + c] = OPA ? Cdiag[w] * x[(size_t)w * C + c] - tot : -tot;
         }
     }
@@ -1157,6 +1176,7 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
         BEM_TRY(A.alloc(&P->L, (size_t)nbox * np * C));
     }
     BEM_TRY(A.alloc(&P->ytmp, (size_t)P->N * C));
+    if (!P->diag_mode) BEM_TRY(A.alloc(&P->yfar, (size_t)P->N * C));
     BEM_TRY(A.alloc(&P->xptr, 2));
     BEM_TRY(A.alloc(&P->yptr, 2));
     if (mx) BEM_TRY(A.alloc(&P->xf, (size_t)std::max(P->N, P->nchi) * C));
@@ -1180,11 +1200,50 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
     return BEM_OK;
 }
 
+// near-field sums of every node into ytmp
+template <class R, int C>
+static int launch_near(bem_plan *P, int op, double kwave, const R *f, double *ytmp, cudaStream_t s) {
+    const TreeView tv = view_of(P);
+    const QuadView qv = quad_of(P);
+    const Tree &t = P->t;
+    const int *sk = P->skip;
+    if constexpr (sizeof(R) == sizeof(float)) {
+        const int ni = P->near_nitems[C - 1];
+        const int2 *it = P->near_items[C - 1];
+        if (ni == 0) return BEM_OK;
+        // blocks per item
+        int ns = 1;
+        while (ns < NF2_MAXC && ni * ns < NF2_WAVES * 3 * P->sm_count) ns *= 2;
+        auto near = [&](auto shared, auto alone, size_t sm) {
+            return launch_cluster(ns > 1 ? shared : alone, (unsigned)(ni * ns), NF2_T, sm, ns, s, ns, it, tv, qv, kwave, f,
+                                  ytmp, P->wave, sk);
+        };
+#define BEM_NEAR(C_, DL_, TAB_) \
+    return near(k_near_f32<C_, DL_, TAB_, true>, k_near_f32<C_, DL_, TAB_, false>, nf2_dyn_bytes(C_, TAB_))
+        // (two points of one near field are at most some 4 sides apart; see near_pairs_apply)
+        if (C == 2 && kwave * t.side * 8.0 * (NF2_TAB / (2.0 * M_PI)) >= NF2_MAXPHASE) {
+            if (op == BEM_OP_A) BEM_NEAR(2, true, false);
+            BEM_NEAR(2, false, false);
+        }
+        if (op == BEM_OP_A) BEM_NEAR(C, true, true);
+        BEM_NEAR(C, false, true);
+#undef BEM_NEAR
+    } else {
+        if (near_pairs_apply(P, C, kwave)) return launch_near_pairs<C>(P, op, kwave, f, ytmp, s);
+        if constexpr (C == 2) {
+            if (op == BEM_OP_A) (k_near<true><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tv, qv, kwave, f, ytmp, sk), ::bem::count_launch());
+            else (k_near<false><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tv, qv, kwave, f, ytmp, sk), ::bem::count_launch());
+            BEM_LAUNCH_CHECK();
+        }
+        return BEM_OK;
+    }
+}
+
 // ev (optional, BEM_NSTAGES + 1 events): recorded before the first stage and
 // after every stage, for per-stage timing outside graphs.
 template <class R, int C>
-static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *ytmp, cudaStream_t s,
-                   cudaEvent_t *ev) {
+static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *ytmp, double *yfar, cudaStream_t s,
+                   cudaEvent_t *ev, cudaStream_t fork) {
     if (ev) BEM_CUDA(cudaEventRecord(ev[0], s));
     const Tabs tb = tabs_of(P);
     const TreeView tv = view_of(P);
@@ -1196,6 +1255,13 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     const int Q = (int)P->Q;
     (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, f, sk), ::bem::count_launch());
     if (ev) BEM_CUDA(cudaEventRecord(ev[1], s));
+    // the near field reads the strengths alone: under a capture it takes a branch
+    // of its own beside the expansions
+    auto near = [&](cudaStream_t ns) -> int { return launch_near<R, C>(P, op, kwave, f, ytmp, ns); };
+    if (fork) {
+        BEM_CUDA(cudaEventRecord(P->fork_ev[0], s));
+        BEM_CUDA(cudaStreamWaitEvent(fork, P->fork_ev[0], 0));
+    }
     if constexpr (sizeof(R) == sizeof(float)) {
         if (op == BEM_OP_A && P->p2m_W)
             launch_p2m_stored<C>(t.nleaf, np, tv, P->p2m_W, f, M, sk, s);
@@ -1205,40 +1271,22 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
         BEM_TRY(launch_p2m_pairs<C>(P, op == BEM_OP_A, f, M, s));
     }
     BEM_LAUNCH_CHECK();
+    if (fork) {
+        BEM_TRY(near(fork));
+        BEM_CUDA(cudaEventRecord(P->fork_ev[1], fork));
+    }
     if (ev) BEM_CUDA(cudaEventRecord(ev[2], s));
     BEM_TRY((launch_translations<R, C>(P, M, L, s, ev)));
-    if constexpr (sizeof(R) == sizeof(float)) {
-        const int ni = P->near_nitems[C - 1];
-        const int2 *it = P->near_items[C - 1];
-        // blocks per item
-        int ns = 1;
-        while (ns < NF2_MAXC && ni * ns < NF2_WAVES * 3 * P->sm_count) ns *= 2;
-        auto near = [&](auto shared, auto alone, size_t sm) {
-            return launch_cluster(ns > 1 ? shared : alone, (unsigned)(ni * ns), NF2_T, sm, ns, s, ns, it, tb, tv, qv, kwave,
-                                  (const float *)f, (const float *)L, ytmp, P->wave, sk);
-        };
-#define BEM_NEAR(C_, DL_, TAB_) \
-    BEM_TRY(near(k_near_f32<C_, DL_, TAB_, true>, k_near_f32<C_, DL_, TAB_, false>, nf2_dyn_bytes(C_, TAB_)))
-        if (ni > 0) {
-            // (two points of one near field are at most some 4 sides apart; see near_pairs_apply)
-            if (C == 2 && kwave * t.side * 8.0 * (NF2_TAB / (2.0 * M_PI)) >= NF2_MAXPHASE) {
-                if (op == BEM_OP_A) BEM_NEAR(2, true, false);
-                else BEM_NEAR(2, false, false);
-            } else {
-                if (op == BEM_OP_A) BEM_NEAR(C, true, true);
-                else BEM_NEAR(C, false, true);
-            }
-#undef BEM_NEAR
-        }
-    } else {
-        if (near_pairs_apply(P, C, kwave)) {
-            BEM_TRY(launch_near_pairs<C>(P, op, kwave, f, L, ytmp, s));
-        } else if constexpr (C == 2) {
-            if (op == BEM_OP_A) (k_near<true><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
-            else (k_near<false><<<t.nleaf, NF_T, 0, s>>>(t.nleaf, tb, tv, qv, kwave, f, L, ytmp, sk), ::bem::count_launch());
-        }
-    }
+    if (!fork) BEM_TRY(near(s));
+    // L2P beside the near field where there is an array for its result, else after it
+    const int ni = P->near_nitems[C - 1];
+    constexpr int SLOTS = sizeof(R) == sizeof(float) ? NF2_SLOTS : ND_SLOTS;
+    if (ni > 0)
+        (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, L, yfar ? yfar : ytmp,
+                                                                 yfar ? 0 : 1, sk),
+         ::bem::count_launch());
     BEM_LAUNCH_CHECK();
+    if (fork) BEM_CUDA(cudaStreamWaitEvent(s, P->fork_ev[1], 0));
     if (ev) BEM_CUDA(cudaEventRecord(ev[6], s));
     return BEM_OK;
 }
@@ -1294,46 +1342,47 @@ int field_moments(bem_plan *P, const void *phi, const void *chi, cudaStream_t s)
 // from the device slots P->xptr[0] / P->yptr[0].  with_diag = 0 leaves the
 // regular far + near sums in the regular-sum buffer (used for the diagonal).
 // wb (optional) names the work buffers of this product; NULL = the plan's.
+// fork (optional, under a capture only): a second stream for the near field.
 int enqueue_matvec_raw(bem_plan *P, int op, int green, double kwave, int with_diag, cudaStream_t s,
-                       cudaEvent_t *ev, const WorkBufs *wb) {
+                       cudaEvent_t *ev, const WorkBufs *wb, cudaStream_t fork) {
     const int C = green == BEM_HELMHOLTZ ? 2 : 1;
     const bool mx = P->prm.precision == BEM_MIXED;
     WorkBufs w;
     if (wb) w = *wb;
-    else if (mx) w = WorkBufs{P->ff, P->fM, P->fL, P->ytmp};
-    else w = WorkBufs{P->f, P->M, P->L, P->ytmp};
+    else if (mx) w = WorkBufs{P->ff, P->fM, P->fL, P->ytmp, with_diag ? P->yfar : nullptr};
+    else w = WorkBufs{P->f, P->M, P->L, P->ytmp, with_diag ? P->yfar : nullptr};
     if (!mx) {
         double *f = (double *)w.f, *M = (double *)w.M, *L = (double *)w.L;
-        if (C == 1) BEM_TRY((run_fmm<double, 1>(P, op, kwave, f, M, L, w.ytmp, s, ev)));
-        else BEM_TRY((run_fmm<double, 2>(P, op, kwave, f, M, L, w.ytmp, s, ev)));
+        if (C == 1) BEM_TRY((run_fmm<double, 1>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
+        else BEM_TRY((run_fmm<double, 2>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
     } else {
         float *f = (float *)w.f, *M = (float *)w.M, *L = (float *)w.L;
-        if (C == 1) BEM_TRY((run_fmm<float, 1>(P, op, kwave, f, M, L, w.ytmp, s, ev)));
-        else BEM_TRY((run_fmm<float, 2>(P, op, kwave, f, M, L, w.ytmp, s, ev)));
+        if (C == 1) BEM_TRY((run_fmm<float, 1>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
+        else BEM_TRY((run_fmm<float, 2>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
     }
     if (!with_diag) return BEM_OK;
-    double *const ytmp = w.ytmp;
+    double *const ytmp = w.ytmp, *const yfar = w.yfar;
     const int N = (int)P->N;
     const Correction &K = P->corr;
     const int blocks = (N * 32 + 255) / 256;
 #define BEM_COMBINE(RV, VD, VS)                                                                                 \
     if (op == BEM_OP_A) {                                                                                       \
-        if (C == 1) (k_combine<RV, 1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
-        else (k_combine<RV, 2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
+        if (C == 1) (k_combine<RV, 1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
+        else (k_combine<RV, 2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
     } else {                                                                                                    \
-        if (C == 1) (k_combine<RV, 1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
-        else (k_combine<RV, 2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
+        if (C == 1) (k_combine<RV, 1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
+        else (k_combine<RV, 2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
     }
     if (mx) {
         const int64_t nx = (int64_t)(op == BEM_OP_A ? N : P->nchi) * C;
         (k_x_float<<<(int)std::min<int64_t>((nx + 255) / 256, 4096), 256, 0, s>>>(nx, P->xptr, P->xf, P->skip),
          ::bem::count_launch());
         if (op == BEM_OP_A) {
-            if (C == 1) (k_combine_f<1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());
-            else (k_combine_f<2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+            if (C == 1) (k_combine_f<1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+            else (k_combine_f<2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
         } else {
-            if (C == 1) (k_combine_f<1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());
-            else (k_combine_f<2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+            if (C == 1) (k_combine_f<1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+            else (k_combine_f<2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
         }
     } else {
         BEM_COMBINE(double, K.valD, K.valS)
@@ -1426,7 +1475,7 @@ void free_fmm(bem_plan *P) {
     Arena &A = P->arena;
     for (void *q : {(void *)P->d_m, (void *)P->d_n, (void *)P->d_k, (void *)P->d_idx3, (void *)P->d_fact,
                     (void *)P->f, (void *)P->M, (void *)P->L, (void *)P->ff, (void *)P->fM,
-                    (void *)P->fL, (void *)P->ytmp, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->d_lev_p})
+                    (void *)P->fL, (void *)P->ytmp, (void *)P->yfar, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->d_lev_p})
         A.release(q);
     P->p2m_W = nullptr;
     P->xf = nullptr;
@@ -1434,7 +1483,7 @@ void free_fmm(bem_plan *P) {
     P->lev_var = false;
     P->d_m = P->d_n = P->d_k = P->d_idx3 = nullptr;
     P->d_fact = nullptr;
-    P->f = P->M = P->L = P->ytmp = nullptr;
+    P->f = P->M = P->L = P->ytmp = P->yfar = nullptr;
     P->ff = P->fM = P->fL = nullptr;
     P->xptr = nullptr;
     P->yptr = nullptr;
@@ -1501,7 +1550,7 @@ extern "C" int bem_matvec_noalloc(bem_plan *P, int op, const void *x_dev, void *
         // this product's work buffers are carved from the scratch and passed to
         // the launches as arguments; the plan's own fields are not touched
         unsigned char *base = (unsigned char *)g_noalloc_addr[P->device];
-        const WorkBufs w{base, base + bf, base + bf + bm, (double *)(base + bf + 2 * bm)};
+        const WorkBufs w{base, base + bf, base + bf + bm, (double *)(base + bf + 2 * bm), nullptr};
         cudaStream_t s = (cudaStream_t)cuda_stream;
         rc = set_slots(P, x_dev, y_dev, s);
         if (rc == BEM_OK) {

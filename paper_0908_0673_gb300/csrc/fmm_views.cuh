@@ -33,12 +33,12 @@ Tabs tabs_of(const bem_plan *P);
 TreeView view_of(const bem_plan *P);
 QuadView quad_of(const bem_plan *P);
 
-// float64 near field + L2P in float32 pairs (near_f64.cu)
+// float64 near field in float32 pairs (near_f64.cu)
 constexpr int ND_SLOTS = 32;            // targets per work item
 int near_pairs_prepare(bem_plan *P);
 bool near_pairs_apply(const bem_plan *P, int C, double kwave);
 template <int C>
-int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, const double *L, double *ytmp, cudaStream_t s);
+int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, double *ytmp, cudaStream_t s);
 
 // P2M of float64 plans in float32 pairs (p2m_f64.cu)
 int p2m_pairs_prepare();

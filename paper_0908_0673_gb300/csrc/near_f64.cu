@@ -1,5 +1,5 @@
-// Near field (regular rule over the near-list boxes) fused with L2P for
-// float64 plans, in float32 pairs (dfloat.cuh).
+// Near field (regular rule over the near-list boxes) of float64 plans, in
+// float32 pairs (dfloat.cuh).
 //
 // In float64 arithmetic a pair of the double layer is about 17 instructions on
 // a pipe with 1/64 of the float32 rate, which bound the whole product.  In
@@ -29,8 +29,8 @@
 // Layout as the float32 kernel (fmm.cu): a work item is one leaf and up to 32
 // of its targets; G = ceil(targets / U) target groups x (256 / G) source
 // slices, sources staged in shared memory in rounds of 512.  A cluster of 1 to
-// 8 blocks shares an item (each takes a contiguous share of its sources and of
-// its local-expansion terms) and block 0 adds the shares in rank order through
+// 8 blocks shares an item (each takes a contiguous share of its sources) and
+// block 0 adds the shares in rank order through
 // distributed shared memory: small trees have fewer items than the chip has
 // SMs.  Deterministic for a given plan.
 #include <algorithm>
@@ -251,9 +251,8 @@ __device__ __forceinline__ void pair_step(const P2 (&tH)[3], const P2 (&t1)[3], 
 }
 
 template <int C, bool DL>
-__global__ void __launch_bounds__(ND_T, 2) k_near_pairs(int ns, const int2 *__restrict__ items, Tabs tb, TreeView tv,
-                                                        QuadView qv, double kwave, const double *__restrict__ f,
-                                                        const double *__restrict__ L, double *__restrict__ ytmp,
+__global__ void __launch_bounds__(ND_T, 2) k_near_pairs(int ns, const int2 *__restrict__ items, TreeView tv, QuadView qv,
+                                                        double kwave, const double *__restrict__ f, double *__restrict__ ytmp,
                                                         const float4 *__restrict__ circle, const int *__restrict__ skip) {
     if (skip && *skip) return;                       // every block of the cluster reads the same word
     constexpr int U = nd_u(C);
@@ -263,8 +262,7 @@ __global__ void __launch_bounds__(ND_T, 2) k_near_pairs(int ns, const int2 *__re
     __shared__ int pref[ND_ENT + 1], ebase[ND_ENT];
     __shared__ float eoff[ND_ENT][9];                // entry box centre - target leaf centre, scaled, three words
     __shared__ float tpos[SLOTS][9];                 // target - target leaf centre: H, L1, L2
-    __shared__ double px[PMAX + 1][SLOTS], py[PMAX + 1][SLOTS];
-    __shared__ double part[ND_T / 32][SLOTS][C], share[SLOTS][C];
+    __shared__ double share[SLOTS][C];
     __shared__ float wmax[ND_T / 32];
     __shared__ int wexp[ND_T / 32];
     const int rank = ns > 1 ? (int)cluster_rank() : 0;
@@ -464,48 +462,7 @@ __global__ void __launch_bounds__(ND_T, 2) k_near_pairs(int ns, const int2 *__re
                 }
         }
     }
-    // powers of the targets' offsets in units of the leaf's edge
-    const int p = order_of(tb, tv.level[b]), np = tb.np, P1 = tb.p + 1;
-    const double h = scalbn(tv.side, -tv.level[b]);
-    if (tid < 2 * SLOTS) {
-        const int slot = tid % SLOTS, k = t0 + (slot < nt ? slot : 0);
-        const double d = tid < SLOTS ? (tv.tx[k] - cb[0]) / h : (tv.ty[k] - cb[1]) / h;
-        double (*pw)[SLOTS] = tid < SLOTS ? px : py;
-        double v = 1.0;
-        for (int e = 0; e <= p; e++) {
-            pw[e][slot] = v;
-            v *= d;
-        }
-    }
     __syncthreads();                                 // sources done: the staged region is reused below
-    // local expansion: rows (m, n) of z polynomials (Horner), shared by the warps and the cluster
-    {
-        const int slot = lane, k = t0 + (slot < nt ? slot : 0);
-        const double z = (tv.tz[k] - cb[2]) / h;
-        double loc[C];
-#pragma unroll
-        for (int c = 0; c < C; c++) loc[c] = 0.0;
-        const int nrow = (p + 1) * (p + 2) / 2;
-        int m = 0, first = 0;                        // rows of m start at first
-        for (int r = rank * (ND_T / 32) + warp; r < nrow; r += ns * (ND_T / 32)) {
-            while (r - first >= p + 1 - m) first += p + 1 - m++;
-            const int n = r - first;
-            const int *id = tb.idx3 + (m * P1 + n) * P1;
-            double v[C];
-#pragma unroll
-            for (int c = 0; c < C; c++) v[c] = 0.0;
-            for (int e = p - m - n; e >= 0; e--) {
-                const double *Lb = L + ((size_t)b * np + __ldg(id + e)) * C;
-#pragma unroll
-                for (int c = 0; c < C; c++) v[c] = fma(v[c], z, __ldg(Lb + c));
-            }
-            const double xy = px[m][slot] * py[n][slot];
-#pragma unroll
-            for (int c = 0; c < C; c++) loc[c] = fma(v[c], xy, loc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < C; c++) part[warp][slot][c] = loc[c];
-    }
     // slices: eight threads per target add every eighth slice, then each other's sums
     float2 *red = (float2 *)stage;                   // [C][slot][S]
     if (worker)
@@ -535,12 +492,7 @@ __global__ void __launch_bounds__(ND_T, 2) k_near_pairs(int ns, const int2 *__re
                 const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sll, o);
                 df_add(sh, sll, oh, ol);
             }
-            if ((tid & 7) == 0) {
-                double loc = 0.0;
-#pragma unroll
-                for (int w = 0; w < ND_T / 32; w++) loc += part[w][slot][c];
-                share[slot][c] = ((double)sh + (double)sll) * unit + loc;
-            }
+            if ((tid & 7) == 0) share[slot][c] = ((double)sh + (double)sll) * unit;
         }
     }
     if (ns > 1) cluster_sync(); else __syncthreads();
@@ -583,7 +535,7 @@ int circle_table(int device, const float4 **out) {
 }
 
 template <int C, bool DL>
-int launch(bem_plan *P, double kwave, const double *f, const double *L, double *ytmp, cudaStream_t s) {
+int launch(bem_plan *P, double kwave, const double *f, double *ytmp, cudaStream_t s) {
     const int ni = P->near_nitems[C - 1];
     if (ni == 0) return BEM_OK;
     // blocks per item: the smallest power of two that fills two blocks per SM
@@ -596,7 +548,7 @@ int launch(bem_plan *P, double kwave, const double *f, const double *L, double *
         tv.near_idx = P->leaf_near_idx;
     }
     BEM_TRY(launch_cluster(k_near_pairs<C, DL>, (unsigned)(ni * ns), ND_T, nd_dyn_bytes(C, DL), ns, s, ns,
-                           (const int2 *)P->near_items[C - 1], tabs_of(P), tv, quad_of(P), kwave, f, L, ytmp, P->circle,
+                           (const int2 *)P->near_items[C - 1], tv, quad_of(P), kwave, f, ytmp, P->circle,
                            (const int *)P->skip));
     return BEM_OK;
 }
@@ -622,10 +574,10 @@ int near_pairs_prepare(bem_plan *P) {
 }
 
 template <int C>
-int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, const double *L, double *ytmp, cudaStream_t s) {
-    return op == BEM_OP_A ? launch<C, true>(P, kwave, f, L, ytmp, s) : launch<C, false>(P, kwave, f, L, ytmp, s);
+int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, double *ytmp, cudaStream_t s) {
+    return op == BEM_OP_A ? launch<C, true>(P, kwave, f, ytmp, s) : launch<C, false>(P, kwave, f, ytmp, s);
 }
-template int launch_near_pairs<1>(bem_plan *, int, double, const double *, const double *, double *, cudaStream_t);
-template int launch_near_pairs<2>(bem_plan *, int, double, const double *, const double *, double *, cudaStream_t);
+template int launch_near_pairs<1>(bem_plan *, int, double, const double *, double *, cudaStream_t);
+template int launch_near_pairs<2>(bem_plan *, int, double, const double *, double *, cudaStream_t);
 
 }  // namespace bem
