@@ -815,48 +815,60 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
 // ---------------------------------------------------------------------------
 constexpr int L2P_T = 256;
 template <class R, int C, int SLOTS>
-__global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, Tabs tb, TreeView tv, const R *__restrict__ L,
+__global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, Tabs tb, TreeView tv,
+                                               const int *__restrict__ mexp, double inv_side, const R *__restrict__ L,
                                                double *__restrict__ y, int add, const int *__restrict__ skip) {
     if (skip && *skip) return;
-    constexpr int PARTS = L2P_T / SLOTS;
+    constexpr int PARTS = L2P_T / SLOTS, W = sizeof(R) == sizeof(float) ? 2 : 1;
     extern __shared__ __align__(16) unsigned char l2p_sm[];
-    __shared__ R px[PMAX + 1][SLOTS], py[PMAX + 1][SLOTS];
-    __shared__ double red[PARTS][SLOTS][C];
-    R *sL = (R *)l2p_sm;                              // [np of the leaf's order][C]
+    __shared__ R px[PMAX + 1][SLOTS], py[PMAX + 1][SLOTS], pz[SLOTS];
+    __shared__ R red[PARTS][SLOTS][C][W];
+    R *sL = (R *)l2p_sm;                              // [np of the leaf's order][C], row (m, n) by row, k ascending
+    __shared__ short rows[(PMAX + 1) * (PMAX + 2) / 2][2];   // m | n << 8, first coefficient
     const int2 item = items[blockIdx.x];
     const int b = tv.leaves[item.x], tid = threadIdx.x, slot = tid % SLOTS, part = tid / SLOTS;
     const int t0 = item.y, nt = min(SLOTS, tv.ne[b] - t0), k = t0 + (slot < nt ? slot : 0);
     const int p = order_of(tb, tv.level[b]), npl = np_of(p);
-    for (int i = tid; i < npl * C; i += L2P_T) sL[i] = L[(size_t)b * tb.np * C + i];
-    const double ih = scalbn(1.0 / tv.side, tv.level[b]);     // 1 / edge of the leaf
-    const R z = (R)((tv.tz[k] - tv.cz[b]) * ih);
-    if (part < 2) {
-        const R d = (R)((part ? tv.ty[k] - tv.cy[b] : tv.tx[k] - tv.cx[b]) * ih);
-        R (*pw)[SLOTS] = part ? py : px, v = (R)1;
-        for (int e = 0; e <= p; e++) {
-            pw[e][slot] = v;
-            v *= d;
+    auto row_at = [&](int m, int n) { return npl - np_of(p - m) + n * (p - m + 1) - n * (n - 1) / 2; };
+    for (int i = tid; i < npl; i += L2P_T) {
+        const int e = __ldg(mexp + i), m = e & 255, n = e >> 8 & 255, at = row_at(m, n) + (e >> 16 & 255);
+#pragma unroll
+        for (int c = 0; c < C; c++) sL[at * C + c] = L[((size_t)b * tb.np + i) * C + c];
+        if ((e >> 16 & 255) == 0) {                   // rows in order of m, then n
+            const int r = m * (p + 1) - m * (m - 1) / 2 + n;
+            rows[r][0] = (short)(m | n << 8);
+            rows[r][1] = (short)at;
+        }
+    }
+    if (part < 3) {
+        const double ih = scalbn(inv_side, tv.level[b]);      // 1 / edge of the leaf
+        const R d = (R)((part == 0 ? tv.tx[k] - tv.cx[b] : part == 1 ? tv.ty[k] - tv.cy[b] : tv.tz[k] - tv.cz[b]) * ih);
+        if (part == 2) {
+            pz[slot] = d;
+        } else {
+            R (*pw)[SLOTS] = part ? py : px, v = (R)1;
+            for (int e = 0; e <= p; e++) {
+                pw[e][slot] = v;
+                v *= d;
+            }
         }
     }
     __syncthreads();
+    const R z = pz[slot];
     const int nrow = (p + 1) * (p + 2) / 2;
     R sum[C], car[C];
 #pragma unroll
     for (int c = 0; c < C; c++) sum[c] = car[c] = (R)0;
-    int m = 0, first = 0;                             // rows of m start at first
     for (int r = part; r < nrow; r += PARTS) {
-        while (r - first >= p + 1 - m) first += p + 1 - m++;
-        const int n = r - first;
-        // coefficients (m, n, e) from the highest degree down: index differences d (d + 1) / 2 + d - m + 1
-        int i = npl - np_of(p) + (p > 0 ? np_of(p - 1) : 0) + (p - m) * (p - m + 1) / 2 + (p - m - n);
+        const int mn = rows[r][0], m = mn & 255, n = mn >> 8;
+        const R *a = sL + rows[r][1] * C;
         R v[C];
 #pragma unroll
         for (int c = 0; c < C; c++) v[c] = (R)0;
-        for (int d = p; d >= m + n; d--) {
+#pragma unroll 4
+        for (int e = p - m - n; e >= 0; e--)
 #pragma unroll
-            for (int c = 0; c < C; c++) v[c] = fma(v[c], z, sL[i * C + c]);
-            i -= d * (d + 1) / 2 + d - m + 1;
-        }
+            for (int c = 0; c < C; c++) v[c] = fma(v[c], z, a[e * C + c]);
         const R xy = px[m][slot] * py[n][slot];
 #pragma unroll
         for (int c = 0; c < C; c++) {
@@ -870,18 +882,26 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
         }
     }
 #pragma unroll
-    for (int c = 0; c < C; c++) red[part][slot][c] = (double)sum[c] - (double)car[c];
+    for (int c = 0; c < C; c++) {
+        red[part][slot][c][0] = sum[c];
+        if constexpr (W == 2) red[part][slot][c][1] = -car[c];
+    }
     __syncthreads();
-    if (tid < nt) {
-        const int node = tv.node_perm[t0 + tid];
+    for (int i = tid; i < nt * C; i += L2P_T) {
+        const int node = tv.node_perm[t0 + i / C];
+        double v;
+        if constexpr (W == 2) {                       // float32 pairs
+            float h = red[0][i / C][i % C][0], l = red[0][i / C][i % C][1];
 #pragma unroll
-        for (int c = 0; c < C; c++) {
-            double v = 0.0;
+            for (int q = 1; q < PARTS; q++) df_add(h, l, red[q][i / C][i % C][0], red[q][i / C][i % C][1]);
+            v = (double)h + (double)l;
+        } else {
+            v = red[0][i / C][i % C][0];
 #pragma unroll
-            for (int q = 0; q < PARTS; q++) v += red[q][tid][c];
-            double *o = y + (size_t)node * C + c;
-            *o = add ? *o + v : v;
+            for (int q = 1; q < PARTS; q++) v += red[q][i / C][i % C][0];
         }
+        double *o = y + (size_t)node * C + i % C;
+        *o = add ? *o + v : v;
     }
 }
 
@@ -889,58 +909,88 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
 // correction SpMV + diagonal: one warp per node row
 //   op A: y = C x - (near + far + K_D x);  op B: y = -(near + far + K_S x)
 // (yfar null: ytmp holds near + far)
+//
+// A warp walks a row's nonzeros, four per lane in flight; the lanes' sums go to
+// shared memory, eight threads add a row's, and one thread per row (all lanes of
+// a warp, for 32 rows a block) takes the float64 end.  With a shuffle reduction
+// and one lane's float64 end per row the float64 pipe (two operations a cycle
+// and SM, whatever the lanes) was 80 % busy: Helmholtz mixed, 40,962 rows,
+// 7.5M nonzeros 64 -> 39 us (with the copy of x), 163,842 rows, 30M nonzeros
+// 214 -> 88.
 // ---------------------------------------------------------------------------
-template <class RV, int C, bool OPA>
-__global__ void k_combine(int N, const int *__restrict__ ptr, const int *__restrict__ col, const RV *__restrict__ val,
-                          const double *__restrict__ Cdiag, const double *__restrict__ ytmp, const double *__restrict__ yfar,
-                          const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
-                          const int *__restrict__ skip) {
+constexpr int CB_T = 256;
+
+// values of a row's end: y = C x - (near + far + s) or -(near + far + s)
+template <int C, bool OPA>
+__device__ __forceinline__ void combine_end(int row, int c, double s, const double *Cdiag, const double *ytmp, const double *yfar,
+                                            const double *x, double *y) {
+    const size_t i = (size_t)row * C + c;
+    const double reg = ytmp[i], tot = (yfar ? reg + yfar[i] : reg) + s;
+    y[i] = OPA ? Cdiag[row] * x[i] - tot : -tot;
+}
+
+template <int C, bool OPA, int RW>
+__global__ void __launch_bounds__(CB_T) k_combine(int N, const int *__restrict__ ptr, const int *__restrict__ col,
+                                                  const double *__restrict__ val, const double *__restrict__ Cdiag,
+                                                  const double *__restrict__ ytmp, const double *__restrict__ yfar,
+                                                  const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
+                                                  const int *__restrict__ skip) {
     if (skip && *skip) return;
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= N) return;
+    constexpr int ROWS = CB_T / 32 * RW;
+    __shared__ double part[ROWS][C][33], total[ROWS][C];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row0 = blockIdx.x * ROWS;
     const double *x = (const double *)*xslot;
     double *y = (double *)*yslot;
-    double s[C];
+    int p[RW + 1];
 #pragma unroll
-    for (int c = 0; c < C; c++) s[c] = 0.0;
-    auto term = [&](int q, int j) {
-        if (C == 1) {
-            s[0] += (double)val[q] * x[j];
-        } else {
-            const double vr = (double)val[2 * (size_t)q], vi = (double)val[2 * (size_t)q + 1];
-            const double xr = x[2 * (size_t)j], xi = x[2 * (size_t)j + 1];
-            s[0] += vr * xr - vi * xi;
-            s[C - 1] += vr * xi + vi * xr;
+    for (int r = 0; r <= RW; r++) p[r] = ptr[min(N, row0 + warp * RW + r)];
+#pragma unroll
+    for (int r = 0; r < RW; r++) {
+        double s[C];
+#pragma unroll
+        for (int c = 0; c < C; c++) s[c] = 0.0;
+        auto term = [&](int q, int j) {
+            if (C == 1) {
+                s[0] += val[q] * x[j];
+            } else {
+                const double vr = val[2 * (size_t)q], vi = val[2 * (size_t)q + 1];
+                const double xr = x[2 * (size_t)j], xi = x[2 * (size_t)j + 1];
+                s[0] += vr * xr - vi * xi;
+                s[C - 1] += vr * xi + vi * xr;
+            }
+        };
+        // four of a lane's columns loaded ahead, nonzeros summed in order
+        constexpr int CU = 4;
+        const int qe = p[r + 1];
+        int q = p[r] + lane;
+        for (; q + 32 * (CU - 1) < qe; q += 32 * CU) {
+            int j[CU];
+#pragma unroll
+            for (int u = 0; u < CU; u++) j[u] = col[q + 32 * u];
+#pragma unroll
+            for (int u = 0; u < CU; u++) term(q + 32 * u, j[u]);
         }
-    };
-    // four of a lane's columns loaded ahead, nonzeros summed in order
-    constexpr int CU = 4;
-    const int qe = ptr[w + 1];
-    int q = ptr[w] + lane;
-    for (; q + 32 * (CU - 1) < qe; q += 32 * CU) {
-        int j[CU];
+        for (; q < qe; q += 32) term(q, col[q]);
 #pragma unroll
-        for (int u = 0; u < CU; u++) j[u] = col[q + 32 * u];
-#pragma unroll
-        for (int u = 0; u < CU; u++) term(q + 32 * u, j[u]);
+        for (int c = 0; c < C; c++) part[warp * RW + r][c][lane] = s[c];
     }
-    for (; q < qe; q += 32) term(q, col[q]);
+    __syncthreads();
+    for (int i = tid; i < ROWS * C * 8; i += CB_T) {  // whole groups of eight threads
+        const int rc = i >> 3, j = i & 7;
+        const double *v = part[rc / C][rc % C] + 4 * j;
+        double s = (v[0] + v[1]) + (v[2] + v[3]);
 #pragma unroll
-    for (int c = 0; c < C; c++)
-        for (int off = 16; off; off >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], off);
-    if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < C; c++) {
-            const double reg = ytmp[(size_t)w * C + c], tot = (yfar ? reg + yfar[(size_t)w * C + c] : reg) + s[c];
-            y[(size_t)w * C + c] = OPA ? Cdiag[w] * x[(size_t)w * C + c] - tot : -tot;
-        }
+        for (int o = 1; o < 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (j == 0) total[rc / C][rc % C] = s;
     }
+    __syncthreads();
+    for (int i = tid; i < ROWS * C; i += CB_T)
+        if (row0 + i / C < N) combine_end<C, OPA>(row0 + i / C, i % C, total[i / C][i % C], Cdiag, ytmp, yfar, x, y);
 }
 
 // float32 correction product (mixed plans): the vector is first copied to
-// float32 (one conversion per entry instead of one per nonzero: float64
-// arithmetic is a small fraction of the float32 rate), each lane sums its
-// nonzeros with compensation, the lanes' sums combine in float64.
+// float32 (one conversion per entry instead of one per nonzero), each lane sums
+// its nonzeros with compensation, the lanes' sums combine as float32 pairs.
 __global__ void k_x_float(int64_t n, const void *const *__restrict__ xslot, float *__restrict__ xf,
                           const int *__restrict__ skip) {
     if (skip && *skip) return;
@@ -949,64 +999,95 @@ __global__ void k_x_float(int64_t n, const void *const *__restrict__ xslot, floa
         xf[i] = (float)x[i];
 }
 
-template <int C, bool OPA>
-__global__ void k_combine_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
-                            const float *__restrict__ val, const float *__restrict__ xf,
-                            const double *__restrict__ Cdiag, const double *__restrict__ ytmp,
-                            const double *__restrict__ yfar, const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
-                            const int *__restrict__ skip) {
+template <int C, bool OPA, int RW>
+__global__ void __launch_bounds__(CB_T) k_combine_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
+                                                    const float *__restrict__ val, const float *__restrict__ xf,
+                                                    const double *__restrict__ Cdiag, const double *__restrict__ ytmp,
+                                                    const double *__restrict__ yfar, const void *const *__restrict__ xslot,
+                                                    void *const *__restrict__ yslot, const int *__restrict__ skip) {
     if (skip && *skip) return;
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= N) return;
-    KahanF k[C];
-    auto term = [&](float2 v, float2 x) {
-        if (C == 1) {
-            k[0].add(v.x * x.x);
-        } else {
-            k[0].add(fmaf(v.x, x.x, -v.y * x.y));
-            k[C - 1].add(fmaf(v.x, x.y, v.y * x.x));
-        }
-    };
+    constexpr int ROWS = CB_T / 32 * RW;
+    __shared__ float2 part[ROWS][C][33], total[ROWS][C];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row0 = blockIdx.x * ROWS;
+    int p[RW + 1];
+#pragma unroll
+    for (int r = 0; r <= RW; r++) p[r] = ptr[min(N, row0 + warp * RW + r)];
     auto ldv = [&](int q) {
         return C == 1 ? make_float2(__ldg(val + q), 0.f) : __ldg(reinterpret_cast<const float2 *>(val) + q);
     };
     auto ldx = [&](int j) {
         return C == 1 ? make_float2(__ldg(xf + j), 0.f) : __ldg(reinterpret_cast<const float2 *>(xf) + j);
     };
-    // four of a lane's nonzeros in flight at a time (columns, values, then
-    // the vector entries), summed in the same order as one at a time
-    constexpr int CU = 4;
-    const int qe = ptr[w + 1];
-    int q = ptr[w] + lane;
-    for (; q + 32 * (CU - 1) < qe; q += 32 * CU) {
-        int j[CU];
-        float2 v[CU], x[CU];
 #pragma unroll
-        for (int u = 0; u < CU; u++) {
-            j[u] = __ldg(col + q + 32 * u);
-            v[u] = ldv(q + 32 * u);
+    for (int r = 0; r < RW; r++) {
+        KahanF k[C];
+        auto term = [&](float2 v, float2 x) {
+            if (C == 1) {
+                k[0].add(v.x * x.x);
+            } else {
+                k[0].add(fmaf(v.x, x.x, -v.y * x.y));
+                k[C - 1].add(fmaf(v.x, x.y, v.y * x.x));
+            }
+        };
+        // four of a lane's nonzeros in flight at a time (columns, values, then
+        // the vector entries), summed in the same order as one at a time
+        constexpr int CU = 4;
+        const int qe = p[r + 1];
+        int q = p[r] + lane;
+        for (; q + 32 * (CU - 1) < qe; q += 32 * CU) {
+            int j[CU];
+            float2 v[CU], x[CU];
+#pragma unroll
+            for (int u = 0; u < CU; u++) {
+                j[u] = __ldg(col + q + 32 * u);
+                v[u] = ldv(q + 32 * u);
+            }
+#pragma unroll
+            for (int u = 0; u < CU; u++) x[u] = ldx(j[u]);
+#pragma unroll
+            for (int u = 0; u < CU; u++) term(v[u], x[u]);
+        }
+        // the rest the same way, entries beyond the row's end as zeros
+        {
+            int j[CU];
+            float2 v[CU], x[CU];
+#pragma unroll
+            for (int u = 0; u < CU - 1; u++) {
+                const bool on = q + 32 * u < qe;
+                j[u] = on ? __ldg(col + q + 32 * u) : -1;
+                v[u] = on ? ldv(q + 32 * u) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < CU - 1; u++) x[u] = j[u] >= 0 ? ldx(j[u]) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < CU - 1; u++)
+                if (j[u] >= 0) term(v[u], x[u]);
         }
 #pragma unroll
-        for (int u = 0; u < CU; u++) x[u] = ldx(j[u]);
-#pragma unroll
-        for (int u = 0; u < CU; u++) term(v[u], x[u]);
+        for (int c = 0; c < C; c++) part[warp * RW + r][c][lane] = make_float2(k[c].s, -k[c].c);
     }
-    for (; q < qe; q += 32) term(ldv(q), ldx(__ldg(col + q)));
-    double s[C];
+    __syncthreads();
+    for (int i = tid; i < ROWS * C * 8; i += CB_T) {  // whole groups of eight threads
+        const int rc = i >> 3, j = i & 7;
+        const float2 *v = part[rc / C][rc % C] + 4 * j;
+        float h = v[0].x, l = v[0].y;
 #pragma unroll
-    for (int c = 0; c < C; c++) {
-        s[c] = (double)k[c].s - (double)k[c].c;
-        for (int off = 16; off; off >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], off);
-    }
-    if (lane == 0) {
-        const double *x = (const double *)*xslot;
-        double *y = (double *)*yslot;
+        for (int u = 1; u < 4; u++) df_add(h, l, v[u].x, v[u].y);
 #pragma unroll
-        for (int c = 0; c < C; c++) {
-            const double reg = ytmp[(size_t)w * C + c], tot = (yfar ? reg + yfar[(size_t)w * C + c] : reg) + s[c];
-            y[(size_t)w * C + c] = OPA ? Cdiag[w] * x[(size_t)w * C + c] - tot : -tot;
+        for (int o = 1; o < 8; o <<= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
+            df_add(h, l, oh, ol);
         }
+        if (j == 0) total[rc / C][rc % C] = make_float2(h, l);
     }
+    __syncthreads();
+    const double *x = (const double *)*xslot;
+    double *y = (double *)*yslot;
+    for (int i = tid; i < ROWS * C; i += CB_T)
+        if (row0 + i / C < N) {
+            const float2 s = total[i / C][i % C];
+            combine_end<C, OPA>(row0 + i / C, i % C, (double)s.x + (double)s.y, Cdiag, ytmp, yfar, x, y);
+        }
 }
 
 // C_i = 1 + (regular Laplace double layer of phi = 1) + (correction row sum),
@@ -1282,7 +1363,7 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     const int ni = P->near_nitems[C - 1];
     constexpr int SLOTS = sizeof(R) == sizeof(float) ? NF2_SLOTS : ND_SLOTS;
     if (ni > 0)
-        (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, L, yfar ? yfar : ytmp,
+        (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, P->sy_mexp, 1.0 / tv.side, L, yfar ? yfar : ytmp,
                                                                  yfar ? 0 : 1, sk),
          ::bem::count_launch());
     BEM_LAUNCH_CHECK();
@@ -1364,30 +1445,39 @@ int enqueue_matvec_raw(bem_plan *P, int op, int green, double kwave, int with_di
     double *const ytmp = w.ytmp, *const yfar = w.yfar;
     const int N = (int)P->N;
     const Correction &K = P->corr;
-    const int blocks = (N * 32 + 255) / 256;
-#define BEM_COMBINE(RV, VD, VS)                                                                                 \
-    if (op == BEM_OP_A) {                                                                                       \
-        if (C == 1) (k_combine<RV, 1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
-        else (k_combine<RV, 2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, VD, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
-    } else {                                                                                                    \
-        if (C == 1) (k_combine<RV, 1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch()); \
-        else (k_combine<RV, 2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, VS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());       \
-    }
+    // four rows a warp where that still makes eight blocks per SM
+    const bool four = N >= 32 * 8 * P->sm_count;
+    const int blocks = four ? (N + 31) / 32 : (N + 7) / 8;
+    const bool a = op == BEM_OP_A;
+    const int *ptr = a ? K.ptrD : K.ptrS, *col = a ? K.colD : K.colS;
     if (mx) {
-        const int64_t nx = (int64_t)(op == BEM_OP_A ? N : P->nchi) * C;
+        const int64_t nx = (int64_t)(a ? N : P->nchi) * C;
         (k_x_float<<<(int)std::min<int64_t>((nx + 255) / 256, 4096), 256, 0, s>>>(nx, P->xptr, P->xf, P->skip),
          ::bem::count_launch());
-        if (op == BEM_OP_A) {
-            if (C == 1) (k_combine_f<1, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
-            else (k_combine_f<2, true><<<blocks, 256, 0, s>>>(N, K.ptrD, K.colD, K.fvalD, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+        auto go = [&](auto kernel) {
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.fvalD : K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip),
+             ::bem::count_launch());
+        };
+        if (four) {
+            if (C == 1) a ? go(k_combine_f<1, true, 4>) : go(k_combine_f<1, false, 4>);
+            else a ? go(k_combine_f<2, true, 4>) : go(k_combine_f<2, false, 4>);
         } else {
-            if (C == 1) (k_combine_f<1, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
-            else (k_combine_f<2, false><<<blocks, 256, 0, s>>>(N, K.ptrS, K.colS, K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip), ::bem::count_launch());
+            if (C == 1) a ? go(k_combine_f<1, true, 1>) : go(k_combine_f<1, false, 1>);
+            else a ? go(k_combine_f<2, true, 1>) : go(k_combine_f<2, false, 1>);
         }
     } else {
-        BEM_COMBINE(double, K.valD, K.valS)
+        auto go = [&](auto kernel) {
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.valD : K.valS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip),
+             ::bem::count_launch());
+        };
+        if (four) {
+            if (C == 1) a ? go(k_combine<1, true, 4>) : go(k_combine<1, false, 4>);
+            else a ? go(k_combine<2, true, 4>) : go(k_combine<2, false, 4>);
+        } else {
+            if (C == 1) a ? go(k_combine<1, true, 1>) : go(k_combine<1, false, 1>);
+            else a ? go(k_combine<2, true, 1>) : go(k_combine<2, false, 1>);
+        }
     }
-#undef BEM_COMBINE
     BEM_LAUNCH_CHECK();
     if (ev) BEM_CUDA(cudaEventRecord(ev[7], s));
     return BEM_OK;
