@@ -661,7 +661,7 @@ static int gm_enqueue_start(GmSolver &g) {
     return BEM_OK;
 }
 
-constexpr int GM_CHUNK = 2;         // Arnoldi steps per chunk (two chunks in flight)
+constexpr int GM_CHUNK = 1;         // Arnoldi steps per chunk (two chunks in flight: at most one step too many)
 
 template <int C>
 static int gm_enqueue_cycle(GmSolver &g) {
