@@ -59,12 +59,13 @@ int set_slots(bem_plan *P, const void *x, void *y, cudaStream_t s) {
 int enqueue_matvec(bem_plan *P, int op, int green, double k, cudaStream_t s) {
     cudaGraphExec_t &ge = P->graph[op];
     if (!ge) {
-        if (!P->fork_ev[1]) {
+        if (!P->fork_ev[3]) {
             // the expansions' chain of short kernels before the near field's long one
             int least = 0, greatest = 0;
             BEM_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
             if (!P->capture_stream) BEM_CUDA(cudaStreamCreateWithPriority(&P->capture_stream, cudaStreamNonBlocking, greatest));
             if (!P->fork_stream) BEM_CUDA(cudaStreamCreateWithPriority(&P->fork_stream, cudaStreamNonBlocking, least));
+            if (!P->corr_stream) BEM_CUDA(cudaStreamCreateWithPriority(&P->corr_stream, cudaStreamNonBlocking, least));
             for (auto &e : P->fork_ev)
                 if (!e) BEM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         }
@@ -242,6 +243,7 @@ bem_plan::~bem_plan() {
     if (hostbuf) cudaFreeHost(hostbuf);
     if (capture_stream) cudaStreamDestroy(capture_stream);
     if (fork_stream) cudaStreamDestroy(fork_stream);
+    if (corr_stream) cudaStreamDestroy(corr_stream);
     for (auto e : fork_ev)
         if (e) cudaEventDestroy(e);
     for (auto st : setup_stream)
@@ -557,11 +559,12 @@ int bem_plan_stage_times(bem_plan *P, int op, const void *x_dev, void *y_dev, in
     for (int r = 0; r < reps && rc == BEM_OK; r++) {
         rc = enqueue_matvec_raw(P, op, P->green, P->k, 1, s, ev);
         if (rc != BEM_OK) break;
-        cudaError_t e = cudaEventSynchronize(ev[BEM_NSTAGES]);
+        cudaError_t e = cudaEventSynchronize(ev[BEM_NSTAGES - 1]);
         if (e != cudaSuccess) { rc = cuda_fail(e, "cudaEventSynchronize", __FILE__, __LINE__); break; }
         for (int i = 0; i < BEM_NSTAGES; i++) {
             float t = 0.f;
-            cudaEventElapsedTime(&t, ev[i], ev[i + 1]);
+            if (i == BEM_NSTAGES - 1) cudaEventElapsedTime(&t, ev[BEM_NSTAGES], ev[0]);   // the correction goes first
+            else cudaEventElapsedTime(&t, ev[i], ev[i + 1]);
             ms[i] += t / reps;
         }
     }

@@ -305,7 +305,6 @@ struct FmmState {
     double *f = nullptr;                // quadrature strengths [Q] (x2 for complex)
     double *M = nullptr, *L = nullptr;  // [nbox][np] scaled moments / locals (x2 complex)
     double *ytmp = nullptr;             // [N] near regular sums (x2 complex), or near + far
-    double *yfar = nullptr;             // [N] far sums, when held apart
     float *fM = nullptr, *fL = nullptr, *ff = nullptr;   // mixed-precision copies
     const void **xptr = nullptr;        // device slot: input vector of the next matvec
     void **yptr = nullptr;              // device slot: output vector
@@ -367,8 +366,8 @@ struct bem_plan : bem::FmmState {
     // graphs
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     long long graph_kernels[2] = {0, 0};
-    cudaStream_t capture_stream = nullptr, fork_stream = nullptr;   // the product's graph: expansions, near field
-    cudaEvent_t fork_ev[2] = {nullptr, nullptr};
+    cudaStream_t capture_stream = nullptr, fork_stream = nullptr, corr_stream = nullptr;   // the product's graph: expansions, near field, correction
+    cudaEvent_t fork_ev[4] = {nullptr, nullptr, nullptr, nullptr};
     // M2L on canonical offset classes (m2l_tc.cu: tensor-core form and tables;
     // m2l_simt.cu: SIMT form)
     int sy_ncls = 0;
@@ -460,7 +459,6 @@ int set_slots(bem_plan *P, const void *x, void *y, cudaStream_t s);
 struct WorkBufs {
     void *f, *M, *L;
     double *ytmp;
-    double *yfar;                       // null: the far sums are added to ytmp
 };
 int enqueue_matvec_raw(bem_plan *P, int op, int green, double k, int with_diag, cudaStream_t s,
                        cudaEvent_t *ev = nullptr, const WorkBufs *wb = nullptr, cudaStream_t fork = nullptr);

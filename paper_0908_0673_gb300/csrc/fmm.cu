@@ -810,14 +810,17 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
 // ---------------------------------------------------------------------------
 // L2P: the local expansion at the targets of a leaf (the near field's work
 // items).  256 / SLOTS threads per target share its rows (m, n) of polynomials
-// in z (Horner), float32 rows added with compensation.  The result goes to y, or
-// is added to it (ADD, where the near field wrote the same array before).
+// in z (Horner), float32 rows added with compensation.  It ends a product: out
+// holds the correction's part already and near the near field's, so
+//   out -= near + far
+// (out null: near += far, the diagonal's regular sums).
 // ---------------------------------------------------------------------------
 constexpr int L2P_T = 256;
 template <class R, int C, int SLOTS>
 __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, Tabs tb, TreeView tv,
                                                const int *__restrict__ mexp, double inv_side, const R *__restrict__ L,
-                                               double *__restrict__ y, int add, const int *__restrict__ skip) {
+                                               double *__restrict__ near, void *const *__restrict__ yslot,
+                                               const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int PARTS = L2P_T / SLOTS, W = sizeof(R) == sizeof(float) ? 2 : 1;
     extern __shared__ __align__(16) unsigned char l2p_sm[];
@@ -887,8 +890,9 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
         if constexpr (W == 2) red[part][slot][c][1] = -car[c];
     }
     __syncthreads();
+    double *out = yslot ? (double *)*yslot : nullptr;
     for (int i = tid; i < nt * C; i += L2P_T) {
-        const int node = tv.node_perm[t0 + i / C];
+        const size_t at = (size_t)tv.node_perm[t0 + i / C] * C + i % C;
         double v;
         if constexpr (W == 2) {                       // float32 pairs
             float h = red[0][i / C][i % C][0], l = red[0][i / C][i % C][1];
@@ -900,15 +904,15 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
 #pragma unroll
             for (int q = 1; q < PARTS; q++) v += red[q][i / C][i % C][0];
         }
-        double *o = y + (size_t)node * C + i % C;
-        *o = add ? *o + v : v;
+        v += near[at];
+        if (out) out[at] -= v;
+        else near[at] = v;
     }
 }
 
 // ---------------------------------------------------------------------------
-// correction SpMV + diagonal: one warp per node row
-//   op A: y = C x - (near + far + K_D x);  op B: y = -(near + far + K_S x)
-// (yfar null: ytmp holds near + far)
+// correction SpMV + diagonal, the first part of a product to reach the output:
+//   op A: y = C x - K_D x;  op B: y = -K_S x
 //
 // A warp walks a row's nonzeros, four per lane in flight; the lanes' sums go to
 // shared memory, eight threads add a row's, and one thread per row (all lanes of
@@ -920,19 +924,16 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
 // ---------------------------------------------------------------------------
 constexpr int CB_T = 256;
 
-// values of a row's end: y = C x - (near + far + s) or -(near + far + s)
+// a row's end
 template <int C, bool OPA>
-__device__ __forceinline__ void combine_end(int row, int c, double s, const double *Cdiag, const double *ytmp, const double *yfar,
-                                            const double *x, double *y) {
+__device__ __forceinline__ void row_end(int row, int c, double s, const double *Cdiag, const double *x, double *y) {
     const size_t i = (size_t)row * C + c;
-    const double reg = ytmp[i], tot = (yfar ? reg + yfar[i] : reg) + s;
-    y[i] = OPA ? Cdiag[row] * x[i] - tot : -tot;
+    y[i] = OPA ? Cdiag[row] * x[i] - s : -s;
 }
 
 template <int C, bool OPA, int RW>
-__global__ void __launch_bounds__(CB_T) k_combine(int N, const int *__restrict__ ptr, const int *__restrict__ col,
+__global__ void __launch_bounds__(CB_T) k_corr(int N, const int *__restrict__ ptr, const int *__restrict__ col,
                                                   const double *__restrict__ val, const double *__restrict__ Cdiag,
-                                                  const double *__restrict__ ytmp, const double *__restrict__ yfar,
                                                   const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
                                                   const int *__restrict__ skip) {
     if (skip && *skip) return;
@@ -985,7 +986,7 @@ __global__ void __launch_bounds__(CB_T) k_combine(int N, const int *__restrict__
     }
     __syncthreads();
     for (int i = tid; i < ROWS * C; i += CB_T)
-        if (row0 + i / C < N) combine_end<C, OPA>(row0 + i / C, i % C, total[i / C][i % C], Cdiag, ytmp, yfar, x, y);
+        if (row0 + i / C < N) row_end<C, OPA>(row0 + i / C, i % C, total[i / C][i % C], Cdiag, x, y);
 }
 
 // float32 correction product (mixed plans): the vector is first copied to
@@ -1000,10 +1001,9 @@ __global__ void k_x_float(int64_t n, const void *const *__restrict__ xslot, floa
 }
 
 template <int C, bool OPA, int RW>
-__global__ void __launch_bounds__(CB_T) k_combine_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
+__global__ void __launch_bounds__(CB_T) k_corr_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
                                                     const float *__restrict__ val, const float *__restrict__ xf,
-                                                    const double *__restrict__ Cdiag, const double *__restrict__ ytmp,
-                                                    const double *__restrict__ yfar, const void *const *__restrict__ xslot,
+                                                    const double *__restrict__ Cdiag, const void *const *__restrict__ xslot,
                                                     void *const *__restrict__ yslot, const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int ROWS = CB_T / 32 * RW;
@@ -1086,7 +1086,7 @@ __global__ void __launch_bounds__(CB_T) k_combine_f(int N, const int *__restrict
     for (int i = tid; i < ROWS * C; i += CB_T)
         if (row0 + i / C < N) {
             const float2 s = total[i / C][i % C];
-            combine_end<C, OPA>(row0 + i / C, i % C, (double)s.x + (double)s.y, Cdiag, ytmp, yfar, x, y);
+            row_end<C, OPA>(row0 + i / C, i % C, (double)s.x + (double)s.y, Cdiag, x, y);
         }
 }
 
@@ -1257,7 +1257,6 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
         BEM_TRY(A.alloc(&P->L, (size_t)nbox * np * C));
     }
     BEM_TRY(A.alloc(&P->ytmp, (size_t)P->N * C));
-    if (!P->diag_mode) BEM_TRY(A.alloc(&P->yfar, (size_t)P->N * C));
     BEM_TRY(A.alloc(&P->xptr, 2));
     BEM_TRY(A.alloc(&P->yptr, 2));
     if (mx) BEM_TRY(A.alloc(&P->xf, (size_t)std::max(P->N, P->nchi) * C));
@@ -1320,11 +1319,57 @@ static int launch_near(bem_plan *P, int op, double kwave, const R *f, double *yt
     }
 }
 
-// ev (optional, BEM_NSTAGES + 1 events): recorded before the first stage and
-// after every stage, for per-stage timing outside graphs.
+// the correction's part of a product into the output
 template <class R, int C>
-static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *ytmp, double *yfar, cudaStream_t s,
+static int launch_correction(bem_plan *P, int op, cudaStream_t s) {
+    const int N = (int)P->N;
+    const Correction &K = P->corr;
+    // four rows a warp where that still makes eight blocks per SM
+    const bool four = N >= 32 * 8 * P->sm_count;
+    const int blocks = four ? (N + 31) / 32 : (N + 7) / 8;
+    const bool a = op == BEM_OP_A;
+    const int *ptr = a ? K.ptrD : K.ptrS, *col = a ? K.colD : K.colS;
+    if constexpr (sizeof(R) == sizeof(float)) {
+        const int64_t nx = (int64_t)(a ? N : P->nchi) * C;
+        (k_x_float<<<(int)std::min<int64_t>((nx + 255) / 256, 4096), 256, 0, s>>>(nx, P->xptr, P->xf, P->skip),
+         ::bem::count_launch());
+        auto go = [&](auto kernel) {
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.fvalD : K.fvalS, P->xf, P->C, P->xptr, P->yptr, P->skip),
+             ::bem::count_launch());
+        };
+        if (four) a ? go(k_corr_f<C, true, 4>) : go(k_corr_f<C, false, 4>);
+        else a ? go(k_corr_f<C, true, 1>) : go(k_corr_f<C, false, 1>);
+    } else {
+        auto go = [&](auto kernel) {
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.valD : K.valS, P->C, P->xptr, P->yptr, P->skip),
+             ::bem::count_launch());
+        };
+        if (four) a ? go(k_corr<C, true, 4>) : go(k_corr<C, false, 4>);
+        else a ? go(k_corr<C, true, 1>) : go(k_corr<C, false, 1>);
+    }
+    BEM_LAUNCH_CHECK();
+    return BEM_OK;
+}
+
+// ev (optional, BEM_NSTAGES + 1 events): ev[0] recorded before P2Q, ev[i] after
+// stage i, and the last event before the correction, which comes first; for
+// per-stage timing outside graphs.
+//
+// Under a capture the correction (memory-bound, needs the input vector alone) and
+// the near field (arithmetic, needs the strengths alone) take branches of their
+// own beside the expansions; L2P ends the product when all three are done.
+template <class R, int C>
+static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *ytmp, int with_diag, cudaStream_t s,
                    cudaEvent_t *ev, cudaStream_t fork) {
+    if (ev) BEM_CUDA(cudaEventRecord(ev[BEM_NSTAGES], s));
+    if (with_diag) {
+        if (fork) {
+            BEM_CUDA(cudaEventRecord(P->fork_ev[0], s));
+            BEM_CUDA(cudaStreamWaitEvent(P->corr_stream, P->fork_ev[0], 0));
+        }
+        BEM_TRY((launch_correction<R, C>(P, op, fork ? P->corr_stream : s)));
+        if (fork) BEM_CUDA(cudaEventRecord(P->fork_ev[1], P->corr_stream));
+    }
     if (ev) BEM_CUDA(cudaEventRecord(ev[0], s));
     const Tabs tb = tabs_of(P);
     const TreeView tv = view_of(P);
@@ -1336,12 +1381,10 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     const int Q = (int)P->Q;
     (k_p2q<R, C><<<(Q + 255) / 256, 256, 0, s>>>(Q, P->npe, el, P->q.w, P->xptr, f, sk), ::bem::count_launch());
     if (ev) BEM_CUDA(cudaEventRecord(ev[1], s));
-    // the near field reads the strengths alone: under a capture it takes a branch
-    // of its own beside the expansions
     auto near = [&](cudaStream_t ns) -> int { return launch_near<R, C>(P, op, kwave, f, ytmp, ns); };
     if (fork) {
-        BEM_CUDA(cudaEventRecord(P->fork_ev[0], s));
-        BEM_CUDA(cudaStreamWaitEvent(fork, P->fork_ev[0], 0));
+        BEM_CUDA(cudaEventRecord(P->fork_ev[2], s));
+        BEM_CUDA(cudaStreamWaitEvent(fork, P->fork_ev[2], 0));
     }
     if constexpr (sizeof(R) == sizeof(float)) {
         if (op == BEM_OP_A && P->p2m_W)
@@ -1354,20 +1397,22 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     BEM_LAUNCH_CHECK();
     if (fork) {
         BEM_TRY(near(fork));
-        BEM_CUDA(cudaEventRecord(P->fork_ev[1], fork));
+        BEM_CUDA(cudaEventRecord(P->fork_ev[3], fork));
     }
     if (ev) BEM_CUDA(cudaEventRecord(ev[2], s));
     BEM_TRY((launch_translations<R, C>(P, M, L, s, ev)));
     if (!fork) BEM_TRY(near(s));
-    // L2P beside the near field where there is an array for its result, else after it
+    if (fork) {
+        if (with_diag) BEM_CUDA(cudaStreamWaitEvent(s, P->fork_ev[1], 0));
+        BEM_CUDA(cudaStreamWaitEvent(s, P->fork_ev[3], 0));
+    }
     const int ni = P->near_nitems[C - 1];
     constexpr int SLOTS = sizeof(R) == sizeof(float) ? NF2_SLOTS : ND_SLOTS;
     if (ni > 0)
-        (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, P->sy_mexp, 1.0 / tv.side, L, yfar ? yfar : ytmp,
-                                                                 yfar ? 0 : 1, sk),
+        (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, P->sy_mexp, 1.0 / tv.side, L,
+                                                                 ytmp, with_diag ? P->yptr : nullptr, sk),
          ::bem::count_launch());
     BEM_LAUNCH_CHECK();
-    if (fork) BEM_CUDA(cudaStreamWaitEvent(s, P->fork_ev[1], 0));
     if (ev) BEM_CUDA(cudaEventRecord(ev[6], s));
     return BEM_OK;
 }
@@ -1423,63 +1468,25 @@ int field_moments(bem_plan *P, const void *phi, const void *chi, cudaStream_t s)
 // from the device slots P->xptr[0] / P->yptr[0].  with_diag = 0 leaves the
 // regular far + near sums in the regular-sum buffer (used for the diagonal).
 // wb (optional) names the work buffers of this product; NULL = the plan's.
-// fork (optional, under a capture only): a second stream for the near field.
+// fork (optional, under a capture only): a second stream for the near field, and
+// corr_stream takes the correction.
 int enqueue_matvec_raw(bem_plan *P, int op, int green, double kwave, int with_diag, cudaStream_t s,
                        cudaEvent_t *ev, const WorkBufs *wb, cudaStream_t fork) {
     const int C = green == BEM_HELMHOLTZ ? 2 : 1;
     const bool mx = P->prm.precision == BEM_MIXED;
     WorkBufs w;
     if (wb) w = *wb;
-    else if (mx) w = WorkBufs{P->ff, P->fM, P->fL, P->ytmp, with_diag ? P->yfar : nullptr};
-    else w = WorkBufs{P->f, P->M, P->L, P->ytmp, with_diag ? P->yfar : nullptr};
+    else if (mx) w = WorkBufs{P->ff, P->fM, P->fL, P->ytmp};
+    else w = WorkBufs{P->f, P->M, P->L, P->ytmp};
     if (!mx) {
         double *f = (double *)w.f, *M = (double *)w.M, *L = (double *)w.L;
-        if (C == 1) BEM_TRY((run_fmm<double, 1>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
-        else BEM_TRY((run_fmm<double, 2>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
+        if (C == 1) BEM_TRY((run_fmm<double, 1>(P, op, kwave, f, M, L, w.ytmp, with_diag, s, ev, fork)));
+        else BEM_TRY((run_fmm<double, 2>(P, op, kwave, f, M, L, w.ytmp, with_diag, s, ev, fork)));
     } else {
         float *f = (float *)w.f, *M = (float *)w.M, *L = (float *)w.L;
-        if (C == 1) BEM_TRY((run_fmm<float, 1>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
-        else BEM_TRY((run_fmm<float, 2>(P, op, kwave, f, M, L, w.ytmp, w.yfar, s, ev, fork)));
+        if (C == 1) BEM_TRY((run_fmm<float, 1>(P, op, kwave, f, M, L, w.ytmp, with_diag, s, ev, fork)));
+        else BEM_TRY((run_fmm<float, 2>(P, op, kwave, f, M, L, w.ytmp, with_diag, s, ev, fork)));
     }
-    if (!with_diag) return BEM_OK;
-    double *const ytmp = w.ytmp, *const yfar = w.yfar;
-    const int N = (int)P->N;
-    const Correction &K = P->corr;
-    // four rows a warp where that still makes eight blocks per SM
-    const bool four = N >= 32 * 8 * P->sm_count;
-    const int blocks = four ? (N + 31) / 32 : (N + 7) / 8;
-    const bool a = op == BEM_OP_A;
-    const int *ptr = a ? K.ptrD : K.ptrS, *col = a ? K.colD : K.colS;
-    if (mx) {
-        const int64_t nx = (int64_t)(a ? N : P->nchi) * C;
-        (k_x_float<<<(int)std::min<int64_t>((nx + 255) / 256, 4096), 256, 0, s>>>(nx, P->xptr, P->xf, P->skip),
-         ::bem::count_launch());
-        auto go = [&](auto kernel) {
-            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.fvalD : K.fvalS, P->xf, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip),
-             ::bem::count_launch());
-        };
-        if (four) {
-            if (C == 1) a ? go(k_combine_f<1, true, 4>) : go(k_combine_f<1, false, 4>);
-            else a ? go(k_combine_f<2, true, 4>) : go(k_combine_f<2, false, 4>);
-        } else {
-            if (C == 1) a ? go(k_combine_f<1, true, 1>) : go(k_combine_f<1, false, 1>);
-            else a ? go(k_combine_f<2, true, 1>) : go(k_combine_f<2, false, 1>);
-        }
-    } else {
-        auto go = [&](auto kernel) {
-            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.valD : K.valS, P->C, ytmp, yfar, P->xptr, P->yptr, P->skip),
-             ::bem::count_launch());
-        };
-        if (four) {
-            if (C == 1) a ? go(k_combine<1, true, 4>) : go(k_combine<1, false, 4>);
-            else a ? go(k_combine<2, true, 4>) : go(k_combine<2, false, 4>);
-        } else {
-            if (C == 1) a ? go(k_combine<1, true, 1>) : go(k_combine<1, false, 1>);
-            else a ? go(k_combine<2, true, 1>) : go(k_combine<2, false, 1>);
-        }
-    }
-    BEM_LAUNCH_CHECK();
-    if (ev) BEM_CUDA(cudaEventRecord(ev[7], s));
     return BEM_OK;
 }
 
@@ -1565,7 +1572,7 @@ void free_fmm(bem_plan *P) {
     Arena &A = P->arena;
     for (void *q : {(void *)P->d_m, (void *)P->d_n, (void *)P->d_k, (void *)P->d_idx3, (void *)P->d_fact,
                     (void *)P->f, (void *)P->M, (void *)P->L, (void *)P->ff, (void *)P->fM,
-                    (void *)P->fL, (void *)P->ytmp, (void *)P->yfar, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->d_lev_p})
+                    (void *)P->fL, (void *)P->ytmp, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->d_lev_p})
         A.release(q);
     P->p2m_W = nullptr;
     P->xf = nullptr;
@@ -1573,7 +1580,7 @@ void free_fmm(bem_plan *P) {
     P->lev_var = false;
     P->d_m = P->d_n = P->d_k = P->d_idx3 = nullptr;
     P->d_fact = nullptr;
-    P->f = P->M = P->L = P->ytmp = P->yfar = nullptr;
+    P->f = P->M = P->L = P->ytmp = nullptr;
     P->ff = P->fM = P->fL = nullptr;
     P->xptr = nullptr;
     P->yptr = nullptr;
@@ -1640,7 +1647,7 @@ extern "C" int bem_matvec_noalloc(bem_plan *P, int op, const void *x_dev, void *
         // this product's work buffers are carved from the scratch and passed to
         // the launches as arguments; the plan's own fields are not touched
         unsigned char *base = (unsigned char *)g_noalloc_addr[P->device];
-        const WorkBufs w{base, base + bf, base + bf + bm, (double *)(base + bf + 2 * bm), nullptr};
+        const WorkBufs w{base, base + bf, base + bf + bm, (double *)(base + bf + 2 * bm)};
         cudaStream_t s = (cudaStream_t)cuda_stream;
         rc = set_slots(P, x_dev, y_dev, s);
         if (rc == BEM_OK) {
