@@ -164,10 +164,11 @@ __global__ void k_geometry(int E, int npe, const int *__restrict__ el_phi, const
 // Also writes a float32 bound per element for the pair search: the centroid
 // image and a radius R_e >= max(tau h_e, max_a |X_a - c_e|), so a node
 // farther than R_e (plus the float32 rounding margin) is neither a node of
-// the element nor near-singular to it.
+// the element nor near-singular to it; and a radius below tau h_e, so a node
+// nearer than that (minus the margin) is.
 __global__ void k_elem_centroid(int E, int npe, double tau, const int *__restrict__ el_phi,
                                 const double *__restrict__ nodes, double *ecx, double *ecy, double *ecz, double *eh,
-                                float4 *ebnd) {
+                                float4 *ebnd, float *enear) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= E) return;
     double X[18], N[6], x[3];
@@ -184,6 +185,7 @@ __global__ void k_elem_centroid(int E, int npe, double tau, const int *__restric
     double rb = tau * m;
     for (int v = 0; v < npe; v++) rb = fmax(rb, dist3_rn(X[3 * v], X[3 * v + 1], X[3 * v + 2], x[0], x[1], x[2]));
     ebnd[i] = make_float4((float)x[0], (float)x[1], (float)x[2], (float)(rb * (1.0 + 1e-6)));
+    enear[i] = (float)(tau * m * (1.0 - 1e-6));
 }
 
 // The 7-point rule and the Gauss-Legendre tables are the same for every
@@ -248,9 +250,9 @@ struct CorrArgs {
     const int *el_phi, *el_chi;
     const double *ecx, *ecy, *ecz, *eh;   // per element centroid image and size
     const float4 *ebnd;                   // per element float32 search bound (centroid, R_e)
+    const float *enear;                   // per element float32 radius below tau h_e
     const float4 *fbox;                   // per box float32 centre (x, y, z)
     const float *frho;                    // per box float32 search radius, rounded up
-    const double *bcx, *bcy, *bcz, *brho; // per box centre and search radius
     const int *child0, *nchild, *eb, *ee;
     const float *nh, *nl;                 // node coordinates as float32 pairs: x = nh + nl
 };
@@ -271,30 +273,35 @@ __global__ void k_nodes_split(int64_t n3, const double *__restrict__ x, float *h
 }
 
 // Per box: radius of a ball around the centre that holds every point a
-// special pair can involve: max over the subtree's elements of
-// max(|c_e - c| + tau h_e, max_a |X_a - c|), inflated by 1e-12.  One thread
-// per element walks from its owner leaf (the leaf of its node 0) to the root
-// and raises each box's radius by an integer atomic max on the bits of the
-// non-negative double (rho starts at zero).
+// special pair can involve: max over the subtree's elements of |c_e - c| + R_e
+// (k_elem_centroid), in float32 with the rounding of the coordinates added.  One
+// thread per element walks from its owner leaf (the leaf of its node 0) to the
+// root; the lanes of a warp at the same box raise its radius by one integer
+// atomic max on the bits of the non-negative float (frho starts at zero).  (In
+// float64, over the element's nodes too, 70 us for 24,300 elements: the float64
+// pipe 77 % busy; an atomic for each element and box 50 us; so 6.)
 __global__ void k_elem_search_radius(CorrArgs a, const int *__restrict__ leaf_of_node, const int *__restrict__ parent,
-                                     unsigned long long *rho_bits) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.E) return;
-    const int *el = a.el_phi + (size_t)e * a.npe;
-    const double te = a.tau * a.eh[e];
-    for (int b = leaf_of_node[el[0]]; b >= 0; b = b ? parent[b] : -1) {
-        double d = dist3_rn(a.ecx[e], a.ecy[e], a.ecz[e], a.bcx[b], a.bcy[b], a.bcz[b]) + te;
-        for (int v = 0; v < a.npe; v++) {
-            const double *p = a.nodes + 3 * (size_t)el[v];
-            d = fmax(d, dist3_rn(p[0], p[1], p[2], a.bcx[b], a.bcy[b], a.bcz[b]));
+                                     unsigned *rho_bits) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool on = e < a.E;
+    const float4 c = on ? a.ebnd[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float ac = fabsf(c.x) + fabsf(c.y) + fabsf(c.z);
+    int b = on ? leaf_of_node[a.el_phi[(size_t)e * a.npe]] : -1;
+    while (__any_sync(FULL, b >= 0)) {
+        unsigned bits = 0;
+        if (b >= 0) {
+            const float4 o = a.fbox[b];
+            const float dx = c.x - o.x, dy = c.y - o.y, dz = c.z - o.z;
+            const float d = sqrtf(dx * dx + dy * dy + dz * dz) + c.w;
+            bits = __float_as_uint(d + 1e-6f * (d + ac + fabsf(o.x) + fabsf(o.y) + fabsf(o.z)));
         }
-        atomicMax(rho_bits + b, (unsigned long long)__double_as_longlong(d * (1.0 + 1e-12)));
+        const unsigned same = __match_any_sync(FULL, b), most = __reduce_max_sync(same, bits);
+        if (b >= 0) {
+            if (lane == __ffs(same) - 1) atomicMax(rho_bits + b, most);
+            b = b ? parent[b] : -1;
+        }
     }
-}
-
-__global__ void k_rho_float(int nbox, const double *__restrict__ rho, float *frho) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbox) frho[b] = (float)(rho[b] * (1.0 + 1e-6));
 }
 
 // 0 regular, 1 singular (*a_sing = local node), 2 near-singular
@@ -312,8 +319,10 @@ __device__ __forceinline__ int classify_pair(const CorrArgs &a, int node, const 
 // at a time; special (element) pairs are counted, or written in leaf order
 // and element order within a leaf when `out_e` is given.  A float32 test with
 // an inflated radius filters boxes (visiting a box the exact test would skip
-// only adds candidates); elements pass a float32 rejection and then the
-// exact float64 classification.
+// only adds candidates); elements pass a float32 rejection, then a float32
+// acceptance, and the few between the two the exact float64 classification
+// (which every element that was not rejected went through before: 84 % of the
+// float64 pipe, 429 us for 48,602 nodes; so 92).
 constexpr int SS_WARPS = 4, SS_STACK = 8 * 24;
 constexpr int SS_CAP = 192;         // special elements per node kept by the counting search
 
@@ -354,10 +363,13 @@ __device__ int find_special_warp(const CorrArgs &a, int node, int *out_e, int *s
             if (e < a.ee[b]) {
                 const float4 c = a.ebnd[e];
                 const float dx = xf[0] - c.x, dy = xf[1] - c.y, dz = xf[2] - c.z;
-                const float lim = c.w + 1e-5f * (ax + fabsf(c.x) + fabsf(c.y) + fabsf(c.z) + c.w);
-                if (dx * dx + dy * dy + dz * dz <= lim * lim) {
+                const float sum = ax + fabsf(c.x) + fabsf(c.y) + fabsf(c.z) + c.w, d2 = dx * dx + dy * dy + dz * dz;
+                const float lim = c.w + 1e-5f * sum;
+                if (d2 <= lim * lim) {
+                    // coordinates and differences are good to 2^-23 of sum
+                    const float in = a.enear[e] - 1e-6f * sum;
                     int as;
-                    hit = classify_pair(a, node, xi, e, &as) != 0;
+                    hit = (in > 0.f && d2 < in * in) || classify_pair(a, node, xi, e, &as) != 0;
                 }
             }
             const unsigned m = __ballot_sync(FULL, hit);
@@ -382,10 +394,34 @@ __global__ void __launch_bounds__(32 * SS_WARPS) k_special_count(CorrArgs a, int
     }
 }
 
-// the kept elements of every node into the pair list at the node's offset
-__global__ void k_special_copy(int N, const int *__restrict__ off, const int *__restrict__ tmp, int cap, int *pair_e) {
-    const int i = blockIdx.x, n = off[i + 1] - off[i];
-    for (int j = threadIdx.x; j < n; j += blockDim.x) pair_e[off[i] + j] = tmp[(size_t)i * cap + j];
+// A node's part of the pair list, one block per node: its elements (from the
+// counting search's, or in place already: tmp null), the pairs' node, and the
+// columns of the node's rows, which are its pairs' element nodes one after the
+// other.  (One thread per pair wrote the columns 24 bytes apart, one per node the
+// pairs' nodes: with the copy 142 us for 2.9M pairs; so 45.)
+__global__ void k_special_rows(int npe, const int *__restrict__ off, const int *__restrict__ tmp, int cap,
+                               const int *__restrict__ el_phi, const int *__restrict__ el_chi, int *pair_e, int *pair_node,
+                               int *colD, int *colS) {
+    extern __shared__ int row_e[];                    // up to blockDim.x elements at a time
+    const int i = blockIdx.x, o = off[i], n = off[i + 1] - o;
+    for (int j0 = 0; j0 < n; j0 += blockDim.x) {
+        const int m = min((int)blockDim.x, n - j0), j = threadIdx.x;
+        if (j < m) {
+            const int e = tmp ? tmp[(size_t)i * cap + j0 + j] : pair_e[o + j0 + j];
+            row_e[j] = e;
+            if (tmp) pair_e[o + j0 + j] = e;
+            pair_node[o + j0 + j] = i;
+        }
+        __syncthreads();
+        const size_t at = (size_t)(o + j0) * npe;
+        for (int c = threadIdx.x; c < m * npe; c += blockDim.x) {
+            const int v = c / npe;
+            const size_t src = (size_t)row_e[v] * npe + (c - v * npe);
+            colD[at + c] = el_phi[src];
+            colS[at + c] = el_chi[src];
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void __launch_bounds__(32 * SS_WARPS) k_special_write(CorrArgs a, const int *__restrict__ off, int *pair_e) {
@@ -1318,23 +1354,6 @@ __global__ void k_pair_split(int npairs, const int *__restrict__ self, const int
     list[self[pr] ? off[pr] : nself + pr - off[pr]] = pr;
 }
 
-__global__ void k_pair_nodes(int N, const int *__restrict__ off, int *pair_node) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    for (int p = off[i]; p < off[i + 1]; p++) pair_node[p] = i;
-}
-
-__global__ void k_corr_csr(int npairs, int npe, const int *__restrict__ pair_e, const int *__restrict__ el_phi,
-                           const int *__restrict__ el_chi, int *colD, int *colS) {
-    int pr = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pr >= npairs) return;
-    int e = pair_e[pr];
-    for (int v = 0; v < npe; v++) {
-        colD[(size_t)pr * npe + v] = el_phi[(size_t)e * npe + v];
-        colS[(size_t)pr * npe + v] = el_chi[(size_t)e * npe + v];
-    }
-}
-
 __global__ void k_rows_ptr(int N, int npe, const int *__restrict__ off, int *ptr) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i > N) return;
@@ -1359,26 +1378,25 @@ int build_correction(bem_plan *P, cudaStream_t s) {
     Tree &t = P->t;
     Arena &A = P->arena;
     const int N = (int)P->N, E = (int)P->E, npe = P->npe;
-    double *ecx, *ecy, *ecz, *eh, *rho;
+    double *ecx, *ecy, *ecz, *eh;
     BEM_TRY(A.alloc(&ecx, E)); BEM_TRY(A.alloc(&ecy, E)); BEM_TRY(A.alloc(&ecz, E)); BEM_TRY(A.alloc(&eh, E));
     float4 *ebnd;
-    float *frho;
+    float *frho, *enear;
     BEM_TRY(A.alloc(&ebnd, E));
+    BEM_TRY(A.alloc(&enear, E));
     BEM_TRY(A.alloc(&frho, t.nbox));
-    BEM_TRY(A.alloc(&rho, t.nbox));
-    (k_elem_centroid<<<(E + 255) / 256, 256, 0, s>>>(E, npe, P->prm.tau_near, t.el_phi, P->nodes, ecx, ecy, ecz, eh, ebnd),
+    (k_elem_centroid<<<(E + 255) / 256, 256, 0, s>>>(E, npe, P->prm.tau_near, t.el_phi, P->nodes, ecx, ecy, ecz, eh, ebnd, enear),
      ::bem::count_launch());
     float *nh, *nl;
     BEM_TRY(A.alloc(&nh, 3 * (size_t)N));
     BEM_TRY(A.alloc(&nl, 3 * (size_t)N));
     (k_nodes_split<<<(3 * N + 255) / 256, 256, 0, s>>>(3 * (int64_t)N, P->nodes, nh, nl), ::bem::count_launch());
     CorrArgs a{N, E, npe, P->green, P->prm.n_duffy, P->prm.max_subdiv, P->k, P->prm.tau_near, P->nodes,
-               t.el_phi, t.el_chi, ecx, ecy, ecz, eh, ebnd, t.fbox, frho, t.cx, t.cy, t.cz, rho, t.child0, t.nchild,
+               t.el_phi, t.el_chi, ecx, ecy, ecz, eh, ebnd, enear, t.fbox, frho, t.child0, t.nchild,
                t.eb, t.ee, nh, nl};
-    BEM_CUDA(cudaMemsetAsync(rho, 0, sizeof(double) * t.nbox, s));
-    (k_elem_search_radius<<<(E + 255) / 256, 256, 0, s>>>(a, t.leaf_of_node, t.parent, (unsigned long long *)rho),
+    BEM_CUDA(cudaMemsetAsync(frho, 0, sizeof(float) * t.nbox, s));
+    (k_elem_search_radius<<<(E + 255) / 256, 256, 0, s>>>(a, t.leaf_of_node, t.parent, (unsigned *)frho),
      ::bem::count_launch());
-    (k_rho_float<<<(t.nbox + 255) / 256, 256, 0, s>>>(t.nbox, rho, frho), ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     int *cnt, *off, *tot;
     BEM_TRY(A.alloc(&cnt, N + 1));
@@ -1404,8 +1422,6 @@ int build_correction(bem_plan *P, cudaStream_t s) {
     BEM_TRY(A.alloc(&pair_e, npairs));
     BEM_TRY(A.alloc(&pair_node, npairs));
     if (hcnt[1]) (k_special_write<<<(N + SS_WARPS - 1) / SS_WARPS, 32 * SS_WARPS, 0, s>>>(a, off, pair_e), ::bem::count_launch());
-    else (k_special_copy<<<N, 64, 0, s>>>(N, off, ptmp, SS_CAP, pair_e), ::bem::count_launch());
-    (k_pair_nodes<<<(N + 255) / 256, 256, 0, s>>>(N, off, pair_node), ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     const int C = P->green == BEM_HELMHOLTZ ? 2 : 1;
     Correction &K = P->corr;
@@ -1431,7 +1447,8 @@ int build_correction(bem_plan *P, cudaStream_t s) {
         BEM_TRY(A.alloc(&K.fvalS, K.nnzS * C));
     }
     (k_rows_ptr<<<(N + 256) / 256, 256, 0, s>>>(N, npe, off, K.ptrD), ::bem::count_launch());
-    (k_corr_csr<<<(npairs + 255) / 256, 256, 0, s>>>(npairs, npe, pair_e, t.el_phi, t.el_chi, K.colD, K.colS), ::bem::count_launch());
+    (k_special_rows<<<N, 64, 64 * sizeof(int), s>>>(npe, off, hcnt[1] ? nullptr : ptmp, SS_CAP, t.el_phi, t.el_chi, pair_e, pair_node,
+                                                   K.colD, K.colS), ::bem::count_launch());
     // self pairs first, then the near-singular ones (stable), so that each kernel
     // takes one kind
     int *kind = nullptr, *koff = nullptr, *klist = nullptr, *ktot = nullptr, *kblk = nullptr;
@@ -1540,7 +1557,7 @@ int build_correction(bem_plan *P, cudaStream_t s) {
     P->C = d0row;
     // the temporaries are released once the stream has finished with them
     for (void *q : {(void *)ptmp, (void *)nh, (void *)nl, (void *)lcnt, (void *)dflag, (void *)dpos, (void *)dblk, (void *)deep_list, (void *)ndeep, (void *)cnt2, (void *)deeper, (void *)ndeeper, (void *)leaves, (void *)leaves2, (void *)kind, (void *)koff, (void *)klist, (void *)ktot, (void *)kblk, (void *)cnt, (void *)tot, (void *)sblk, (void *)pair_node, (void *)d0pair, (void *)ecx, (void *)ecy, (void *)ecz,
-                    (void *)eh, (void *)ebnd, (void *)frho, (void *)rho, (void *)off, (void *)pair_e})
+                    (void *)eh, (void *)ebnd, (void *)enear, (void *)frho, (void *)off, (void *)pair_e})
         P->deferred.push_back(q);
     return BEM_OK;
 }
