@@ -1154,6 +1154,7 @@ constexpr int NE_W = 8;             // lanes per pair in the evaluation
 constexpr int NE_WARPS = 4;         // warps per block of the evaluation
 
 __host__ __device__ constexpr int nw_slots(int levels) { return levels == 2 ? 16 : 64; }
+constexpr size_t ne_smem(int levels) { return sizeof(float4) * 2 * (NE_WARPS * 32 / NE_W) * (1 + nw_slots(levels)); }
 
 // LEVELS = 2: cnt[li] = leaves, or -1 and flag[li] = 1 for a deeper pair;
 // LEVELS = 3: the list is the deeper pairs' (length min(nlist, *nlist_dev)),
@@ -1263,6 +1264,7 @@ __global__ void __launch_bounds__(32 * NE_WARPS) k_near_eval(CorrArgs a, int nli
     __shared__ R sd[G][3 * NPE];
     __shared__ R smono[G][18];                           // float32: the map's monomial coefficients
     __shared__ int skey[NE_CHUNK], sorder[NE_CHUNK];
+    extern __shared__ float4 spiece[];                   // [group][1 + slots][a, e | f, determinant]
     __shared__ R srule[3][NQ];                           // the rule in shared memory: lanes read different points
     if (threadIdx.x < NQ) {
         srule[0][threadIdx.x] = rule_s<R>(threadIdx.x);
@@ -1301,29 +1303,37 @@ __global__ void __launch_bounds__(32 * NE_WARPS) k_near_eval(CorrArgs a, int nli
             constexpr bool MONO = sizeof(R) == sizeof(float);
             if (MONO) {
                 for (int i = sl; i < 18; i += W) smono[g][i] = mono_coef<R, NPE>(sd[g], i / 3, i % 3);
-                __syncwarp(wmask);
             }
+            // the pieces' corner, edges and determinant: decoded once (for each of a
+            // piece's seven points before: 1.32 ms for 2.8M pairs; so 1.16)
+            {
+                const unsigned *lv = leaves + (size_t)li * slots;
+                float4 *out = spiece + g * (slots + 1) * 2;
+                for (int i = sl; i < skey[o]; i += W) {
+                    const PieceF P = code_piece(lv[i]);
+                    const float e0 = P.b0 - P.a0, e1 = P.b1 - P.a1, f0 = P.c0 - P.a0, f1 = P.c1 - P.a1;
+                    out[2 * i + 2] = make_float4(P.a0, P.a1, e0, e1);
+                    out[2 * i + 3] = make_float4(f0, f1, fabsf(e0 * f1 - e1 * f0), 0.f);   // exact: dyadic numbers
+                }
+                if (sl == 0) {
+                    out[0] = make_float4(0.f, 0.f, 1.f, 0.f);
+                    out[1] = make_float4(0.f, 1.f, -1.f, 0.f);
+                }
+            }
+            __syncwarp(wmask);
             R v[NVP];
 #pragma unroll
             for (int i = 0; i < NVP; i++) v[i] = 0;
             const int npt = NQ * (1 + skey[o]);
-            const unsigned *lv = leaves + (size_t)li * slots;
             // point j = NQ pc + q: pc = 0 the regular rule (negative weights),
             // pc >= 1 leaf pc - 1; lane sl takes j = sl, sl + W, ...
             int pc = sl / NQ, q = sl % NQ;
             for (int j = sl; j < npt; j += W) {
-                R s, t, w;
-                const R rs = srule[0][q], rt = srule[1][q], rw = srule[2][q];
-                if (pc == 0) {
-                    s = rs; t = rt; w = -rw;
-                } else {
-                    // the q-th point of the rule on the piece, as leaf_point
-                    const PieceF P = code_piece(lv[pc - 1]);
-                    const R e0 = (R)P.b0 - (R)P.a0, e1 = (R)P.b1 - (R)P.a1, f0 = (R)P.c0 - (R)P.a0, f1 = (R)P.c1 - (R)P.a1;
-                    s = (R)P.a0 + rs * e0 + rt * f0;
-                    t = (R)P.a1 + rs * e1 + rt * f1;
-                    w = rw * fabs(e0 * f1 - e1 * f0);
-                }
+                // the q-th point of the rule on the piece, as leaf_point
+                const float4 p0 = spiece[(g * (slots + 1) + pc) * 2], p1 = spiece[(g * (slots + 1) + pc) * 2 + 1];
+                const R rs = srule[0][q], rt = srule[1][q];
+                const R s = (R)p0.x + rs * (R)p0.z + rt * (R)p1.x, t = (R)p0.y + rs * (R)p0.w + rt * (R)p1.y;
+                const R w = srule[2][q] * (R)p1.z;
                 if (MONO) point_acc_mono<R, HELM, NPE>(smono[g], kk, s, t, w, v);
                 else eval_st<R, HELM, NPE>(sd[g], kk, s, t, w, v);
                 pc += W / NQ;
@@ -1521,11 +1531,11 @@ int build_correction(bem_plan *P, cudaStream_t s) {
 #define BEM_SW(R, H, NP)                                                                                          \
     do {                                                                                                          \
         if (nnear > 0) {                                                                                          \
-            (k_near_eval<R, H, NP, NE_W><<<ge, 32 * NE_WARPS, 0, s>>>(a, nnear, nullptr, nw_slots(2), klist + nself,\
+            (k_near_eval<R, H, NP, NE_W><<<ge, 32 * NE_WARPS, ne_smem(2), s>>>(a, nnear, nullptr, nw_slots(2), klist + nself,\
                                                                        pair_node, pair_e, lcnt, leaves, corr_out<R>(K.fvalD, K.valD),\
                                                                        corr_out<R>(K.fvalS, K.valS), d0pair),                           \
              ::bem::count_launch());                                                                              \
-            (k_near_eval<R, H, NP, NE_W><<<ge2, 32 * NE_WARPS, 0, s>>>(a, dcap, ndeep, nw_slots(3), deep_list,     \
+            (k_near_eval<R, H, NP, NE_W><<<ge2, 32 * NE_WARPS, ne_smem(3), s>>>(a, dcap, ndeep, nw_slots(3), deep_list, \
                                                                         pair_node, pair_e, cnt2, leaves2, corr_out<R>(K.fvalD, K.valD),\
                                                                         corr_out<R>(K.fvalS, K.valS), d0pair),                          \
              ::bem::count_launch());                                                                              \
