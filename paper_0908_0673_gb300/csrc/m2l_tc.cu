@@ -73,7 +73,7 @@ __device__ __forceinline__ uint32_t mom_off(int r, int k) {   // byte offset in 
 constexpr int TC_XLD = 36;              // row stride (floats) of the epilogue's transpose buffer
 constexpr int TC_XPOSE = 32 * TC_XLD;   // floats of one epilogue warp's transpose buffer
 struct TcLayout {
-    size_t img, stage, sgn, xpose, bars, total;
+    size_t img, stage, sgn, xpose, bars, steps, total;
 };
 __host__ __device__ inline TcLayout tc_layout(const TcPlan &g, int ldp) {
     TcLayout L;
@@ -83,7 +83,8 @@ __host__ __device__ inline TcLayout tc_layout(const TcPlan &g, int ldp) {
     L.sgn = L.stage + (size_t)TC_NS * 2 * TC_PLANE;
     L.xpose = L.sgn + ((48 * (size_t)(ldp / 32) * 4 + 15) / 16) * 16;
     L.bars = L.xpose + (size_t)TC_EPI * TC_XPOSE * 4;
-    L.total = L.bars + 16 * 8 + 16 + 1024;
+    L.steps = L.bars + 16 * 8 + 16;
+    L.total = L.steps + TC_MAXKS * 16;
     return L;
 }
 
@@ -146,6 +147,21 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
         tc::mbar_fence_init();
     }
     for (int i = tid; i < 48 * nw; i += TC_T) sSgn[i] = a.sgn[i];
+    // a K-step's operands: low words of the image descriptors (hi, lo plane) and
+    // the instruction descriptors of its rows up to 256 and beyond (0: none)
+    uint4 *sStep = (uint4 *)(smem + LY.steps);
+    for (int j = tid; j < TC_MAXKS; j += TC_T) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (j < G.nks) {
+            const bool second = j >= G.ks_split;        // in the image's second part (it starts at ks_off[ks_split])
+            const uint32_t at = tc::smem_u32(sImg) + (uint32_t)(G.ks_off[j] - (second ? G.part_floats[0] : 0)) * 4u;
+            v.x = (uint32_t)tc::smem_desc(at, 128, 256);
+            v.y = (uint32_t)tc::smem_desc(at + (uint32_t)G.part_floats[second] * 4u, 128, 256);
+            v.z = tc::idesc_tf32(TC_M, min(256, G.ks_n[j]));
+            v.w = G.ks_n[j] > 256 ? tc::idesc_tf32(TC_M, G.ks_n[j] - 256) : 0u;
+        }
+        sStep[j] = v;
+    }
     if (warp == 0) tc::tmem_alloc(sTmem, 512);
     tc::tc_fence_before_sync();
     __syncthreads();
@@ -224,7 +240,10 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
         if (lane == 0) {
             const bool split = G.ks_split < G.nks;
             const uint32_t pb0 = (uint32_t)G.part_floats[0] * 4u, pb1 = (uint32_t)G.part_floats[1] * 4u;
-            const uint32_t ih = tc::smem_u32(sImg), st0 = tc::smem_u32(sStage);
+            const uint32_t st0 = tc::smem_u32(sStage);
+            const int jsplit = split ? G.ks_split : -1;
+            // high words of the descriptors
+            const uint64_t da = tc::smem_desc(0, 128, 1024) & ~0xffffffffull, db = tc::smem_desc(0, 128, 256) & ~0xffffffffull;
             int it = 0, cur_cls = -1, cur_part = -1;
             uint32_t nfree = 0;
             bool ok = true;
@@ -257,15 +276,21 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
                 const uint32_t dacc = tmem + ((k & 1) ? (uint32_t)colB : 0u);
                 for (int kc = 0; kc < a.nkc && ok; kc++, it++) {
                     const int s = it % TC_NS;
+                    // the chunk's operands before the wait: with the descriptors put
+                    // together from the plan's tables between the MMAs a K-step took
+                    // some 500 cycles of this thread against 25 of tensor work
+                    uint4 op[4];
+#pragma unroll
+                    for (int ks = 0; ks < 4; ks++) op[ks] = sStep[kc * 4 + ks];
+                    const uint32_t ab = st0 + (uint32_t)s * 2u * TC_PLANE;
+                    const uint32_t ah = (uint32_t)tc::smem_desc(ab, 128, 1024), al = (uint32_t)tc::smem_desc(ab + TC_PLANE, 128, 1024);
                     ok = wait_or_abort(&full[s], (uint32_t)((it / TC_NS) & 1), sAbort);
                     if (!ok) break;
                     tc::tc_fence_after_sync();
-                    const uint32_t ab = st0 + (uint32_t)s * 2u * TC_PLANE;
-                    const uint64_t ah0 = tc::smem_desc(ab, 128, 1024), al0 = tc::smem_desc(ab + TC_PLANE, 128, 1024);
+#pragma unroll
                     for (int ks = 0; ks < 4; ks++) {
-                        const int j = kc * 4 + ks;
-                        if (j >= G.nks) break;
-                        if (split && j == G.ks_split) {
+                        if (op[ks].z == 0u) break;            // beyond the last K-step
+                        if (kc * 4 + ks == jsplit) {
                             // every MMA so far reads the first part: once they have
                             // completed, the second part replaces it
                             tc::mma_commit(imgfree);
@@ -276,19 +301,16 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
                             if (!ok) break;
                             tc::tc_fence_after_sync();
                         }
-                        const int pbase = cur_part ? G.part_floats[0] : 0;   // == ks_off[ks_split]
-                        const uint32_t il = ih + (cur_part ? pb1 : pb0);
-                        const uint32_t boff = (uint32_t)(G.ks_off[j] - pbase) * 4u;
-                        const int n = G.ks_n[j];
-                        for (int part = 0; part < n; part += 256) {
-                            const int nn = min(256, n - part);
-                            const uint32_t po = boff + (uint32_t)(part / 8) * 256u;
-                            const uint64_t bh = tc::smem_desc(ih + po, 128, 256), bl = tc::smem_desc(il + po, 128, 256);
-                            const uint32_t id = tc::idesc_tf32(TC_M, nn), d = dacc + (uint32_t)part;
-                            const uint64_t ao = (uint64_t)ks * 16u;   // 256 B per K-step
-                            tc::mma_tf32(d, ah0 + ao, bh, id, j > 0);
-                            tc::mma_tf32(d, ah0 + ao, bl, id, true);
-                            tc::mma_tf32(d, al0 + ao, bh, id, true);
+                        const uint64_t xh = da | (ah + ks * 16u), xl = da | (al + ks * 16u);   // 256 B per K-step
+                        const uint64_t bh = db | op[ks].x, bl = db | op[ks].y;
+                        const bool more = kc > 0 || ks > 0;
+                        tc::mma_tf32(dacc, xh, bh, op[ks].z, more);
+                        tc::mma_tf32(dacc, xh, bl, op[ks].z, true);
+                        tc::mma_tf32(dacc, xl, bh, op[ks].z, true);
+                        if (op[ks].w != 0u) {                 // rows beyond 256 (8 KB on in the image)
+                            tc::mma_tf32(dacc + 256u, xh, bh + 512u, op[ks].w, more);
+                            tc::mma_tf32(dacc + 256u, xh, bl + 512u, op[ks].w, true);
+                            tc::mma_tf32(dacc + 256u, xl, bh + 512u, op[ks].w, true);
                         }
                     }
                     if (!ok) break;
