@@ -173,24 +173,6 @@ __global__ void __launch_bounds__(GM_T) k_orth_fused(int n, int nv, const double
     }
 }
 
-// V_out = x / *den (0 if *den is 0) and z = M^-1 V_out: the next Arnoldi
-// vector and the preconditioned product's input
-template <int C>
-__global__ void k_scale_precond(int n, const double *__restrict__ x, const double *__restrict__ den, double *vout,
-                                const double *__restrict__ dinv, double *z, const int *__restrict__ skip) {
-    if (skip && *skip) return;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const double d = *den, di = dinv[r];
-#pragma unroll
-    for (int c = 0; c < C; c++) {
-        const double v = d > 0.0 ? x[(size_t)r * C + c] / d : 0.0;
-        vout[(size_t)r * C + c] = v;
-        z[(size_t)r * C + c] = di * v;
-    }
-}
-
-// out = sum of |v|^2 partials
 template <int C>
 __global__ void k_nrm2_partial(int n, const double *__restrict__ v, double *partial, const int *__restrict__ skip) {
     if (skip && *skip) return;
@@ -215,15 +197,31 @@ __global__ void k_nrm2_final(const double *__restrict__ partial, double *out, co
 }
 
 // r = b - r  (r holds A x on entry)
-__global__ void k_resid(int n, const double *__restrict__ b, double *r, const int *__restrict__ skip) {
+// r = b - r and the partial sums of |r|^2
+template <int C>
+__global__ void k_resid_nrm2(int n, const double *__restrict__ b, double *r, double *partial, const int *__restrict__ skip) {
     if (skip && *skip) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) r[i] = b[i] - r[i];
+    __shared__ double red[GM_T];
+    double s = 0.0;
+    for (int i = blockIdx.x * GM_T + threadIdx.x; i < n * C; i += GM_BLK * GM_T) {
+        const double v = b[i] - r[i];
+        r[i] = v;
+        s += v * v;
+    }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int off = GM_T / 2; off; off >>= 1) {
+        if (threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
-
-// istate: [0] skip (set inside a cycle once converged), [1] steps of the
-// cycle, [2] halt (the solve has ended: every kernel of the solve returns)
-__global__ void k_arm(int *st) { st[0] = st[2]; }
+// before a product: the stop flag back to the halt flag, the product's slots
+__global__ void k_arm(int *st, const void **xptr, void **yptr, void *const *src, void *y) {
+    st[0] = st[2];
+    xptr[0] = *src;
+    yptr[0] = y;
+}
 
 // Targets of a mixed-precision solve.  The float32 operator's rounding leaves
 // a true (float64) residual floor of 2-5e-8.  Arnoldi steps go on until the
@@ -424,15 +422,34 @@ __global__ void k_xupdate(int n, const double *__restrict__ V, size_t ld, GmStat
     for (int c = 0; c < C; c++) x[(size_t)r * C + c] += dinv[r] * a[c];
 }
 
-__global__ void k_cycle_init(GmState S, int m) {
-    S.st[0] = S.st[2];
-    S.st[1] = 0;
-    if (S.st[2]) return;
-    for (int i = 0; i < 2 * (m + 1); i++) S.g[i] = 0.0;
-    S.g[0] = S.sc[1];   // beta
+// The start of a cycle: V_0 = r / ||r|| and M^-1 V_0 for the first product;
+// block 0 also resets the small system and points every product of the cycle at
+// z and w.  (One launch; the three parts had one each.)
+template <int C>
+__global__ void k_cycle_begin(int n, GmState S, int m, double *v0, const double *__restrict__ dinv, double *z, double *w,
+                              const void **xptr, void **yptr) {
+    const bool halted = S.st[2] != 0;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) {
+            S.st[0] = S.st[2];
+            S.st[1] = 0;
+            xptr[0] = z;
+            yptr[0] = w;
+        }
+        if (!halted)
+            for (int i = threadIdx.x; i < 2 * (m + 1); i += blockDim.x) S.g[i] = i == 0 ? S.sc[1] : 0.0;   // beta
+    }
+    if (halted) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    const double d = S.sc[1], di = dinv[r];
+#pragma unroll
+    for (int c = 0; c < C; c++) {
+        const double v = d > 0.0 ? v0[(size_t)r * C + c] / d : 0.0;
+        v0[(size_t)r * C + c] = v;
+        z[(size_t)r * C + c] = di * v;
+    }
 }
-
-// pointer slots of a solve: [0] chi (Neumann data), [1] x (the solution)
 __global__ void k_set_ptrs(void **slot, const void *chi, void *x) {
     slot[0] = (void *)chi;
     slot[1] = x;
@@ -442,10 +459,6 @@ __global__ void k_set_ptrs_tab(void **slot, const void *const *chi_tab, void *co
     slot[1] = x_tab[i];
 }
 // product input / output slots from a solve slot
-__global__ void k_slot_io(const void **xptr, void **yptr, void *const *src, void *y) {
-    xptr[0] = *src;
-    yptr[0] = y;
-}
 __global__ void k_zero_slot(void *const *slot, size_t n, const int *__restrict__ skip) {
     if (skip && *skip) return;
     double *x = (double *)*slot;
@@ -526,8 +539,7 @@ static int gm_k_start(bem_plan *P, double tol, cudaStream_t s, bool raw) {
     double *partial = P->scal + 16;
     GmState S = gm_state<C>(P);
     int *skip = P->istate;
-    (k_arm<<<1, 1, 0, s>>>(P->istate), ::bem::count_launch());
-    (k_slot_io<<<1, 1, 0, s>>>(P->xptr, P->yptr, (void *const *)P->gm_slot, P->bvec), ::bem::count_launch());
+    (k_arm<<<1, 1, 0, s>>>(P->istate, P->xptr, P->yptr, (void *const *)P->gm_slot, P->bvec), ::bem::count_launch());
     BEM_TRY(gm_product(P, BEM_OP_B, s, raw));
     (k_nrm2_partial<C><<<GM_BLK, GM_T, 0, s>>>(n, P->bvec, partial, skip), ::bem::count_launch());
     (k_nrm2_final<<<1, 32, 0, s>>>(partial, S.sc + 0, skip), ::bem::count_launch());
@@ -540,15 +552,13 @@ static int gm_k_start(bem_plan *P, double tol, cudaStream_t s, bool raw) {
 // true residual r = b - A x into V_0 (unscaled), beta = ||r||
 template <int C>
 static int gm_k_residual(bem_plan *P, cudaStream_t s, bool raw) {
-    const int n = (int)P->N, ne = n * C, eb = (ne + 255) / 256;
+    const int n = (int)P->N;
     double *V = P->V, *partial = P->scal + 16;
     GmState S = gm_state<C>(P);
     int *skip = P->istate;
-    (k_arm<<<1, 1, 0, s>>>(P->istate), ::bem::count_launch());
-    (k_slot_io<<<1, 1, 0, s>>>(P->xptr, P->yptr, (void *const *)P->gm_slot + 1, V), ::bem::count_launch());
+    (k_arm<<<1, 1, 0, s>>>(P->istate, P->xptr, P->yptr, (void *const *)P->gm_slot + 1, V), ::bem::count_launch());
     BEM_TRY(gm_product(P, BEM_OP_A, s, raw));
-    (k_resid<<<eb, 256, 0, s>>>(ne, P->bvec, V, skip), ::bem::count_launch());
-    (k_nrm2_partial<C><<<GM_BLK, GM_T, 0, s>>>(n, V, partial, skip), ::bem::count_launch());
+    (k_resid_nrm2<C><<<GM_BLK, GM_T, 0, s>>>(n, P->bvec, V, partial, skip), ::bem::count_launch());
     (k_nrm2_final<<<1, 32, 0, s>>>(partial, S.sc + 1, skip), ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     return BEM_OK;
@@ -561,10 +571,8 @@ template <int C>
 static int gm_k_cycle_begin(bem_plan *P, cudaStream_t s) {
     const int n = (int)P->N, nb = (n + 255) / 256;
     GmState S = gm_state<C>(P);
-    (k_scale_precond<C><<<nb, 256, 0, s>>>(n, P->V, S.sc + 1, P->V, P->dinv, P->zbuf, P->istate), ::bem::count_launch());
-    (k_cycle_init<<<1, 1, 0, s>>>(S, P->gm_restart), ::bem::count_launch());
-    // every product of the cycle reads M^-1 V_j from zbuf and writes w
-    BEM_TRY(set_slots(P, P->zbuf, P->w, s));
+    (k_cycle_begin<C><<<nb, 256, 0, s>>>(n, S, P->gm_restart, P->V, P->dinv, P->zbuf, P->w, P->xptr, P->yptr),
+     ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     return BEM_OK;
 }
