@@ -50,12 +50,12 @@ FLOPS_PER_PAIR_PAIRS = 190.0              # double layer in float32 pairs (float
 # capture of this workload (the command is in profiles/); reported while the
 # kernel's source file is unchanged, null otherwise.
 NCU_TRAFFIC = {
-    # k_near_f32 (unchanged since its capture; the file's other kernels changed)
-    "near_l2p": {"bytes": 7472896, "source": "paper_0908_0673_gb300/csrc/fmm.cu",
-                 "sha256": "4317124a9ff3d54da8a2ff674b49021ac10198ab50caef2b27b527477827ca7e"},
+    # k_near_f32 + k_l2p (order-10 products)
+    "near_l2p": {"bytes": 6426624 + 3205632, "source": "paper_0908_0673_gb300/csrc/fmm.cu",
+                 "sha256": "12510e466fad0650e9b1305a153b2aa0c82c11a51c3711bb58a56fe1a96a1113"},
     # the M2L stage: k_m2l_permute + k_m2l_tc + k_m2l_gather_sym (order-10 products)
-    "m2l": {"bytes": 1217024 + (35090432 + 46180096) + 123055872, "source": "paper_0908_0673_gb300/csrc/m2l_tc.cu",
-            "sha256": "e7871ff432f963f53dd84460d1103eb7b3af23f26d5a89e5156d1826afe70520"},
+    "m2l": {"bytes": 1217280 + (35175168 + 43993600) + (122822400 + 138240), "source": "paper_0908_0673_gb300/csrc/m2l_tc.cu",
+            "sha256": "9c140fd3a2a67fa8c171236e292f7ff8c7dbaa2532f25c5519d5f0ab974b7ce6"},
 }
 
 
