@@ -220,6 +220,18 @@ struct TcPlan {
     int part_floats[2] = {0, 0};        // floats of each part's plane
 };
 
+// Power of two by which a box's points reach beyond its edge, for float64 plans,
+// whose moments pass through float32 pairs.  Elements belong to the leaf of
+// their first node, so a box of small elements may own ones of many edges, and
+// (offset / edge)^16 of an offset of 300 edges is beyond float32.  Moments of
+// such a box are formed and multiplied in units of edge x 2^e, about its radius
+// r (2^(e-1) < r / edge < 2^(e+1)).  Below 8 edges e is 0: degree 20 then still
+// lies within the 2^75 of the largest where a pair keeps both its words.
+__host__ __device__ inline int box_reach(double r, double side, int level) {
+    const int e = ilogb(r) - (ilogb(side) - level);
+    return r > 0.0 && e > 2 ? e : 0;
+}
+
 // Tree and plan state (everything device-resident unless named h_*).
 struct Tree {
     int nlev = 0;                       // number of levels (root = level 0)
@@ -376,7 +388,7 @@ struct bem_plan : bem::FmmState {
     int m2l_src_lmin = 0, m2l_tgt_lmin = 0;
     double *sy_rho = nullptr;           // [class][3] canonical offsets / h_t
     double *sy_kh = nullptr;            // [class] k h_t (Helmholtz)
-    int *sy_dl = nullptr;               // [class] level difference
+    int *sy_dl = nullptr;               // [class] level difference, plus the source's box_reach in float64 plans
     int *sy_sig_u = nullptr;            // [pair] symmetry id (permutation * 8 + sign bits)
     std::vector<int> sy_hcls, sy_hsig, sy_hsrc, sy_hip;   // host: per pair class, symmetry, source; list offsets
     std::vector<int> sy_hlev, sy_hdl;                     // host: per canonical class, target level (when keyed) and dl

@@ -37,6 +37,9 @@
 // multiply-adds (261), packing over the pairs (275: T copied twice into
 // registers).  The form before rebuilt T for every tile and walked every column
 // in every warp (FMA pipe 23 % busy).
+// In float64 plans a source box with box_reach e > 0 enters with its moments x
+// 2^(-e |a|), and the class's dl (part of its key) holds e beside the level
+// difference.
 // Rows go to a buffer pair by pair and a gather sums each target's in list
 // order: deterministic, no atomics.
 #include <algorithm>
@@ -391,19 +394,27 @@ __global__ void __launch_bounds__(MG_T, W == 1 ? 3 : 2) k_m2l_gemm(const __grid_
 }
 
 // Moments under each axis permutation, in words, one block per box; float64
-// plans scale each box's by a power of two (its largest exponent, to E[box])
+// plans scale each box's by a power of two (its largest exponent, to E[box]),
+// and by 2^(-reach |a|) where its points reach far beyond its edge
 template <class R, int C>
 __global__ void __launch_bounds__(256) k_m2l_words(int np, int ldq, const unsigned short *__restrict__ fwd,
-                                                   const R *__restrict__ M, float *__restrict__ Mq, int *__restrict__ Eb,
+                                                   const int *__restrict__ mexp, const int *__restrict__ level,
+                                                   const double *__restrict__ radius, double side, const R *__restrict__ M, float *__restrict__ Mq, int *__restrict__ Eb,
                                                    const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int WC = (sizeof(R) == 8 ? 2 : 1) * C;
     const size_t box = blockIdx.x;
     const R *m = M + box * np * C;
+    const int reach = sizeof(R) == 8 ? box_reach(radius[box], side, level[box]) : 0;
+    auto moment = [&](int i) -> R {                       // i = coefficient x C + component
+        if constexpr (sizeof(R) == 8)
+            if (reach) return scalbn(m[i], -reach * (__ldg(mexp + i / C) >> 24));
+        return m[i];
+    };
     int E = 1;
     if constexpr (sizeof(R) == 8) {
         __shared__ int we[8];
-        for (int i = threadIdx.x; i < np * C; i += 256) E = max(E, (int)((unsigned)__double2hiint(m[i]) >> 20) & 0x7ff);
+        for (int i = threadIdx.x; i < np * C; i += 256) E = max(E, (int)((unsigned)__double2hiint(moment(i)) >> 20) & 0x7ff);
 #pragma unroll
         for (int o = 16; o; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
         if ((threadIdx.x & 31) == 0) we[threadIdx.x >> 5] = E;
@@ -422,7 +433,7 @@ __global__ void __launch_bounds__(256) k_m2l_words(int np, int ldq, const unsign
             const int f = __ldg(fwd + (size_t)q * 8 * np + k) & 0x7fff;
 #pragma unroll
             for (int c = 0; c < C; c++) {
-                if constexpr (sizeof(R) == 8) df_bits(m[f * C + c], E, v[2 * c], v[2 * c + 1]);
+                if constexpr (sizeof(R) == 8) df_bits(moment(f * C + c), E, v[2 * c], v[2 * c + 1]);
                 else v[c] = m[f * C + c];
             }
         }
@@ -662,7 +673,9 @@ int launch_m2l_sy(bem_plan *P, const R *M, R *L, cudaStream_t s) {
     a.skip = P->skip;
     const size_t sm = mg_smem(W, C, a.np);
     if (P->sy_ntile > 0)
-        (k_m2l_words<R, C><<<t.nbox, 256, 0, s>>>(a.np, a.ldq, P->sy_fwd, M, P->sg_Mq, P->sg_E, P->skip), ::bem::count_launch());
+        (k_m2l_words<R, C><<<t.nbox, 256, 0, s>>>(a.np, a.ldq, P->sy_fwd, P->sy_mexp, t.level, t.r, t.side, M, P->sg_Mq,
+                                                  P->sg_E, P->skip),
+         ::bem::count_launch());
     // one run of targets at a time: its tiles, then the gather of its targets
     for (size_t r = 0; r + 1 < P->sy_bt.size(); r++) {
         const int bt0 = P->sy_bt[r], nt = P->sy_bt[r + 1] - bt0, tg0 = P->sy_bb[r], ntg = P->sy_bb[r + 1] - tg0;

@@ -522,7 +522,8 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
     const int nfull = (int)dls.size();
     // every exact offset class maps to one canonical class and one symmetry
     // key: level difference, target level (Helmholtz: the derivatives depend
-    // on k h_t; zero for Laplace), sorted absolute offset components
+    // on k h_t; zero for Laplace) and the source's box_reach from bit 8 on,
+    // sorted absolute offset components
     struct Key {
         long long v[5];
         bool operator<(const Key &o) const {
@@ -575,6 +576,7 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
     std::vector<int> fcan(nfull), dlc;
     std::vector<double> rho, khc;
     P->sy_hlev.clear();
+    P->sy_hdl.clear();
     const bool helm = P->green == BEM_HELMHOLTZ;
     int nc = 0;
     for (int i = 0; i < nfull; i++) {
@@ -585,9 +587,11 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
             rho.push_back(k.v[2] * sc);
             rho.push_back(k.v[3] * sc);
             rho.push_back(k.v[4] * sc);
-            khc.push_back(helm ? P->k * std::ldexp(P->t.side, -(int)k.v[1]) : 0.0);
-            dlc.push_back(dl);
-            P->sy_hlev.push_back((int)k.v[1]);
+            const int lv = (int)(k.v[1] & 255), reach = (int)(k.v[1] >> 8);
+            khc.push_back(helm ? P->k * std::ldexp(P->t.side, -lv) : 0.0);
+            dlc.push_back(dl + reach);
+            P->sy_hdl.push_back(dl);
+            P->sy_hlev.push_back(lv);
             nc++;
         }
         fcan[fidx[i]] = nc - 1;
@@ -613,7 +617,6 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
     BEM_TRY(up(&P->sy_rho, rho));
     BEM_TRY(up(&P->sy_kh, khc));
     BEM_TRY(up(&P->sy_dl, dlc));
-    P->sy_hdl = dlc;
     BEM_TRY(up(&P->sy_sig_u, P->sy_hsig));
     return BEM_OK;
 }

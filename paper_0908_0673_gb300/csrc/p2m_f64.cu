@@ -9,7 +9,9 @@
 // their normal derivative are formed once per point, then each k costs two pair
 // multiply-adds (one for the single layer), packed over two points.  Powers come
 // from shared memory, built per 64 points; strengths are folded into the x
-// powers (real) at a power-of-two scale taken from the block's largest.
+// powers (real) at a power-of-two scale taken from the block's largest.  Offsets
+// are taken in units of the edge x 2^box_reach, so that the powers stay in
+// float32's range; the factor returns with the float64 sums.
 // Measured: 61,236 points, p = 10, double layer 593 -> 98 us; 31,500 points,
 // single layer 205 -> 37; 20,160 points, Helmholtz double layer 399 -> 68; 8,960
 // points, p = 8 (56 leaves, four blocks each) 164 -> 23.  About 9,300 float32
@@ -89,10 +91,10 @@ __global__ void __launch_bounds__(PP_T, KM <= 11 && C == 1 ? 2 : 1) k_p2m_pairs(
 #pragma unroll
     for (int w = 0; w < PP_T / 32; w++) E = max(E, wexp[w]);
     E = min(E, 2046);                                   // an infinity or NaN carries itself
-    // offsets and normals in units of the leaf's edge
-    const int es = ilogb(tv.side);
-    float uh, ul;                                       // 2^es / edge: the plan's pairs hold offsets x 2^-es
-    df_split(1.0 / scalbn(tv.side, -tv.level[b] - es), uh, ul);
+    // offsets and normals in units of the leaf's edge x 2^reach
+    const int es = ilogb(tv.side), reach = box_reach(tv.r[b], tv.side, tv.level[b]);
+    float uh, ul;                                       // 2^es / unit: the plan's pairs hold offsets x 2^-es
+    df_split(1.0 / scalbn(tv.side, reach - tv.level[b] - es), uh, ul);
     // row of this thread, in order of m + n (rows of a warp have about the same length)
     const bool worker = grp < groups;
     int deg = 0, r = tid - grp * nrow;
@@ -210,7 +212,11 @@ __global__ void __launch_bounds__(PP_T, KM <= 11 && C == 1 ? 2 : 1) k_p2m_pairs(
             }
         }
     __syncthreads();
-    const double unit = scalbn(1.0, E - 1023 - (DL ? es : 0));   // normals were taken over edge 2^-es
+    const double unit = scalbn(1.0, E - 1023 - (DL ? es : 0));   // normals were taken over the unit x 2^-es
+    // back from the unit to the edge: 2^(reach |a|)
+    auto in_edges = [&](double v, int i) {
+        return reach ? scalbn(v, reach * (tb.m[i / C] + tb.n[i / C] + tb.k[i / C])) : v;
+    };
     for (int i = tid; i < npl * C; i += PP_T) {
         float h = 0.f, l = 0.f;
         for (int g = 0; g < groups; g++) {
@@ -219,7 +225,7 @@ __global__ void __launch_bounds__(PP_T, KM <= 11 && C == 1 ? 2 : 1) k_p2m_pairs(
         }
         const double v = ((double)h + (double)l) * unit;
         if (ns > 1) share[i] = v;
-        else M[(size_t)b * np * C + i] = v;
+        else M[(size_t)b * np * C + i] = in_edges(v, i);
     }
     if (ns > 1) {
         cluster_sync();
@@ -227,7 +233,7 @@ __global__ void __launch_bounds__(PP_T, KM <= 11 && C == 1 ? 2 : 1) k_p2m_pairs(
             for (int i = tid; i < npl * C; i += PP_T) {
                 double v = share[i];
                 for (int q = 1; q < ns; q++) v += peer_double(share + i, q);
-                M[(size_t)b * np * C + i] = v;
+                M[(size_t)b * np * C + i] = in_edges(v, i);
             }
         cluster_sync();                                 // no block leaves while block 0 reads its share
     }

@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(TT) k_m2l_tables(int ncls, int p, int np, int 
 // hashing: the product's top bits depend on every bit of the key; the table
 // starts small and doubles at half load, so it stays in cache); a key that
 // does not pack goes to an ordered map.  Per class its offset vector, level
-// difference and key level, in order of first appearance.
+// difference and key level, in order of first appearance.  The level field holds
+// the source's box_reach (float64 plans) in its bits from 8 on; such keys do not pack.
 struct ClassSet {
     std::vector<unsigned long long> tkey = std::vector<unsigned long long>(4096, 0ull);
     std::vector<int> tval = std::vector<int>(4096, -1);
@@ -308,7 +309,7 @@ struct ClassSet {
     int find_or_add(long long kx, long long ky, long long kz, int dl, int lv) {
         constexpr int KB = 17;
         constexpr long long KMAX = (1ll << (KB - 1)) - 1;
-        if (std::llabs(kx) <= KMAX && std::llabs(ky) <= KMAX && std::llabs(kz) <= KMAX && dl > -64 && dl < 64) {
+        if (std::llabs(kx) <= KMAX && std::llabs(ky) <= KMAX && std::llabs(kz) <= KMAX && dl > -64 && dl < 64 && lv < 64) {
             const unsigned long long key =
                 1ull + (((unsigned long long)(kx + KMAX)) | ((unsigned long long)(ky + KMAX) << KB) |
                         ((unsigned long long)(kz + KMAX) << (2 * KB)) | ((unsigned long long)(dl + 64) << (3 * KB)) |
@@ -360,7 +361,7 @@ struct ClassSet {
 };
 
 // the classes of the pairs of boxes [b0, b1), in a set of their own
-static void number_classes(int b0, int b1, bool by_level, const int *lev, const int *ix, const int *iy, const int *iz,
+static void number_classes(int b0, int b1, bool by_level, const int *reach, const int *lev, const int *ix, const int *iy, const int *iz,
                            const int *ip, const int *ii, int *pair_cls, ClassSet &S) {
     for (int b = b0; b < b1; b++) {
         const int lb = lev[b], xb = ix[b], yb = iy[b], zb = iz[b], lv = by_level ? lb : 0;
@@ -369,7 +370,7 @@ static void number_classes(int b0, int b1, bool by_level, const int *lev, const 
             // 2 rho 2^e = (2 i_t + 1) 2^e - (2 i_s + 1) 2^(dl + e), an integer vector
             const long long ft = 1ll << e, fs = 1ll << (dl + e);
             pair_cls[u] = S.find_or_add((2ll * xb + 1) * ft - (2ll * ix[s] + 1) * fs, (2ll * yb + 1) * ft - (2ll * iy[s] + 1) * fs,
-                                        (2ll * zb + 1) * ft - (2ll * iz[s] + 1) * fs, dl, lv);
+                                        (2ll * zb + 1) * ft - (2ll * iz[s] + 1) * fs, dl, lv | reach[s] << 8);
         }
     }
 }
@@ -384,6 +385,12 @@ int build_m2l_classes(bem_plan *P) {
     BEM_CUDA(cudaMemcpy(iz.data(), t.iz, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
     BEM_CUDA(cudaMemcpy(ip.data(), t.inter_ptr, sizeof(int) * (t.nbox + 1), cudaMemcpyDeviceToHost));
     if (t.n_inter) BEM_CUDA(cudaMemcpy(ii.data(), t.inter_idx, sizeof(int) * t.n_inter, cudaMemcpyDeviceToHost));
+    std::vector<int> reach(t.nbox, 0);
+    if (P->prm.precision == BEM_F64) {
+        std::vector<double> r(t.nbox);
+        BEM_CUDA(cudaMemcpy(r.data(), t.r, sizeof(double) * t.nbox, cudaMemcpyDeviceToHost));
+        for (int b = 0; b < t.nbox; b++) reach[b] = box_reach(r[b], t.side, lev[b]);
+    }
     const bool helm = P->green == BEM_HELMHOLTZ;
     const bool by_level = helm || P->prm.p_min > 0;   // the target level enters the key
     // Classes are numbered in order of first appearance over the pairs in list
@@ -404,9 +411,9 @@ int build_m2l_classes(bem_plan *P) {
     {
         std::vector<std::thread> th;
         for (int k = 1; k < nth; k++)
-            th.emplace_back(number_classes, bcut[k], bcut[k + 1], by_level, lev.data(), ix.data(), iy.data(),
+            th.emplace_back(number_classes, bcut[k], bcut[k + 1], by_level, reach.data(), lev.data(), ix.data(), iy.data(),
                             iz.data(), ip.data(), ii.data(), pair_cls.data(), std::ref(sets[k]));
-        number_classes(bcut[0], bcut[1], by_level, lev.data(), ix.data(), iy.data(), iz.data(), ip.data(), ii.data(),
+        number_classes(bcut[0], bcut[1], by_level, reach.data(), lev.data(), ix.data(), iy.data(), iz.data(), ip.data(), ii.data(),
                        pair_cls.data(), sets[0]);
         for (auto &x : th) x.join();
     }
