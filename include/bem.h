@@ -184,7 +184,8 @@ void bem_plan_destroy(bem_plan *plan);
 
 /* One fast matrix multiplication (Section 3.6, steps 1-4) plus the stored
  * correction and the diagonal: op BEM_OP_A: y = C x - D x; BEM_OP_B: y = -S x.
- * x_dev: device [n_phi] (op A) or [n_chi] (op B); y_dev: device [n_phi].
+ * x_dev: device [n_phi] (op A) or [n_chi] (op B); y_dev: device [n_phi]; they
+ * may overlap (y is written when x has been read).
  * Stream ordered; no host synchronisation. */
 int bem_matvec(bem_plan *plan, int op, const void *x_dev, void *y_dev, void *cuda_stream);
 
@@ -358,7 +359,8 @@ int bem_plan_peak_footprint(const bem_plan *plan, size_t *hbm_bytes);
 #define BEM_NSTATS 14
 int bem_plan_stats(const bem_plan *plan, int64_t *stats);
 
-/* Stages of one product, in launch order, for bem_plan_stage_times. */
+/* Stages of one product for bem_plan_stage_times, which launches the last one
+ * first (it reads the input vector alone); L2P ends the product. */
 #define BEM_NSTAGES 7   /* P2Q, P2M, M2M, M2L, L2L, near field + L2P, correction + diagonal */
 
 /* Runs the product y = op x `reps` times outside its graph with CUDA events

@@ -352,6 +352,7 @@ struct FmmState {
     float *sg_Mq = nullptr;             // [box][6][sg_ldq][words] moments under each axis permutation, per product
     float *p2m_W = nullptr;             // [Q][np] stored double-layer P2M weights (float32 plans)
     float *xf = nullptr;                // float32 copy of a product's input (correction product)
+    double *ycor = nullptr;             // [N] correction's part of a product (x2 for complex)
     std::vector<int> lev_p;             // expansion order of each tree level
     int *d_lev_p = nullptr;
     bool lev_var = false;               // the order varies with the level (p_min > 0 and more than one order)

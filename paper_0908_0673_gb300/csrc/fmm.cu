@@ -6,9 +6,9 @@
 //   M2M  coefficient shift child -> parent                            (Eq. 8)
 //   M2L  local expansion from the interaction list                     (Eq. 7)
 //   L2L  expansion shift parent -> child, with binomials               (Eq. 9)
-//   L2P  local expansion at every vertex of a leaf, fused with
 //   P2P  the regular-rule sum over the elements of the near-field boxes
-//   then the stored special-pair correction and the diagonal C.
+//   the stored special-pair correction and the diagonal C
+//   L2P  local expansion at every vertex of a leaf; it adds the parts up.
 //
 // Moments and locals are stored scaled by powers of the box edge h:
 // Ms_alpha = I_alpha / h^|alpha|, Ls_beta = F_beta h^|beta|, so that every
@@ -810,17 +810,18 @@ __global__ void __launch_bounds__(NF2_T, C == 1 || TAB ? 3 : 4)
 // ---------------------------------------------------------------------------
 // L2P: the local expansion at the targets of a leaf (the near field's work
 // items).  256 / SLOTS threads per target share its rows (m, n) of polynomials
-// in z (Horner), float32 rows added with compensation.  It ends a product: out
-// holds the correction's part already and near the near field's, so
-//   out -= near + far
+// in z (Horner), float32 rows added with compensation.  It ends a product and
+// alone writes its output, which may be the input's memory, when every other
+// part has been summed from the input:
+//   out = corr - (near + far)
 // (out null: near += far, the diagonal's regular sums).
 // ---------------------------------------------------------------------------
 constexpr int L2P_T = 256;
 template <class R, int C, int SLOTS>
 __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, Tabs tb, TreeView tv,
                                                const int *__restrict__ mexp, double inv_side, const R *__restrict__ L,
-                                               double *__restrict__ near, void *const *__restrict__ yslot,
-                                               const int *__restrict__ skip) {
+                                               double *__restrict__ near, const double *__restrict__ corr,
+                                               void *const *__restrict__ yslot, const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int PARTS = L2P_T / SLOTS, W = sizeof(R) == sizeof(float) ? 2 : 1;
     extern __shared__ __align__(16) unsigned char l2p_sm[];
@@ -905,13 +906,14 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(const int2 *__restrict__ items, T
             for (int q = 1; q < PARTS; q++) v += red[q][i / C][i % C][0];
         }
         v += near[at];
-        if (out) out[at] -= v;
+        if (out) out[at] = corr[at] - v;
         else near[at] = v;
     }
 }
 
 // ---------------------------------------------------------------------------
-// correction SpMV + diagonal, the first part of a product to reach the output:
+// correction SpMV + diagonal, a product's part from the input vector alone, into
+// a buffer of the plan's:
 //   op A: y = C x - K_D x;  op B: y = -K_S x
 //
 // A warp walks a row's nonzeros, four per lane in flight; the lanes' sums go to
@@ -934,14 +936,13 @@ __device__ __forceinline__ void row_end(int row, int c, double s, const double *
 template <int C, bool OPA, int RW>
 __global__ void __launch_bounds__(CB_T) k_corr(int N, const int *__restrict__ ptr, const int *__restrict__ col,
                                                   const double *__restrict__ val, const double *__restrict__ Cdiag,
-                                                  const void *const *__restrict__ xslot, void *const *__restrict__ yslot,
+                                                  const void *const *__restrict__ xslot, double *__restrict__ y,
                                                   const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int ROWS = CB_T / 32 * RW;
     __shared__ double part[ROWS][C][33], total[ROWS][C];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, row0 = blockIdx.x * ROWS;
     const double *x = (const double *)*xslot;
-    double *y = (double *)*yslot;
     int p[RW + 1];
 #pragma unroll
     for (int r = 0; r <= RW; r++) p[r] = ptr[min(N, row0 + warp * RW + r)];
@@ -1004,7 +1005,7 @@ template <int C, bool OPA, int RW>
 __global__ void __launch_bounds__(CB_T) k_corr_f(int N, const int *__restrict__ ptr, const int *__restrict__ col,
                                                     const float *__restrict__ val, const float *__restrict__ xf,
                                                     const double *__restrict__ Cdiag, const void *const *__restrict__ xslot,
-                                                    void *const *__restrict__ yslot, const int *__restrict__ skip) {
+                                                    double *__restrict__ y, const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int ROWS = CB_T / 32 * RW;
     __shared__ float2 part[ROWS][C][33], total[ROWS][C];
@@ -1082,7 +1083,6 @@ __global__ void __launch_bounds__(CB_T) k_corr_f(int N, const int *__restrict__ 
     }
     __syncthreads();
     const double *x = (const double *)*xslot;
-    double *y = (double *)*yslot;
     for (int i = tid; i < ROWS * C; i += CB_T)
         if (row0 + i / C < N) {
             const float2 s = total[i / C][i % C];
@@ -1260,6 +1260,7 @@ int alloc_fmm(bem_plan *P, cudaStream_t s) {
     BEM_TRY(A.alloc(&P->xptr, 2));
     BEM_TRY(A.alloc(&P->yptr, 2));
     if (mx) BEM_TRY(A.alloc(&P->xf, (size_t)std::max(P->N, P->nchi) * C));
+    if (!P->diag_mode) BEM_TRY(A.alloc(&P->ycor, (size_t)P->N * C));
     if (mx && !P->diag_mode && !P->lev_var) {
         // stored P2M weights of the double layer (op A, every product of a solve)
         BEM_TRY(A.alloc(&P->p2m_W, (size_t)P->Q * np));
@@ -1319,7 +1320,7 @@ static int launch_near(bem_plan *P, int op, double kwave, const R *f, double *yt
     }
 }
 
-// the correction's part of a product into the output
+// the correction's part of a product into ycor
 template <class R, int C>
 static int launch_correction(bem_plan *P, int op, cudaStream_t s) {
     const int N = (int)P->N;
@@ -1334,14 +1335,14 @@ static int launch_correction(bem_plan *P, int op, cudaStream_t s) {
         (k_x_float<<<(int)std::min<int64_t>((nx + 255) / 256, 4096), 256, 0, s>>>(nx, P->xptr, P->xf, P->skip),
          ::bem::count_launch());
         auto go = [&](auto kernel) {
-            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.fvalD : K.fvalS, P->xf, P->C, P->xptr, P->yptr, P->skip),
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.fvalD : K.fvalS, P->xf, P->C, P->xptr, P->ycor, P->skip),
              ::bem::count_launch());
         };
         if (four) a ? go(k_corr_f<C, true, 4>) : go(k_corr_f<C, false, 4>);
         else a ? go(k_corr_f<C, true, 1>) : go(k_corr_f<C, false, 1>);
     } else {
         auto go = [&](auto kernel) {
-            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.valD : K.valS, P->C, P->xptr, P->yptr, P->skip),
+            (kernel<<<blocks, CB_T, 0, s>>>(N, ptr, col, a ? K.valD : K.valS, P->C, P->xptr, P->ycor, P->skip),
              ::bem::count_launch());
         };
         if (four) a ? go(k_corr<C, true, 4>) : go(k_corr<C, false, 4>);
@@ -1357,7 +1358,8 @@ static int launch_correction(bem_plan *P, int op, cudaStream_t s) {
 //
 // Under a capture the correction (memory-bound, needs the input vector alone) and
 // the near field (arithmetic, needs the strengths alone) take branches of their
-// own beside the expansions; L2P ends the product when all three are done.
+// own beside the expansions; L2P ends the product when all three are done, and
+// no kernel before it writes the output.
 template <class R, int C>
 static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *ytmp, int with_diag, cudaStream_t s,
                    cudaEvent_t *ev, cudaStream_t fork) {
@@ -1410,7 +1412,7 @@ static int run_fmm(bem_plan *P, int op, double kwave, R *f, R *M, R *L, double *
     constexpr int SLOTS = sizeof(R) == sizeof(float) ? NF2_SLOTS : ND_SLOTS;
     if (ni > 0)
         (k_l2p<R, C, SLOTS><<<ni, L2P_T, sizeof(R) * np * C, s>>>(P->near_items[C - 1], tb, tv, P->sy_mexp, 1.0 / tv.side, L,
-                                                                 ytmp, with_diag ? P->yptr : nullptr, sk),
+                                                                 ytmp, P->ycor, with_diag ? P->yptr : nullptr, sk),
          ::bem::count_launch());
     BEM_LAUNCH_CHECK();
     if (ev) BEM_CUDA(cudaEventRecord(ev[6], s));
@@ -1572,10 +1574,11 @@ void free_fmm(bem_plan *P) {
     Arena &A = P->arena;
     for (void *q : {(void *)P->d_m, (void *)P->d_n, (void *)P->d_k, (void *)P->d_idx3, (void *)P->d_fact,
                     (void *)P->f, (void *)P->M, (void *)P->L, (void *)P->ff, (void *)P->fM,
-                    (void *)P->fL, (void *)P->ytmp, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->d_lev_p})
+                    (void *)P->fL, (void *)P->ytmp, (void *)P->xptr, (void *)P->yptr, (void *)P->p2m_W, (void *)P->xf, (void *)P->ycor, (void *)P->d_lev_p})
         A.release(q);
     P->p2m_W = nullptr;
     P->xf = nullptr;
+    P->ycor = nullptr;
     P->d_lev_p = nullptr;
     P->lev_var = false;
     P->d_m = P->d_n = P->d_k = P->d_idx3 = nullptr;
