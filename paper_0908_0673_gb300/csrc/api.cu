@@ -316,6 +316,8 @@ int bem_plan_create(bem_mesh *mesh, int green, double k, const bem_fmm_params *p
     P->device = mesh->ctx->device;
     P->sm_count = mesh->ctx->sm_count;
     P->arena.cache = mesh->ctx->cache;
+    P->arena.fence = &P->fence;
+    BEM_CUDA(P->fence.init());
     P->green = green;
     P->k = green == BEM_HELMHOLTZ ? k : 0.0;
     P->prm = prm;
@@ -352,7 +354,8 @@ int bem_plan_create(bem_mesh *mesh, int green, double k, const bem_fmm_params *p
         if (e != cudaSuccess) rc = cuda_fail(e, "plan set-up", __FILE__, __LINE__);
     }
     if (rc != BEM_OK) {
-        for (auto st : P->setup_stream) cudaStreamSynchronize(st);
+        for (auto st : P->setup_stream)
+            if (cudaStreamSynchronize(st) != cudaSuccess) P->fence.unknown = true;
         delete P;
         return rc;
     }
@@ -363,7 +366,7 @@ int bem_plan_create(bem_mesh *mesh, int green, double k, const bem_fmm_params *p
 void bem_plan_destroy(bem_plan *plan) {
     if (!plan) return;
     cudaSetDevice(plan->device);
-    cudaDeviceSynchronize();
+    if (!plan->fence.idle()) plan->fence.unknown = true;   // its blocks are then freed, not kept for reuse
     delete plan;
 }
 
@@ -373,7 +376,9 @@ int bem_matvec(bem_plan *P, int op, const void *x_dev, void *y_dev, void *cuda_s
     cudaStream_t s = (cudaStream_t)cuda_stream;
     BEM_TRY(set_slots(P, x_dev, y_dev, s));
     BEM_CUDA(cudaMemsetAsync(P->skip, 0, sizeof(int), s));
-    return enqueue_matvec(P, op, P->green, P->k, s);
+    const int rc = enqueue_matvec(P, op, P->green, P->k, s);
+    P->fence.mark(s);
+    return rc;
 }
 
 int bem_solve(bem_plan *P, const void *chi_dev, void *phi_dev, int nrhs, const bem_solve_params *params,
@@ -386,7 +391,9 @@ int bem_solve(bem_plan *P, const void *chi_dev, void *phi_dev, int nrhs, const b
     if (sp.method != BEM_GMRES && sp.method != BEM_BICGSTAB) { set_error("bem_solve: unknown method %d", sp.method); return BEM_EINVAL; }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     BEM_CUDA(cudaMemsetAsync(P->skip, 0, sizeof(int), s));
-    return solve(P, chi_dev, phi_dev, nrhs, &sp, info, s);
+    const int rc = solve(P, chi_dev, phi_dev, nrhs, &sp, info, s);
+    P->fence.mark(s);
+    return rc;
 }
 
 int bem_plan_tree_sizes(const bem_plan *P, bem_tree_view *v) {
@@ -404,7 +411,7 @@ int bem_plan_tree_sizes(const bem_plan *P, bem_tree_view *v) {
 int bem_plan_export_tree(const bem_plan *P, bem_tree_view *v) {
     if (!P || !v) { set_error("bem_plan_export_tree: NULL argument"); return BEM_EINVAL; }
     BEM_CUDA(cudaSetDevice(P->device));
-    BEM_CUDA(cudaDeviceSynchronize());
+    BEM_CUDA(P->fence.wait());
     const Tree &t = P->t;
     const int nb = t.nbox;
     std::vector<int> lev, ix, iy, iz, par, nch, np_, ni, ip, ii, lon, perm, eb;
@@ -447,7 +454,7 @@ int bem_plan_export_correction(const bem_plan *P, int64_t *counts, int64_t *rowD
     counts[1] = K.nnzS;
     if (!rowD && !rowS) return BEM_OK;
     BEM_CUDA(cudaSetDevice(P->device));
-    BEM_CUDA(cudaDeviceSynchronize());
+    BEM_CUDA(P->fence.wait());
     const int C = P->green == BEM_HELMHOLTZ ? 2 : 1;
     std::vector<int> ptr, cD, cS;
     std::vector<double> vD, vS;
@@ -476,7 +483,7 @@ int bem_plan_export_expansions(const bem_plan *P, int32_t *mnk, double *moments,
         for (int a = 0; a < mi.np; a++) { mnk[3 * a] = mi.m[a]; mnk[3 * a + 1] = mi.n[a]; mnk[3 * a + 2] = mi.k[a]; }
     if (!moments && !locals) return BEM_OK;
     BEM_CUDA(cudaSetDevice(P->device));
-    BEM_CUDA(cudaDeviceSynchronize());
+    BEM_CUDA(P->fence.wait());
     const int C = P->green == BEM_HELMHOLTZ ? 2 : 1;
     const size_t n = (size_t)P->t.nbox * mi.np * C;
     std::vector<double> hm(n), hl(n);
@@ -509,7 +516,7 @@ int bem_plan_export_expansions(const bem_plan *P, int32_t *mnk, double *moments,
 int bem_plan_diagonal(const bem_plan *P, double *c) {
     if (!P || !c) { set_error("bem_plan_diagonal: NULL argument"); return BEM_EINVAL; }
     BEM_CUDA(cudaSetDevice(P->device));
-    BEM_CUDA(cudaDeviceSynchronize());
+    BEM_CUDA(P->fence.wait());
     BEM_CUDA(cudaMemcpy(c, P->C, sizeof(double) * P->N, cudaMemcpyDeviceToHost));
     return BEM_OK;
 }
@@ -523,7 +530,7 @@ int bem_plan_footprint(const bem_plan *P, size_t *hbm_bytes) {
 int bem_plan_device_status(const bem_plan *P, int *status) {
     if (!P || !status) { set_error("bem_plan_device_status: NULL argument"); return BEM_EINVAL; }
     BEM_CUDA(cudaSetDevice(P->device));
-    BEM_CUDA(cudaDeviceSynchronize());
+    BEM_CUDA(P->fence.wait());
     BEM_CUDA(cudaMemcpy(status, P->dev_err, sizeof(int), cudaMemcpyDeviceToHost));
     return BEM_OK;
 }
@@ -569,6 +576,7 @@ int bem_plan_stage_times(bem_plan *P, int op, const void *x_dev, void *y_dev, in
         }
     }
     for (auto &e : ev) cudaEventDestroy(e);
+    P->fence.mark(s);
     return rc;
 }
 

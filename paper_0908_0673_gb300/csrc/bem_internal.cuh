@@ -78,7 +78,8 @@ __host__ __device__ inline void radon7(int q, double &s, double &t, double &w) {
 // cudaFree synchronises the device).  A request takes the smallest cached
 // block of at least its size and at most twice it.  At most `limit` bytes
 // are kept (environment BEM_CACHE_BYTES, default 4 GiB); what would exceed
-// it is freed.  A block is given back only when no work can still use it.
+// it is freed.  A block is given back only when no work can still use it, so the
+// cached ones can go at any time.
 struct DevCache {
     std::mutex mu;
     std::multimap<size_t, void *> blocks;   // size -> block
@@ -111,17 +112,59 @@ struct DevCache {
     ~DevCache() { flush(); }
 };
 
+// The end of the work that a plan's latest call enqueued.  The plan's memory is
+// given back, and its state read, after a wait for this event and not for the
+// device: a device-wide wait is an error while any other thread captures a
+// graph, ends that capture, and has crashed in the driver beside one.  Work whose
+// end the event cannot mark (a call made under the caller's own capture, whose
+// replays the plan does not see; a mark that failed) sets `unknown`.
+struct Fence {
+    cudaEvent_t ev = nullptr;
+    bool recorded = false, unknown = false;
+    cudaError_t init() { return cudaEventCreateWithFlags(&ev, cudaEventDisableTiming); }
+    void mark(cudaStream_t s) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(s, &st);
+        if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) e = cudaEventRecord(ev, s);
+        else unknown = true;
+        if (e != cudaSuccess) {
+            unknown = true;
+            cudaGetLastError();
+        } else if (st == cudaStreamCaptureStatusNone) {
+            recorded = true;
+        }
+    }
+    // before state is read; with work of unknown end the whole device
+    cudaError_t wait() const {
+        if (unknown) return cudaDeviceSynchronize();
+        return recorded ? cudaEventSynchronize(ev) : cudaSuccess;
+    }
+    // whether no work can still use the plan's memory (waits for it); a failure
+    // is not left behind for the thread's next launch check
+    bool idle() const {
+        if (unknown) return false;
+        if (!recorded || cudaEventSynchronize(ev) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    }
+    ~Fence() {
+        if (ev) cudaEventDestroy(ev);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // device buffers owned by a plan
 // ---------------------------------------------------------------------------
 // Sizes are rounded up to 256 bytes.  Allocations may come from two host
 // threads of one plan build (the lock keeps the lists consistent).  While a
 // build defers, released blocks stay reserved until the build has
-// synchronised its streams (end_defer); otherwise a release waits for the
-// device, as cudaFree would, before the block goes back to the cache.
+// synchronised its streams (end_defer); otherwise a block goes back to the
+// cache when the plan's fence has passed, and to cudaFree, which waits by
+// itself, where it cannot tell.
 struct Arena {
     std::mutex mu;
     std::shared_ptr<DevCache> cache;    // the context's, or none
+    const Fence *fence = nullptr;       // the plan's (with a cache)
     std::vector<void *> ptrs;
     std::vector<size_t> sizes;
     std::vector<std::pair<void *, size_t>> pending;
@@ -141,7 +184,6 @@ struct Arena {
             cudaError_t e = cudaMalloc(&q, want);
             if (e != cudaSuccess && cache) {
                 cudaGetLastError();
-                cudaDeviceSynchronize();
                 cache->flush();
                 e = cudaMalloc(&q, want);
             }
@@ -160,11 +202,8 @@ struct Arena {
             if (ptrs[i] == p && p) {
                 if (deferring) {
                     pending.emplace_back(p, sizes[i]);
-                } else if (cache) {
-                    cudaDeviceSynchronize();
-                    cache->give(p, sizes[i]);
                 } else {
-                    cudaFree(p);
+                    back(p, sizes[i], !fence || fence->idle());
                 }
                 ptrs[i] = nullptr;
                 bytes -= sizes[i];
@@ -174,26 +213,21 @@ struct Arena {
     void end_defer() {
         std::lock_guard<std::mutex> lock(mu);
         deferring = false;
-        for (auto &b : pending) {
-            if (cache) cache->give(b.first, b.second);
-            else cudaFree(b.first);
-        }
+        for (auto &b : pending) back(b.first, b.second, true);
         pending.clear();
+    }
+    void back(void *p, size_t n, bool idle) {
+        if (cache && idle) cache->give(p, n);
+        else cudaFree(p);
     }
     ~Arena() {
         bool any = !pending.empty();
         for (void *p : ptrs) any = any || p;
         if (!any) return;
-        if (cache) cudaDeviceSynchronize();
+        const bool idle = !fence || fence->idle();
         for (size_t i = 0; i < ptrs.size(); i++)
-            if (ptrs[i]) {
-                if (cache) cache->give(ptrs[i], sizes[i]);
-                else cudaFree(ptrs[i]);
-            }
-        for (auto &b : pending) {
-            if (cache) cache->give(b.first, b.second);
-            else cudaFree(b.first);
-        }
+            if (ptrs[i]) back(ptrs[i], sizes[i], idle);
+        for (auto &b : pending) back(b.first, b.second, idle);
     }
 };
 
@@ -367,6 +401,7 @@ struct bem_plan : bem::FmmState {
     bem_fmm_params prm{};
     int64_t N = 0, E = 0, Q = 0, nchi = 0;
     int npe = 0;
+    bem::Fence fence;                   // end of the latest call's work (outlives the arena)
     bem::Arena arena;
     bem::Tree t;
     bem::Quad q;

@@ -697,6 +697,11 @@ extern "C" int bem_field(bem_plan *P, const void *phi_dev, const void *chi_dev, 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     BEM_CUDA(cudaSetDevice(P->device));
     BEM_CUDA(cudaMemsetAsync(P->skip, 0, sizeof(int), s));
+    struct Mark {                                        // also where a call below fails
+        bem_plan *P;
+        cudaStream_t s;
+        ~Mark() { P->fence.mark(s); }
+    } mark{P, s};
     BEM_TRY(field_moments(P, phi_dev, chi_dev, s));
     const double *ph = (const double *)phi_dev, *ch = (const double *)chi_dev;
     double *u = (double *)u_dev;

@@ -1658,6 +1658,7 @@ extern "C" int bem_matvec_noalloc(bem_plan *P, int op, const void *x_dev, void *
             rc = e == cudaSuccess ? BEM_OK : cuda_fail(e, "cudaMemsetAsync", __FILE__, __LINE__);
         }
         if (rc == BEM_OK) rc = enqueue_matvec_raw(P, op, P->green, P->k, 1, s, nullptr, &w);
+        P->fence.mark(s);
     }
     cudaSetDevice(prev_dev);
     return rc;

@@ -1240,6 +1240,7 @@ int bem_batch_submit(bem_batch *b, bem_plan *P, const void *chi_dev, void *phi_d
     BEM_TRY(gm_init(g, P, (const double *)chi_dev, (double *)phi_dev, &sp, b->streams[free_slot]));
     b->used[free_slot] = 1;
     int rc = gm_run(g, false);
+    P->fence.mark(g.s);
     if (rc != BEM_OK) { b->used[free_slot] = 2; g.status = rc; g.phase = 3; }
     *slot_out = free_slot;
     return rc;
@@ -1254,8 +1255,12 @@ int bem_batch_progress(bem_batch *b, int *n_active) {
         GmSolver &g = b->slot[i];
         int rc = gm_run(g, false);
         if (rc != BEM_OK) { g.status = rc; g.phase = 3; worst = rc; }
-        if (g.phase == 3) b->used[i] = 2;
-        else act++;
+        if (g.phase == 3) {
+            b->used[i] = 2;
+            g.P->fence.mark(g.s);
+        } else {
+            act++;
+        }
     }
     if (n_active) *n_active = act;
     return worst;
@@ -1381,6 +1386,14 @@ int bem_group_solve(bem_group *G, const void *const *chis, void *const *phis, co
         gs[i].status = BEM_OK;
     }
     cudaStream_t s0 = G->s0;
+    struct Mark {                          // a solve that ends with an error may leave work behind
+        bem_group *G;
+        bool done;
+        ~Mark() {
+            if (!done)
+                for (bem_plan *P : G->plans) P->fence.mark(G->s0);
+        }
+    } mark{G, false};
     BEM_CUDA(cudaMemcpyAsync(G->d_ist, ist.data(), sizeof(int *) * n, cudaMemcpyHostToDevice, s0));
     BEM_CUDA(cudaMemcpyAsync(G->d_sc, sc.data(), sizeof(double *) * n, cudaMemcpyHostToDevice, s0));
     BEM_CUDA(cudaMemcpyAsync(G->d_chi, h_chi, sizeof(void *) * n, cudaMemcpyHostToDevice, s0));
@@ -1455,6 +1468,7 @@ int bem_group_solve(bem_group *G, const void *const *chis, void *const *phis, co
         if (gs[i].status == BEM_ENOCONV) worst = BEM_ENOCONV;
     }
     if (launches) *launches = nlaunch;
+    mark.done = true;                      // (synchronised after every launch)
     return worst;
 }
 
