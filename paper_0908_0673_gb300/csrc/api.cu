@@ -6,10 +6,13 @@
 #include <cstdarg>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
 #include <vector>
+
+#include <cuda.h>
 
 #include "bem_internal.cuh"
 
@@ -41,6 +44,54 @@ __global__ void k_set_slots(const void **xs, const void *x, void **ys, void *y) 
     ys[0] = y;
 }
 
+// Loads every kernel of the library on the current device, once per device.  By
+// default a kernel is loaded by its first launch, which synchronises the context
+// and so ends a capture that another thread has in progress; which kernels a
+// plan launches depends on its size, so no warm-up of small plans reaches them all.
+static int load_kernels(int device) {
+    static std::mutex mu;
+    static bool done[64] = {};
+    std::lock_guard<std::mutex> lock(mu);
+    if (device < 0 || device >= 64) { set_error("device %d out of range", device); return BEM_EINVAL; }
+    if (done[device]) return BEM_OK;
+    BEM_CUDA(cudaFree(nullptr));                       // the device's context
+    CUresult (*get_lib)(CUlibrary *, CUkernel) = nullptr;
+    CUresult (*count)(unsigned *, CUlibrary) = nullptr;
+    CUresult (*list)(CUkernel *, unsigned, CUlibrary) = nullptr;
+    CUresult (*get_fn)(CUfunction *, CUkernel) = nullptr;
+    CUresult (*load)(CUfunction) = nullptr;
+    const std::pair<const char *, void **> fns[] = {{"cuKernelGetLibrary", (void **)&get_lib},
+                                                    {"cuLibraryGetKernelCount", (void **)&count},
+                                                    {"cuLibraryEnumerateKernels", (void **)&list},
+                                                    {"cuKernelGetFunction", (void **)&get_fn},
+                                                    {"cuFuncLoad", (void **)&load}};
+    for (auto &f : fns) {
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        BEM_CUDA(cudaGetDriverEntryPointByVersion(f.first, f.second, 12050, cudaEnableDefault, &q));
+        if (q != cudaDriverEntryPointSuccess) { set_error("the driver has no %s", f.first); return BEM_ECUDA; }
+    }
+    for (const void *k : {(const void *)k_set_slots, kernel_of_field(), kernel_of_fmm(), kernel_of_geom(), kernel_of_gmres(),
+                          kernel_of_m2l_simt(), kernel_of_m2l_tc(), kernel_of_near_f64(), kernel_of_p2m_f64(),
+                          kernel_of_translate(), kernel_of_tree()}) {
+        cudaKernel_t kernel = nullptr;
+        BEM_CUDA(cudaGetKernel(&kernel, k));
+        CUlibrary lib = nullptr;
+        unsigned n = 0;
+        CUresult r = get_lib(&lib, (CUkernel)kernel);
+        if (r == CUDA_SUCCESS) r = count(&n, lib);
+        std::vector<CUkernel> all(n);
+        if (r == CUDA_SUCCESS) r = list(all.data(), n, lib);
+        for (unsigned i = 0; i < n && r == CUDA_SUCCESS; i++) {
+            CUfunction fn = nullptr;
+            r = get_fn(&fn, all[i]);
+            if (r == CUDA_SUCCESS) r = load(fn);
+        }
+        if (r != CUDA_SUCCESS) { set_error("loading the kernels failed (driver error %d)", (int)r); return BEM_ECUDA; }
+    }
+    done[device] = true;
+    return BEM_OK;
+}
+
 // Points the plan's input/output slots at x and y, in stream order.
 int set_slots(bem_plan *P, const void *x, void *y, cudaStream_t s) {
     (k_set_slots<<<1, 1, 0, s>>>(P->xptr, x, P->yptr, y), ::bem::count_launch());
@@ -52,9 +103,9 @@ int set_slots(bem_plan *P, const void *x, void *y, cudaStream_t s) {
 // from the plan's device slots.  The kernel sequence is captured once per
 // operator into a CUDA graph (on a private stream, since the legacy default
 // stream cannot be captured) and replayed afterwards.  Another host thread
-// can invalidate a capture in progress (its first launch of a kernel loads
-// the kernel, which synchronises the context); the partial graph is then
-// dropped, this product is enqueued kernel by kernel on s, and the capture
+// can invalidate a capture in progress (a device-wide wait, or the first launch
+// of a kernel that has to be loaded: this library's are loaded with the first
+// context, a caller's own may not be); the partial graph is then dropped, this product is enqueued kernel by kernel on s, and the capture
 // is tried again on the next call.
 int enqueue_matvec(bem_plan *P, int op, int green, double k, cudaStream_t s) {
     cudaGraphExec_t &ge = P->graph[op];
@@ -285,6 +336,7 @@ int bem_ctx_create(int device, bem_ctx **out) {
     BEM_CUDA(cudaGetDeviceCount(&n));
     if (device < 0 || device >= n) { set_error("bem_ctx_create: device %d of %d", device, n); return BEM_EINVAL; }
     BEM_CUDA(cudaSetDevice(device));
+    BEM_TRY(load_kernels(device));
     bem_ctx *c = new (std::nothrow) bem_ctx;
     if (!c) { set_error("bem_ctx_create: out of host memory"); return BEM_ENOMEM; }
     c->device = device;

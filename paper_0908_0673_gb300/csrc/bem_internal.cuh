@@ -465,6 +465,9 @@ struct bem_plan : bem::FmmState {
 };
 
 namespace bem {
+// one kernel of each translation unit (load_kernels)
+const void *kernel_of_field(), *kernel_of_fmm(), *kernel_of_geom(), *kernel_of_gmres(), *kernel_of_m2l_simt(),
+    *kernel_of_m2l_tc(), *kernel_of_near_f64(), *kernel_of_p2m_f64(), *kernel_of_translate(), *kernel_of_tree();
 // stages (each returns BEM_OK or an error code)
 int build_tree(bem_plan *P, cudaStream_t s);
 int build_geometry(bem_plan *P, cudaStream_t s);

@@ -684,6 +684,8 @@ static int launch_field(bem_plan *P, int64_t npts, const double *pts, double *u,
     return BEM_OK;
 }
 
+const void *kernel_of_field() { return (const void *)k_field_harm<float, 1>; }
+
 }  // namespace bem
 
 using namespace bem;

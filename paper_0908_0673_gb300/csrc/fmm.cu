@@ -1617,6 +1617,8 @@ static void *g_noalloc_addr[64];                     // per device ordinal, 0 un
 
 static size_t noalloc_round(size_t b) { return (b + 255) & ~(size_t)255; }
 
+const void *kernel_of_fmm() { return (const void *)k_fill; }
+
 }  // namespace bem
 
 extern "C" int bem_matvec_noalloc(bem_plan *P, int op, const void *x_dev, void *y_dev, void *cuda_stream) {

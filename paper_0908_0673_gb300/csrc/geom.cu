@@ -1572,4 +1572,6 @@ int build_correction(bem_plan *P, cudaStream_t s) {
     return BEM_OK;
 }
 
+const void *kernel_of_geom() { return (const void *)k_nodes_split; }
+
 }  // namespace bem

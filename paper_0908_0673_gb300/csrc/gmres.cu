@@ -1170,6 +1170,8 @@ static int group_capture(bem_group *G, cudaGraphExec_t *out, long long *kernels,
     return BEM_OK;
 }
 
+const void *kernel_of_gmres() { return (const void *)k_backsolve<1>; }
+
 }  // namespace bem
 
 // ---------------------------------------------------------------------------

@@ -719,4 +719,6 @@ template int launch_m2l_sy<float, 2>(bem_plan *, const float *, float *, cudaStr
 template int launch_m2l_sy<double, 1>(bem_plan *, const double *, double *, cudaStream_t);
 template int launch_m2l_sy<double, 2>(bem_plan *, const double *, double *, cudaStream_t);
 
+const void *kernel_of_m2l_simt() { return (const void *)k_m2l_gemm<1, 1>; }
+
 }  // namespace bem

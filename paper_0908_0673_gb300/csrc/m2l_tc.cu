@@ -936,4 +936,6 @@ void set_tc_attributes() {
     cudaFuncSetAttribute(k_m2l_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX);
 }
 
+const void *kernel_of_m2l_tc() { return (const void *)k_m2l_tc; }
+
 }  // namespace bem

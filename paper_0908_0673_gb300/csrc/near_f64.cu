@@ -580,4 +580,6 @@ int launch_near_pairs(bem_plan *P, int op, double kwave, const double *f, double
 template int launch_near_pairs<1>(bem_plan *, int, double, const double *, double *, cudaStream_t);
 template int launch_near_pairs<2>(bem_plan *, int, double, const double *, double *, cudaStream_t);
 
+const void *kernel_of_near_f64() { return (const void *)k_near_pairs<1, true>; }
+
 }  // namespace bem

@@ -280,4 +280,6 @@ int launch_p2m_pairs(bem_plan *P, bool dl, const double *f, double *M, cudaStrea
 template int launch_p2m_pairs<1>(bem_plan *, bool, const double *, double *, cudaStream_t);
 template int launch_p2m_pairs<2>(bem_plan *, bool, const double *, double *, cudaStream_t);
 
+const void *kernel_of_p2m_f64() { return (const void *)k_p2m_pairs<1, true, 11>; }
+
 }  // namespace bem

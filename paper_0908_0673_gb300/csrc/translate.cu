@@ -561,4 +561,6 @@ template int launch_translations<double, 2>(bem_plan *, double *, double *, cuda
 template int launch_translations<float, 1>(bem_plan *, float *, float *, cudaStream_t, cudaEvent_t *);
 template int launch_translations<float, 2>(bem_plan *, float *, float *, cudaStream_t, cudaEvent_t *);
 
+const void *kernel_of_translate() { return (const void *)k_m2l_tables; }
+
 }  // namespace bem

@@ -884,4 +884,6 @@ int build_radii_lists(bem_plan *P, cudaStream_t s) {
     return BEM_OK;
 }
 
+const void *kernel_of_tree() { return (const void *)k_close_ptr; }
+
 }  // namespace bem

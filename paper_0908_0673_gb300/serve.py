@@ -148,9 +148,8 @@ class CudaEngine:
 
     def _warmup(self):
         # One tiny solve of every element type and Green's function, on this
-        # thread, before set-up threads exist: the first launch of each kernel
-        # loads it, and a load in one thread invalidates a graph capture that
-        # another thread has in progress.
+        # thread, before set-up threads exist: the tables that the library fills
+        # once per device, and the memory of its kernels' first launches.
         for et in (I.TRI3, I.TRI6):
             m = I.geodesic(2, et)
             for green, k in ((bem.BEM_LAPLACE, 0.0), (bem.BEM_HELMHOLTZ, 1.0)):
