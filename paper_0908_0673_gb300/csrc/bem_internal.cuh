@@ -39,6 +39,10 @@ extern thread_local long long *tl_capture_count;
         if (r_ != BEM_OK) return r_;                                        \
     } while (0)
 #define BEM_LAUNCH_CHECK() BEM_CUDA(cudaGetLastError())
+// After cudaMemcpy or cudaMemcpyToSymbol from pageable host memory: a copy of up
+// to 64 KB returns when it has been staged, before it is in device memory, and
+// the streams whose kernels read it next do not wait for the default stream.
+#define BEM_COPIES_DONE() BEM_CUDA(cudaStreamSynchronize(cudaStreamLegacy))
 
 constexpr int QBITS = 21;   // Morton bits per axis
 constexpr int PMAX = 20;    // largest supported expansion order

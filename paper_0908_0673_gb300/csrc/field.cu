@@ -629,6 +629,7 @@ int field_prepare(bem_plan *P) {
         if (have[dev] <= p) {
             const std::vector<double> t = harmonic_table(have[dev], p);
             BEM_CUDA(cudaMemcpyToSymbol(g_harm, t.data(), sizeof(double) * t.size(), sizeof(double) * harm_size(have[dev])));
+            BEM_COPIES_DONE();
             have[dev] = p + 1;
         }
     }

@@ -432,6 +432,7 @@ int build_near_items(bem_plan *P) {
         BEM_CUDA(cudaMemcpy(P->near_items[v], sorted.data(), sizeof(int2) * sorted.size(), cudaMemcpyHostToDevice));
         P->near_nitems[v] = (int)items.size();
     }
+    BEM_COPIES_DONE();
     return BEM_OK;
 }
 
@@ -1169,6 +1170,7 @@ static int init_shape_table(int device) {
         }
     }
     BEM_CUDA(cudaMemcpyToSymbol(c_Lq, Lq, sizeof(Lq)));
+    BEM_COPIES_DONE();
     done[device] = true;
     return BEM_OK;
 }
@@ -1190,6 +1192,7 @@ static int wave_table(int device, const float **out) {
         void *p = nullptr;
         BEM_CUDA(cudaGetSymbolAddress(&p, g_wave));
         BEM_CUDA(cudaMemcpy(p, t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice));
+        BEM_COPIES_DONE();
         addr[device] = (const float *)p;
     }
     *out = addr[device];

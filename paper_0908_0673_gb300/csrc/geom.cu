@@ -209,6 +209,7 @@ static int init_rule_tables(int device) {
     std::vector<float2> g01(gx.size());
     for (size_t i = 0; i < gx.size(); i++) g01[i] = make_float2((float)(0.5 * (1.0 + gx[i])), (float)(0.5 * gw[i]));
     BEM_CUDA(cudaMemcpyToSymbol(c_gl01f, g01.data(), sizeof(float2) * g01.size()));
+    BEM_COPIES_DONE();
     done[device] = true;
     return BEM_OK;
 }

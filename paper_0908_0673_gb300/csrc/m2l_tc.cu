@@ -618,6 +618,7 @@ int build_m2l_sym(bem_plan *P, const std::vector<int> &pair_cls, const std::vect
     BEM_TRY(up(&P->sy_kh, khc));
     BEM_TRY(up(&P->sy_dl, dlc));
     BEM_TRY(up(&P->sy_sig_u, P->sy_hsig));
+    BEM_COPIES_DONE();
     return BEM_OK;
 }
 

@@ -528,6 +528,7 @@ int circle_table(int device, const float4 **out) {
         void *p = nullptr;
         BEM_CUDA(cudaGetSymbolAddress(&p, g_circle));
         BEM_CUDA(cudaMemcpy(p, t.data(), sizeof(float4) * ND_TAB, cudaMemcpyHostToDevice));
+        BEM_COPIES_DONE();
         addr[device] = (const float4 *)p;
     }
     *out = addr[device];
