@@ -162,7 +162,10 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
         }
         sStep[j] = v;
     }
-    if (warp == 0) tc::tmem_alloc(sTmem, 512);
+    if (warp == 0) {
+        __syncwarp();
+        tc::tmem_alloc(sTmem, 512);
+    }
     tc::tc_fence_before_sync();
     __syncthreads();
     tc::tc_fence_after_sync();
@@ -322,6 +325,10 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
                 // a copy in flight when a wait gave up: let it land before exit
                 if (!tc::mbar_wait_bounded(bfull, nbulk & 1u, TC_WAIT)) *sAbort = 1;
             }
+            // every MMA issued has completed before the accumulator is released, also
+            // after a wait that gave up (a commit covers its own thread's MMAs only)
+            tc::mma_commit(fin);
+            if (!tc::mbar_wait_bounded(fin, 0, TC_WAIT)) *sAbort = 1;
         }
         __syncwarp();
     } else {
@@ -415,17 +422,14 @@ __global__ void __launch_bounds__(TC_T, 1) k_m2l_tc(const __grid_constant__ TcAr
         tc::cp_async_wait<0>();
         if (pend && ok) convert(it - 1, pvm);
     }
-    // every MMA issued has completed before the accumulator is released
-    __syncthreads();
-    if (tid == 0) {
-        tc::mma_commit(fin);
-        if (!tc::mbar_wait_bounded(fin, 0, TC_WAIT)) *sAbort = 1;
-        if (*sAbort) atomicExch(a.err, 1);
-    }
     tc::tc_fence_before_sync();
     __syncthreads();
     tc::tc_fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, 512);
+    if (tid == 0 && *sAbort) atomicExch(a.err, 1);
+    if (warp == 0) {
+        __syncwarp();                                   // allocation and release are for a converged warp
+        tc::tmem_dealloc(tmem, 512);
+    }
 }
 
 // Class-matrix images of every canonical class: element e of a plane (in the
