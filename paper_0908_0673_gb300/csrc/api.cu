@@ -181,8 +181,8 @@ static int plan_setup(bem_plan *P, cudaStream_t s) {
         BEM_CUDA(cudaMemcpyAsync(P->elems, m->elems.data(), sizeof(int) * P->E * P->npe, cudaMemcpyHostToDevice, s));
         BEM_CUDA(cudaMemcpyAsync(P->chi, m->chi.data(), sizeof(int) * P->E * P->npe, cudaMemcpyHostToDevice, s));
     }
-    BEM_TRY(A.alloc(&P->istate, 4));
-    BEM_CUDA(cudaMemsetAsync(P->istate, 0, sizeof(int) * 4, s));
+    BEM_TRY(A.alloc(&P->istate, 6));
+    BEM_CUDA(cudaMemsetAsync(P->istate, 0, sizeof(int) * 6, s));
     P->skip = P->istate;
     P->dev_err = P->istate + 3;
     // stage timers (wall clock, stream synchronised at every boundary)

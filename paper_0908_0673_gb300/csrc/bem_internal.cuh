@@ -461,7 +461,7 @@ struct bem_plan : bem::FmmState {
     double *scal = nullptr;             // device scalars
     double *hostbuf = nullptr;          // pinned read-back of GMRES scalars
     void **gm_slot = nullptr;           // device pointer slots of the current solve: [0] chi, [1] x
-    int *istate = nullptr;              // device ints: [0] converged flag, [1] steps in cycle
+    int *istate = nullptr;              // device ints of a solve (GmState::st in gmres.cu); [3] is dev_err
     int gm_restart = 0;
     cudaGraphExec_t cycle_graph = nullptr;
     int capture_retries = 0;            // captures invalidated by other host threads

@@ -196,8 +196,7 @@ __global__ void k_nrm2_final(const double *__restrict__ partial, double *out, co
     if (threadIdx.x == 0) *out = sqrt(s);
 }
 
-// r = b - r  (r holds A x on entry)
-// r = b - r and the partial sums of |r|^2
+// r = b - r (r holds A x on entry) and the partial sums of |r|^2
 template <int C>
 __global__ void k_resid_nrm2(int n, const double *__restrict__ b, double *r, double *partial, const int *__restrict__ skip) {
     if (skip && *skip) return;
@@ -273,7 +272,12 @@ static int set_scalar(double *p, double v, cudaStream_t s) {
 struct GmState {
     // scalars: [0] ||b||, [1] beta, [2] |g_{j+1}| / ||b||, [3] tol, [4] ||w||
     double *sc;
-    int *st;        // [0] converged-in-cycle flag, [1] steps done in cycle
+    // [0] stop flag (the cycle's kernels return at once; set by the step that
+    // converges), [1] steps done in the cycle, [2] halt (the solve has ended:
+    // every kernel of it returns), [4 + (j & 1)] the stop flag as step j finds it,
+    // written by the step before: a step's last kernel raises [0] while its other
+    // blocks start, so they read this word instead ([3] is the plan's dev_err)
+    int *st;
     double *H;      // [(m+1)][m] complex pairs
     double *cs, *sn, *g, *y;
     double *hcol;   // [m+1] first Gram-Schmidt pass coefficients
@@ -302,7 +306,11 @@ template <int C>
 __global__ void __launch_bounds__(GM_T) k_step_end(int n, GmState S, int m, int j, const double *__restrict__ npart, int nblk,
                                                    const double *__restrict__ w, double *vout,
                                                    const double *__restrict__ dinv, double *z) {
-    if (S.st[0]) return;
+    int *const next = S.st + 4 + ((j + 1) & 1);
+    if (S.st[4 + (j & 1)]) {                          // no block of this launch writes that word
+        if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) *next = 1;
+        return;
+    }
     __shared__ double nrm, sc[GM_MAXV], ss[2 * GM_MAXV], Hc[2 * (GM_MAXV + 1)];
     const int tid = threadIdx.x;
     if (blockIdx.x + 1 < gridDim.x) {
@@ -369,7 +377,9 @@ __global__ void __launch_bounds__(GM_T) k_step_end(int n, GmState S, int m, int 
         const double est = hypot(g1r, g1i) / bnorm;
         S.sc[2] = est;
         S.st[1] = j + 1;
-        if (est <= tol || wn == 0.0) S.st[0] = 1;
+        const bool stop = est <= tol || wn == 0.0;
+        if (stop) S.st[0] = 1;
+        *next = stop;
     }
     __syncthreads();
     for (int i = tid; i < 2 * (j + 2); i += GM_T) Hg[i] = Hc[i];
@@ -431,7 +441,7 @@ __global__ void k_cycle_begin(int n, GmState S, int m, double *v0, const double 
     const bool halted = S.st[2] != 0;
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) {
-            S.st[0] = S.st[2];
+            S.st[0] = S.st[4] = S.st[5] = S.st[2];
             S.st[1] = 0;
             xptr[0] = z;
             yptr[0] = w;
@@ -450,6 +460,8 @@ __global__ void k_cycle_begin(int n, GmState S, int m, double *v0, const double 
         z[(size_t)r * C + c] = di * v;
     }
 }
+
+// pointer slots of a solve: [0] chi (Neumann data), [1] x (the solution)
 __global__ void k_set_ptrs(void **slot, const void *chi, void *x) {
     slot[0] = (void *)chi;
     slot[1] = x;
@@ -458,7 +470,7 @@ __global__ void k_set_ptrs_tab(void **slot, const void *const *chi_tab, void *co
     slot[0] = (void *)chi_tab[i];
     slot[1] = x_tab[i];
 }
-// product input / output slots from a solve slot
+// x = 0 through a solve slot
 __global__ void k_zero_slot(void *const *slot, size_t n, const int *__restrict__ skip) {
     if (skip && *skip) return;
     double *x = (double *)*slot;
