@@ -283,6 +283,7 @@ struct Tree {
     int *eb = nullptr, *ee = nullptr;   // element range in owner order
     double *cx = nullptr, *cy = nullptr, *cz = nullptr, *r = nullptr;
     float4 *fbox = nullptr;             // float32 centre and radius of each box (search filters)
+    int *reach = nullptr;               // box_reach of each box
     int *leaves = nullptr;              // box ids of the leaves
     int *near_ptr = nullptr, *near_idx = nullptr;
     int *inter_ptr = nullptr, *inter_idx = nullptr;

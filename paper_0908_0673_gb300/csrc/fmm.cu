@@ -1137,7 +1137,7 @@ Tabs tabs_of(const bem_plan *P) {
 TreeView view_of(const bem_plan *P) {
     const Tree &t = P->t;
     return TreeView{t.level, t.ix, t.iy, t.iz, t.parent, t.child0, t.nchild, t.nb, t.ne, t.eb, t.ee, t.leaves,
-                    t.near_ptr, t.near_idx, t.inter_ptr, t.inter_idx, t.node_perm, t.cx, t.cy, t.cz, t.r,
+                    t.near_ptr, t.near_idx, t.inter_ptr, t.inter_idx, t.node_perm, t.reach, t.cx, t.cy, t.cz, t.r,
                     t.tx, t.ty, t.tz, t.side};
 }
 

@@ -18,7 +18,7 @@ __device__ __forceinline__ int order_of(const Tabs &tb, int level) { return tb.l
 
 struct TreeView {
     const int *level, *ix, *iy, *iz, *parent, *child0, *nchild, *nb, *ne, *eb, *ee, *leaves;
-    const int *near_ptr, *near_idx, *inter_ptr, *inter_idx, *node_perm;
+    const int *near_ptr, *near_idx, *inter_ptr, *inter_idx, *node_perm, *reach;
     const double *cx, *cy, *cz, *r, *tx, *ty, *tz;
     double side;
 };

@@ -398,14 +398,14 @@ __global__ void __launch_bounds__(MG_T, W == 1 ? 3 : 2) k_m2l_gemm(const __grid_
 // and by 2^(-reach |a|) where its points reach far beyond its edge
 template <class R, int C>
 __global__ void __launch_bounds__(256) k_m2l_words(int np, int ldq, const unsigned short *__restrict__ fwd,
-                                                   const int *__restrict__ mexp, const int *__restrict__ level,
-                                                   const double *__restrict__ radius, double side, const R *__restrict__ M, float *__restrict__ Mq, int *__restrict__ Eb,
+                                                   const int *__restrict__ mexp, const int *__restrict__ reach_of,
+                                                   const R *__restrict__ M, float *__restrict__ Mq, int *__restrict__ Eb,
                                                    const int *__restrict__ skip) {
     if (skip && *skip) return;
     constexpr int WC = (sizeof(R) == 8 ? 2 : 1) * C;
     const size_t box = blockIdx.x;
     const R *m = M + box * np * C;
-    const int reach = sizeof(R) == 8 ? box_reach(radius[box], side, level[box]) : 0;
+    const int reach = sizeof(R) == 8 ? __ldg(reach_of + box) : 0;
     auto moment = [&](int i) -> R {                       // i = coefficient x C + component
         if constexpr (sizeof(R) == 8)
             if (reach) return scalbn(m[i], -reach * (__ldg(mexp + i / C) >> 24));
@@ -673,7 +673,7 @@ int launch_m2l_sy(bem_plan *P, const R *M, R *L, cudaStream_t s) {
     a.skip = P->skip;
     const size_t sm = mg_smem(W, C, a.np);
     if (P->sy_ntile > 0)
-        (k_m2l_words<R, C><<<t.nbox, 256, 0, s>>>(a.np, a.ldq, P->sy_fwd, P->sy_mexp, t.level, t.r, t.side, M, P->sg_Mq,
+        (k_m2l_words<R, C><<<t.nbox, 256, 0, s>>>(a.np, a.ldq, P->sy_fwd, P->sy_mexp, t.reach, M, P->sg_Mq,
                                                   P->sg_E, P->skip),
          ::bem::count_launch());
     // one run of targets at a time: its tiles, then the gather of its targets

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(PP_T, KM <= 11 && C == 1 ? 2 : 1) k_p2m_pairs(
     for (int w = 0; w < PP_T / 32; w++) E = max(E, wexp[w]);
     E = min(E, 2046);                                   // an infinity or NaN carries itself
     // offsets and normals in units of the leaf's edge x 2^reach
-    const int es = ilogb(tv.side), reach = box_reach(tv.r[b], tv.side, tv.level[b]);
+    const int es = ilogb(tv.side), reach = tv.reach[b];
     float uh, ul;                                       // 2^es / unit: the plan's pairs hold offsets x 2^-es
     df_split(1.0 / scalbn(tv.side, reach - tv.level[b] - es), uh, ul);
     // row of this thread, in order of m + n (rows of a warp have about the same length)

@@ -386,11 +386,8 @@ int build_m2l_classes(bem_plan *P) {
     BEM_CUDA(cudaMemcpy(ip.data(), t.inter_ptr, sizeof(int) * (t.nbox + 1), cudaMemcpyDeviceToHost));
     if (t.n_inter) BEM_CUDA(cudaMemcpy(ii.data(), t.inter_idx, sizeof(int) * t.n_inter, cudaMemcpyDeviceToHost));
     std::vector<int> reach(t.nbox, 0);
-    if (P->prm.precision == BEM_F64) {
-        std::vector<double> r(t.nbox);
-        BEM_CUDA(cudaMemcpy(r.data(), t.r, sizeof(double) * t.nbox, cudaMemcpyDeviceToHost));
-        for (int b = 0; b < t.nbox; b++) reach[b] = box_reach(r[b], t.side, lev[b]);
-    }
+    if (P->prm.precision == BEM_F64)
+        BEM_CUDA(cudaMemcpy(reach.data(), t.reach, sizeof(int) * t.nbox, cudaMemcpyDeviceToHost));
     const bool helm = P->green == BEM_HELMHOLTZ;
     const bool by_level = helm || P->prm.p_min > 0;   // the target level enters the key
     // Classes are numbered in order of first appearance over the pairs in list

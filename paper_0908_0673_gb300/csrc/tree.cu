@@ -657,9 +657,12 @@ __device__ __forceinline__ bool separated(const ListArgs &a, int b, int n) {
 }
 
 __global__ void k_box_floats(int nbox, const double *__restrict__ cx, const double *__restrict__ cy,
-                             const double *__restrict__ cz, const double *__restrict__ r, float4 *fbox) {
+                             const double *__restrict__ cz, const double *__restrict__ r, const int *__restrict__ level,
+                             double side, float4 *fbox, int *reach) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbox) fbox[b] = make_float4((float)cx[b], (float)cy[b], (float)cz[b], (float)r[b]);
+    if (b >= nbox) return;
+    fbox[b] = make_float4((float)cx[b], (float)cy[b], (float)cz[b], (float)r[b]);
+    reach[b] = box_reach(r[b], side, level[b]);
 }
 
 // Walks the parent's near list for box b; when `write`, stores the entries.
@@ -810,7 +813,9 @@ int build_radii_lists(bem_plan *P, cudaStream_t s) {
         BEM_LAUNCH_CHECK();
     }
     BEM_TRY(A.alloc(&t.fbox, t.nbox));
-    (k_box_floats<<<(t.nbox + 255) / 256, 256, 0, s>>>(t.nbox, t.cx, t.cy, t.cz, t.r, t.fbox), ::bem::count_launch());
+    BEM_TRY(A.alloc(&t.reach, t.nbox));
+    (k_box_floats<<<(t.nbox + 255) / 256, 256, 0, s>>>(t.nbox, t.cx, t.cy, t.cz, t.r, t.level, t.side, t.fbox, t.reach),
+     ::bem::count_launch());
     // lists, level by level; level-l lists only read level < l lists
     BEM_TRY(A.alloc(&t.near_ptr, t.nbox + 1));
     BEM_TRY(A.alloc(&t.inter_ptr, t.nbox + 1));
