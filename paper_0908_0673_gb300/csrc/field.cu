@@ -608,6 +608,11 @@ std::vector<double> harmonic_table(int d0, int d1) {
 
 }  // namespace
 
+template <int C>
+static size_t field_smem(int p) {
+    return FW * (((size_t)(p + 1) * 32 * C + (sizeof(WarpShared<C>) + 7) / 8) * sizeof(double));
+}
+
 // The table of degrees <= p on the plan's device (filled once per device and
 // degree, under a lock) and the workspaces of a field evaluation.
 int field_prepare(bem_plan *P) {
@@ -633,6 +638,10 @@ int field_prepare(bem_plan *P) {
             have[dev] = p + 1;
         }
     }
+    // one value for every order: plans of different orders evaluate fields on
+    // different threads, and one must not lower another's limit before its launch
+    BEM_CUDA(cudaFuncSetAttribute(k_field<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)field_smem<1>(PMAX)));
+    BEM_CUDA(cudaFuncSetAttribute(k_field<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)field_smem<2>(PMAX)));
     Arena &A = P->arena;
     BEM_TRY(A.alloc(&P->fd_str, 2 * (size_t)P->Q * C));
     BEM_TRY(A.alloc(&P->fd_elem, (size_t)P->E * (18 + 12 * C)));
@@ -640,11 +649,6 @@ int field_prepare(bem_plan *P) {
     BEM_TRY(A.alloc((float4 **)&P->fd_fcen, (size_t)P->E));
     BEM_TRY(A.alloc(&P->fd_harm, (size_t)P->t.nbox * coef_count(p) * 2 * C));
     return BEM_OK;
-}
-
-template <int C>
-static size_t field_smem(int p) {
-    return FW * (((size_t)(p + 1) * 32 * C + (sizeof(WarpShared<C>) + 7) / 8) * sizeof(double));
 }
 
 template <class R, int C>
@@ -678,7 +682,6 @@ static int launch_field(bem_plan *P, int64_t npts, const double *pts, double *u,
     a.fcen = (const float4 *)P->fd_fcen;
     a.err = P->dev_err;
     const size_t sm = field_smem<C>(p);
-    BEM_CUDA(cudaFuncSetAttribute(k_field<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int64_t nblk = (npts + FW - 1) / FW;
     if (nblk > 0) (k_field<C><<<(unsigned)nblk, FW * 32, sm, s>>>(npts, pts, u, a), ::bem::count_launch());
     BEM_LAUNCH_CHECK();
