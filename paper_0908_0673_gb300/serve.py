@@ -89,25 +89,23 @@ class EngineError(RuntimeError):
 
 # Peak device bytes per geometric node of a plan with the default parameters
 # (p = 10, leaf sizes 32-128, eta = 2, Duffy order 12, tau = 2) and a GMRES(30)
-# basis, by (Green's function, precision).  The correction matrix dominates
-# (a few hundred entries per row for each of D and S); then the translation
-# tables, the diagonal's higher-order buffers (held while the plan's own order
-# is built beside them: both sets of buffers, the stored P2M weights included,
-# exist at the set-up peak) and the Krylov basis.  The values bound the
-# measured peaks (9-28 kB per node on spheres, ellipsoids and graded cubes of
-# 1k-18k quadratic elements, before the two orders overlapped) with a margin;
-# the GPU tests check the bound.  The M2L row buffers (rows are computed and
-# gathered in runs of targets) are capped: the diagonal's order at 128 MiB and
-# the plan's own at the larger of 128 MiB and 14 KiB per node, the class images
-# of the SIMT form at 48 MiB and 4 KiB per node.  The fixed part holds the two
-# 128 MiB and 64 MiB of small tables.
+# basis, by (Green's function, precision), beside a fixed part.  Per node: the
+# correction matrix (a few hundred entries per row for each of D and S) and its
+# set-up temporaries, up to 14 KiB of M2L rows, up to 4 KiB of class images for
+# each of the two orders (the diagonal's buffers are held while the plan's own
+# order is built beside them), the permuted moments, the stored P2M weights, the
+# field workspaces and the Krylov basis.  Fixed: 128 MiB of M2L rows and 48 MiB of
+# class images for each order, which the per-node shares only add to, and 64 MiB
+# of small tables.  Measured above the fixed part on spheres, ellipsoids and cubes
+# of 500 to 200,000 elements, 3 and 6 nodes each, leaf sizes 32 to 128: at most
+# 42.5, 39.0, 53.5 and 47.0 kB per node; the values leave 15 % beyond them.
 _BYTES_PER_NODE = {
-    (bem.BEM_LAPLACE, bem.BEM_F64): 36_000,
-    (bem.BEM_LAPLACE, bem.BEM_MIXED): 36_000,
-    (bem.BEM_HELMHOLTZ, bem.BEM_F64): 44_000,
-    (bem.BEM_HELMHOLTZ, bem.BEM_MIXED): 44_000,
+    (bem.BEM_LAPLACE, bem.BEM_F64): 50_000,
+    (bem.BEM_LAPLACE, bem.BEM_MIXED): 46_000,
+    (bem.BEM_HELMHOLTZ, bem.BEM_F64): 62_000,
+    (bem.BEM_HELMHOLTZ, bem.BEM_MIXED): 55_000,
 }
-_BYTES_FIXED = (64 + 2 * 128) << 20
+_BYTES_FIXED = (64 + 2 * 128 + 2 * 48) << 20
 
 
 def estimate_peak_footprint(n_nodes: int, green: int, precision: int) -> int:
