@@ -45,7 +45,7 @@ METRIC = "FMM-BEM matvecs/s & served solves/s, p50/p99 latency vs plain FP64 at 
 WORKLOAD = "cube45-tri6-laplace"
 SOURCE = (0.2, -0.1, 0.3)
 FLOPS_PER_PAIR = {"A": 20.0, "B": 11.0}   # near-field kernel, Laplace double / single layer
-FLOPS_PER_PAIR_PAIRS = 190.0              # double layer in float32 pairs (float64 plans), float32 flops
+FLOPS_PER_PAIR_PAIRS = 214.0              # double layer in float32 pairs (float64 plans), float32 flops
 # DRAM bytes (read + write) per launch of the dominant kernels, from one ncu
 # capture of this workload (the command is in profiles/); reported while the
 # kernel's source file is unchanged, null otherwise.
@@ -637,7 +637,7 @@ def main():
                 "traffic": ncu_traffic("near_l2p") if kind == 0 else None, "traffic_unit": "bytes per launch",
                 "peak_source": "measured FP32 FMA throughput (bem_measure_peak)",
                 "work": f"{st['near_pairs']} target-source pairs x {per_pair:.0f} flops"
-                        + ("" if kind == 0 else " (95 float32 operations of a pair sum, two flops each)")}
+                        + ("" if kind == 0 else " (107 float32 operations of a pair sum, two flops each)")}
     elif dom == "m2l":
         cpp6 = math.comb(10 + 6, 6)
         flops = st["n_inter"] * 2.0 * cpp6

@@ -55,8 +55,23 @@ extern "C" {
 #define BEM_LAPLACE 0     /* G = 1/(4 pi R), Eq. 1a */
 #define BEM_HELMHOLTZ 1   /* G = exp(jkR)/(4 pi R), Eq. 1b, time factor exp(-j omega t) */
 
-#define BEM_F64 0         /* every stage in float64 */
-#define BEM_MIXED 1       /* near field and expansions in float32, Krylov in float64 */
+/* Precision of a plan.
+ *   BEM_F64    vectors, geometry, correction, M2M, L2L, L2P, sums between stages
+ *              and the Krylov space in float64.  The near field, P2M and M2L
+ *              (positions, strengths, powers, class matrices, products and their
+ *              sums, for the diagonal too) run on unevaluated pairs of float32,
+ *              48 bits at a power-of-two scale taken from the largest value of
+ *              the block, leaf or source box: a product differs from one with
+ *              every stage in float64 by 6e-15 to 5e-14 of its norm (measured,
+ *              largest entry 3.6e-13).  Against that scale values below 2^-75
+ *              keep 24 bits and values below 2^-126, and subnormal strengths,
+ *              count as zero; an infinite strength gives NaN.  (The Helmholtz
+ *              near field of plans with k x 8 root sides above 6,430
+ *              stays in float64.)
+ *   BEM_MIXED  near field and expansions in float32, the correction's values in
+ *              float32 with sums as pairs, Krylov space in float64. */
+#define BEM_F64 0
+#define BEM_MIXED 1
 
 #define BEM_OP_A 0        /* y = C x - D x  (x indexed by node) */
 #define BEM_OP_B 1        /* y = -S x       (x indexed by chi index) */

@@ -241,8 +241,9 @@ static void launch_p2m_stored(int nleaf, int np, const TreeView &tv, const float
 }
 
 // ---------------------------------------------------------------------------
-// near field (regular rule over the near-list boxes), float64 arithmetic: Helmholtz plans whose phases exceed the table of the float32-pair
-// kernel (near_f64.cu), which takes every other float64 product
+// near field (regular rule over the near-list boxes), float64 arithmetic:
+// Helmholtz plans whose phases exceed the table of the float32-pair kernel
+// (near_f64.cu), which takes every other float64 product
 // ---------------------------------------------------------------------------
 constexpr int NF_T = 256, NF_TGT = 64, NF_SL = NF_T / NF_TGT, NF_TILE = 256;
 

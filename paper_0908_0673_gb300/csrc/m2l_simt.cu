@@ -311,7 +311,10 @@ __global__ void __launch_bounds__(MG_T, W == 1 ? 3 : 2) k_m2l_gemm(const __grid_
                 const float4 *t = T + (k0 - off) * TS + (tail ? 0 : g * VB);
                 const float *m = M + (k0 - off) * KS;
                 const unsigned char *par = sPar + k0;
-#define MG_RUN(N_)                                                                                             case N_:                                                                                                       if constexpr (N_ <= NB) run_columns<W, C, N_, NA>(nc, cs, step, t, m, par, s0, s1, acc);                   break;
+#define MG_RUN(N_)                                                                                              \
+    case N_:                                                                                                    \
+        if constexpr (N_ <= NB) run_columns<W, C, N_, NA>(nc, cs, step, t, m, par, s0, s1, acc);                \
+        break;
                 switch (nb) {
                     MG_RUN(1) MG_RUN(2) MG_RUN(3) MG_RUN(4) MG_RUN(5) MG_RUN(6) MG_RUN(7) MG_RUN(8) MG_RUN(9)
                 default: break;

@@ -846,9 +846,6 @@ int build_sym_tables(bem_plan *P, cudaStream_t s) {
             for (int h = 0; h < np; h++) fq[(size_t)q * np + h] = fwd[(size_t)(q * 8) * np + h] & 0x7fff;
         BEM_TRY(up(&P->sy_fwdq, fq));
         const int nw = ldp / 32;
-    const int colB = 512 - ldp;                         // first column of the second accumulator
-    const int gs = colB < ldp ? colB / 32 : 0;          // first group of the first one that the second shares
-    const int novl = colB < ldp ? nw - gs : 0;          // groups the two accumulators share
         std::vector<unsigned> sg(48 * (size_t)nw, 0u);
         for (int sig = 0; sig < 48; sig++)
             for (int h = 0; h < np; h++)

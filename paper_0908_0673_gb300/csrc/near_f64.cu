@@ -23,16 +23,16 @@
 // grid 2^-44, so the differences of two H and of two L1 are exact float32
 // subtractions and the pair's offset keeps its 48 bits however close the two
 // points are: seven operations per component (two words, four operations, left
-// an error of 2^-45 of the near field's extent, 1e-10 of a product).  Strengths are scaled by a power of two taken from the
-// largest one the block reads; both scales return in float64 at the end.
+// an error of 2^-45 of the near field's extent, 1e-10 of a product).  Strengths
+// are scaled by a power of two taken from the largest one the block reads; both
+// scales return in float64 at the end.
 //
 // Layout as the float32 kernel (fmm.cu): a work item is one leaf and up to 32
 // of its targets; G = ceil(targets / U) target groups x (256 / G) source
 // slices, sources staged in shared memory in rounds of 512.  A cluster of 1 to
 // 8 blocks shares an item (each takes a contiguous share of its sources) and
-// block 0 adds the shares in rank order through
-// distributed shared memory: small trees have fewer items than the chip has
-// SMs.  Deterministic for a given plan.
+// block 0 adds the shares in rank order through distributed shared memory: small
+// trees have fewer items than the chip has SMs.  Deterministic for a given plan.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
