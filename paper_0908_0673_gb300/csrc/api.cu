@@ -221,7 +221,7 @@ static int plan_setup(bem_plan *P, cudaStream_t s) {
     // host work beside the correction's enqueue (which waits once for the pair
     // count): the M2L offset classes on a second thread, the near-field work
     // items on this one once the correction is enqueued (the lists were
-    // synchronised above); device copies on the null stream, which the plan's
+    // synchronised above); downloads on the default stream, whose work the plan's
     // non-blocking streams do not wait for
     int host_rc = BEM_OK;
     std::string host_err;
@@ -236,7 +236,7 @@ static int plan_setup(bem_plan *P, cudaStream_t s) {
         cudaError_t e = cudaEventRecord(ev[1], s);
         if (e != cudaSuccess) rc = cuda_fail(e, "cudaEventRecord", __FILE__, __LINE__);
     }
-    if (rc == BEM_OK) rc = build_near_items(P);
+    if (rc == BEM_OK) rc = build_near_items(P, s2);
     worker.join();
     P->setup_ms[4] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - h0).count();
     if (rc == BEM_OK && host_rc != BEM_OK) {

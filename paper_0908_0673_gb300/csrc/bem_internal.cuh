@@ -503,7 +503,7 @@ template <class R, int C>
 int launch_m2m(bem_plan *P, R *M, cudaStream_t s, int lmin = 0);
 int field_prepare(bem_plan *P);
 int field_moments(bem_plan *P, const void *phi, const void *chi, cudaStream_t s);
-int build_near_items(bem_plan *P);
+int build_near_items(bem_plan *P, cudaStream_t s);
 int diagonal_prepare(bem_plan *P, cudaStream_t s);
 int diagonal_product(bem_plan *P, cudaStream_t s);
 int diagonal_finish(bem_plan *P, cudaStream_t s);

@@ -363,8 +363,10 @@ __host__ __device__ constexpr int nf2_stage(int C, bool TAB) { return nf2_tile(C
 // Work items of the near field: one per (leaf, pass of up to NF2_SLOTS targets,
 // ND_SLOTS in float64 plans), ordered by decreasing pair count (targets x near sources, ties in
 // leaf order), so the largest blocks start first and the last wave is made of
-// the smallest.  Each target is summed by one block whatever the order.
-int build_near_items(bem_plan *P) {
+// the smallest.  Each target is summed by one block whatever the order.  Uploads
+// go to the stream of the first product (the diagonal's; pageable sources, staged
+// before the calls return).
+int build_near_items(bem_plan *P, cudaStream_t s) {
     const Tree &t = P->t;
     std::vector<int> nptr(t.nbox + 1), nidx(std::max<int64_t>(1, t.n_near)), nb(t.nbox), ne(t.nbox), eb(t.nbox),
         ee(t.nbox), lv(t.nleaf);
@@ -397,9 +399,9 @@ int build_near_items(bem_plan *P) {
         }
         BEM_TRY(P->arena.alloc(&P->leaf_near_ptr, ptr.size()));
         BEM_TRY(P->arena.alloc(&P->leaf_near_idx, idx.size()));
-        BEM_CUDA(cudaMemcpy(P->leaf_near_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice));
+        BEM_CUDA(cudaMemcpyAsync(P->leaf_near_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, s));
         if (!idx.empty())
-            BEM_CUDA(cudaMemcpy(P->leaf_near_idx, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice));
+            BEM_CUDA(cudaMemcpyAsync(P->leaf_near_idx, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice, s));
     }
     int64_t pairs = 0;
     std::vector<int64_t> src(t.nleaf);
@@ -430,10 +432,9 @@ int build_near_items(bem_plan *P) {
         std::vector<int2> sorted(std::max<size_t>(1, items.size()));
         for (size_t i = 0; i < ord.size(); i++) sorted[i] = items[ord[i]];
         BEM_TRY(P->arena.alloc(&P->near_items[v], sorted.size()));
-        BEM_CUDA(cudaMemcpy(P->near_items[v], sorted.data(), sizeof(int2) * sorted.size(), cudaMemcpyHostToDevice));
+        BEM_CUDA(cudaMemcpyAsync(P->near_items[v], sorted.data(), sizeof(int2) * sorted.size(), cudaMemcpyHostToDevice, s));
         P->near_nitems[v] = (int)items.size();
     }
-    BEM_COPIES_DONE();
     return BEM_OK;
 }
 
