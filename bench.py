@@ -51,11 +51,11 @@ FLOPS_PER_PAIR_PAIRS = 214.0              # double layer in float32 pairs (float
 # kernel's source file is unchanged, null otherwise.
 NCU_TRAFFIC = {
     # k_near_f32 + k_l2p (order-10 products)
-    "near_l2p": {"bytes": 6426624 + 3205632, "source": "paper_0908_0673_gb300/csrc/fmm.cu",
-                 "sha256": "12510e466fad0650e9b1305a153b2aa0c82c11a51c3711bb58a56fe1a96a1113"},
+    "near_l2p": {"bytes": 6426112 + 3204608, "source": "paper_0908_0673_gb300/csrc/fmm.cu",
+                 "sha256": "688ca2b61ec7e22fb90ddf30e94d92f42eaab2aa6972c87045f7f49f9b6f6ba2"},
     # the M2L stage: k_m2l_permute + k_m2l_tc + k_m2l_gather_sym (order-10 products)
-    "m2l": {"bytes": 1217280 + (35175168 + 43993600) + (122822400 + 138240), "source": "paper_0908_0673_gb300/csrc/m2l_tc.cu",
-            "sha256": "9c140fd3a2a67fa8c171236e292f7ff8c7dbaa2532f25c5519d5f0ab974b7ce6"},
+    "m2l": {"bytes": 1216768 + (35236864 + 43760896) + (122820608 + 206080), "source": "paper_0908_0673_gb300/csrc/m2l_tc.cu",
+            "sha256": "a6b061c8b18128ae9c42cc91bd556d6d1c13a253c6982875b2d89f80287a43ab"},
 }
 
 
